@@ -470,7 +470,7 @@ typedef struct {
 EMPPP_API emppp_status emppp_measure_peaks(emppp_peaks* out, void* cuda_stream);
 
 /* The FP64 pair kernel's reciprocal, y[k] = 1 / x[k] for n values (device pointers; synchronous on
- * cuda_stream): the hardware's approximate reciprocal refined by two Newton-Raphson steps, which the
+ * cuda_stream): the hardware's approximate reciprocal refined by one third-order step, which the
  * kernel uses for 1 / (eta . v') and in the root of eq:dt. Exposed so that its error can be measured
  * against the correctly rounded quotient (within 2 units in the last place for finite x > 0 with
  * 2^-1022 < x < 2^1022; no counterpart in the paper). */

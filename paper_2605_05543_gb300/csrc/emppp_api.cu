@@ -428,7 +428,8 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
       CU(cudaEventRecord(h->ev_join, h->aux));
       k += 1;
     }
-    CU(launch_setup(h->ds, mixed_pairs, h->stream));
+    CU(launch_setup(h->ds,
+                    !h->opt.pair_fields ? SetupExt::none : (mixed_pairs ? SetupExt::mixed : SetupExt::fp64), h->stream));
     k += 1;
   }
   if (ordered && refresh_order) CU(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
@@ -596,7 +597,7 @@ emppp_status create_impl(int32_t nbunch, const int64_t* nper, int32_t history_de
   ALLOC(s.rec32, N * D * 12);
   ALLOC(s.slot_t, D);
   ALLOC(s.tab.lhs64, D);
-  ALLOC(s.tab.inv_dtk, D);
+  ALLOC(s.tab.tab64, D);
   ALLOC(s.tab.tab32, D);
   ALLOC(s.u, N * 3);
   ALLOC(s.wts, N);
@@ -619,6 +620,7 @@ emppp_status create_impl(int32_t nbunch, const int64_t* nper, int32_t history_de
   ALLOC(s.scale, (size_t)nbunch * 2);
   ALLOC(s.adapt_info, 3);
   ALLOC(s.ext32, N * kExtCount);
+  ALLOC(s.ext64, N * (kExt64 / 2));
   ALLOC(c->d_mon, (size_t)nbunch);
   ALLOC(c->staging, N * 7);
   ALLOC(c->ord_key, N);
@@ -1046,7 +1048,7 @@ EMPPP_API emppp_status emppp_reset_stats(emppp_handle h) {
 // one evaluation of the self fields of the present state: slot tables, target order, pair kernel,
 // reduction (no push: the state does not change)
 emppp_status enqueue_fields(emppp_handle h, int* dump = nullptr) {
-  CU(launch_setup(h->ds, h->opt.precision == EMPPP_MIXED, h->stream));
+  CU(launch_setup(h->ds, h->opt.precision == EMPPP_MIXED ? SetupExt::mixed : SetupExt::fp64, h->stream));
   const bool ordered = h->target_order != 0;
   if (ordered) CU(launch_target_order(h->ds, h->ord_key, h->order, h->max_bunch, h->stream));
   if (h->opt.precision == EMPPP_MIXED) {

@@ -14,11 +14,12 @@
 //                             origin and beta_ref are per bunch.
 //   slot_t [D]                time stamp of each physical slot.
 //   slot tables [D]           per step: (c (t_n - t_k))^2 in FP64 and FP32, c (t_n - t_k),
-//                             1 / (t_{k+1} - t_k) in FP64 and 1 / (c (t_{k+1} - t_k)) in FP32.
+//                             t_n - t_k and 1 / (t_{k+1} - t_k) in FP64 and 1 / (c (t_{k+1} - t_k)) in FP32.
 //   ext32  [N][5] float4      per step (mixed path): hi/lo of w_{n-1} + v_{n-1} (t_n - t_{n-1}) - origin,
 //                             w_{k0} + v_{k0} (t_n - t_{k0}) - w_n, the chord w_n - w_{k0} with the
 //                             threshold of the oldest-slot bound, and the FP32 record's beta - beta_ref,
 //                             1/gamma^2 and gamma^2 of slot k0 (kExt* below).
+//   ext64  [N][12] double     per step (FP64 path): the out-of-history line of each source (kExt64).
 //   u      [N][3]             present proper velocities (FP64).
 //   Eself/Bself [N][3]        self fields of the current step; Bout [N][3] = Bself + B_ext.
 //   ke     [N]                kinetic-energy terms of the energy monitor (small systems, formed by the push).
@@ -116,9 +117,13 @@ enum {
   kExtCount = 5
 };
 
+// doubles per source of ext64 (FP64 path): w_n (3), the line offset w_{k0} + v_{k0} (t_n - t_{k0}) - w_n (3),
+// v_{k0} (3), c^2 - v_{k0}^2, c w_j and c w_j (c^2 - v_{k0}^2)
+constexpr int kExt64 = 12;
+
 struct SlotTables {
   double* lhs64;    // [D] (c (t_n - t_k))^2, formed as c*(t_n - t_k) then squared (no FMA)
-  double* inv_dtk;  // [D] 1 / (t_{k+1} - t_k) for k < n
+  double2* tab64;   // [D] t_n - t_k and, for k < n, 1 / (t_{k+1} - t_k)
   // [D] FP32 per slot: (upper threshold of (c (t_n - t_k))^2, lower threshold, c (t_n - t_k),
   // 1 / (c (t_{k+1} - t_k)))
   float4* tab32;
@@ -184,6 +189,7 @@ struct DeviceState {
   // w_{k0} + v_{k0} (t_n - t_{k0}) - w_n (where the out-of-history line of eq:linear2 is at t_n), and the
   // oldest slot's chord, bound and velocity (the out-of-history pairs' node test and line)
   float4* ext32;
+  double2* ext64;  // [N][kExt64 / 2] per source and step (FP64 path): the out-of-history line
   // adaptive time step (Sec. 2.4)
   unsigned long long* scale;  // [nbunch][2] bit patterns of eta_min (m, by min) and v_max^2 ((m/s)^2, by max)
   double* adapt_info;         // [3] dt, eta_min, v_max of the last adaptive step
@@ -282,7 +288,9 @@ cudaError_t launch_gather_slot(const DeviceState& s, int p, double* W, double* V
 cudaError_t launch_set_state(const DeviceState& s, long long n, double t, double dt, long long hist_start,
                              const double* u, const double* w, cudaStream_t st);
 cudaError_t launch_prep(const DeviceState& s, cudaStream_t st);
-cudaError_t launch_setup(const DeviceState& s, bool extrap, cudaStream_t st);
+// per-source vectors the set-up launch forms: none, the mixed path's (ext32) or the FP64 path's (ext64)
+enum class SetupExt { none, mixed, fp64 };
+cudaError_t launch_setup(const DeviceState& s, SetupExt ext, cudaStream_t st);
 cudaError_t launch_reset_scale(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_gather_positions(const DeviceState& s, double* x, cudaStream_t st);
 // pair_fp64.cu

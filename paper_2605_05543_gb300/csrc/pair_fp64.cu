@@ -13,12 +13,12 @@
 //      v = v1 + (dt / (t2 - t1)) (v2 - v1), a = (v2 - v1) / (t2 - t1); or, in the comparison variant MID,
 //      the bracket's midpoint values of eq:mid.
 //   3. Lienard-Wiechert E (eq:LW_E) and B = eta_hat x E / c (eq:LW_B), summed over j != i in
-//      blocks of kSumBlock sources (blocked summation keeps the FP64 rounding error of a 65536-term
+//      blocks of kTile sources (blocked summation keeps the FP64 rounding error of a 65536-term
 //      sum near 1e-14 of the sum of magnitudes).
 //   Out of history (eq:linear2) the source moves uniformly with v1 along the line through w_{k0}, and its
 //   Lienard-Wiechert field is Heaviside's field about the line's point at t_n: with X = r - w_{k0} -
 //   v1 (t_n - t_{k0}), E = kq c (c^2 - v1^2) X / [|X|^2 (c^2 - v1^2) + (X.v1)^2]^{3/2}, B = v1 x E / c^2.
-//   It is the same field, without the quadratic and the retarded reconstruction.
+//   It is the same field, without the retarded reconstruction. How 2. and 3. are formed: at the kernel.
 // Targets are taken in the spatial order of order.cu (when given), so that the pairs of a warp mostly
 // take the same branch; which thread evaluates a target does not change its result.
 // The arithmetic is FP64-pipe bound (GB300: 2 DFMA/clk/SM); everything that is not an FP64 result
@@ -32,34 +32,49 @@ namespace emppp {
 
 namespace {
 
-constexpr int kSumBlock = 64;
 constexpr double kCoulomb = 1.0 / (4.0 * kPi * kEps0);
 // the sums run over w_j-weighted fields without the electron's charge constant -e / (4 pi eps0), and over
 // c^2 B; both are scaled once per target
 constexpr double kFieldScale = -kQe * kCoulomb;
 
-// 1 / x for finite x > 0: the hardware's approximate reciprocal refined by two Newton-Raphson steps
-// y <- y + y (1 - x y). Each step squares the relative error, so the approximation's error falls below
-// FP64 rounding after two steps (within a few units in the last place, not correctly rounded), for
-// five FP64-pipe operations instead of a correctly rounded division.
-__device__ __forceinline__ double recip_newton(double x) {
+// 1 / x for finite x > 0: the hardware's approximate reciprocal y (about 2^-20 relative) refined by one
+// step of Householder's third-order iteration, y <- y + y (e + e^2) with e = 1 - x y, which leaves e^3: three
+// FP64-pipe operations (two Newton-Raphson steps, as before, took four). Within a few units in the last
+// place, not correctly rounded.
+__device__ __forceinline__ double recip_refined(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  double e = fma(-x, y, 1.0);
-  y = fma(y, e, y);
-  e = fma(-x, y, 1.0);
-  return fma(y, e, y);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
 }
 
+// The same iteration for the root: with y the hardware's approximation of 1 / sqrt(x), t = x y and
+// e = 1 - x y^2, sqrt(x) = t / sqrt(1 - e) = t + t e (1/2 + 3/8 e) + O(e^3), and 1 / sqrt(x) likewise from y.
+// Both share t, e and the bracket; each costs two more operations.
+struct Root {
+  double y, t, e, q;
+  __device__ __forceinline__ explicit Root(double x) {
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    t = x * y;
+    e = fma(-t, y, 1.0);
+    q = fma(e, 0.375, 0.5);
+  }
+  __device__ __forceinline__ double sqrt() const { return fma(t * e, q, t); }
+  __device__ __forceinline__ double rsqrt() const { return fma(y * e, q, y); }
+};
+
+// finite, positive and normal, decided on the high word: a comparison of doubles would take the FP64 pipe
+__device__ __forceinline__ bool positive_normal(double x) {
+  return (unsigned)(__double2hiint(x) - 0x00100000) < 0x7fe00000u;
+}
 
 struct PairArgs {
   const double* __restrict__ rec64;
   const float* __restrict__ rec32;
-  const double* __restrict__ slot_t;
   const double* __restrict__ lhs64;
   const float4* __restrict__ tab32;  // per slot: FP32 guard-band thresholds of (c (t_n - t_k))^2
-  const double* __restrict__ inv_dtk;
-  const double* __restrict__ wts;
+  const double2* __restrict__ tab64;  // per slot: t_n - t_k, 1 / (t_{k+1} - t_k)
+  const double2* __restrict__ ext64;  // [N][kExt64 / 2] per source (ring.cu)
   const StepState* __restrict__ state;
   double* __restrict__ out;  // [S][N][6] (S = 1: [N][6] temporary) -- see launch
   double* __restrict__ E;
@@ -91,36 +106,59 @@ __device__ __forceinline__ bool node_test(double r0, double r1, double r2, const
 }
 
 struct Window {
-  long long k0, n;
-  int p0, D;
-  int* err;  // device error word (the debug build's range checks)
-  __device__ __forceinline__ int phys(long long k) const {
-    int p = p0 + (int)(debug_index(k, k0, n + 1, err) - k0);
+  int p0, D, nw;  // slots of the usable window k0..n are addressed by their offset l = k - k0 (0..nw-1)
+  int* err;       // device error word (the debug build's range checks)
+  __device__ __forceinline__ int phys(int l) const {
+    const int p = p0 + debug_index(l, 0, nw, err);
     return p >= D ? p - D : p;
   }
 };
 
+// sources staged in shared memory at a time, and the pairs of one partial sum
+constexpr int kTile = 64;
+
 }  // namespace
 
+// What bounds it: the FP64 pipe, 2 operations per SM and clock, so that a warp instruction holds it for 16
+// cycles. Everything else (guess, node tests, indices, loads) runs beside it; the kernel's cost is its count of
+// FP64 operations, about 33 for a pair beyond the history and 72 for one inside it:
+//   - both start from X, the target's separation from where the source's line w1 + v1 (t' - t1) is at t_n, and
+//     from Dh = |X|^2 (c^2 - v1^2) + (X.v1)^2, a sum of non-negative terms. Out of history Heaviside's field
+//     follows at once. Inside it tau = t_n - t_r is the positive root of (c^2 - v1^2) tau^2 - 2 (X.v1) tau -
+//     |X|^2 = 0, whose half-discriminant is Dh: tau = (X.v1 + sqrt(Dh)) / (c^2 - v1^2), or |X|^2 / (sqrt(Dh) -
+//     X.v1) for X.v1 < 0. The sum never cancels, where eq:dt's quadratic about t1 loses (c (t_n - t1) / R)^2;
+//   - on the light cone |eta| = c tau, so no root or division by R is left: with kappa = c R - eta.v =
+//     sqrt(Dh) - (t_r - t1) eta.a, A = c^2 - v^2 + eta.a and H = A v + kappa a, eq:LW_E and eq:LW_B become
+//       E = q c (A eta - tau H) / kappa^3,   c^2 B = q c (H x eta) / kappa^3;
+//   - the parts that one source shares with every target (its oldest slot's line, v, c^2 - v^2 and weights)
+//     come from ext64, formed once per step and source.
+// Against the same inputs in 113 bits, pairs and sums are off by 0.3 to 0.9 of what the previous form was (quadratic
+// about t1, cross products; 50 and 118 operations) over gamma 2 to 197, and by under 1 % of it where R is far
+// below c (t_n - t_{n-1}). One step, before and after: 45.8 and 29.6 ms at N = 16381 (251 slots, closed-form guess),
+// 4.64 and 2.96 ms at N = 4096 (512 slots, bisection); the FP64 pipe is 90 % busy while an SM has work.
 // SHAPE: targets per block (kBlock = shape_block(SHAPE); shapes 3 and 4 run as shape 0)
 template <int PROP, bool ADAPT, bool MID, bool DUMP, int SHAPE>
 __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs a) {
   constexpr int kBlock = shape_block(SHAPE);
   __shared__ int s_item;
+  __shared__ double2 s_e[kTile * (kExt64 / 2)];  // ext64 of the tile's sources
+  // FP32 records of the tile's sources: the bisection's (hi, lo) of the oldest slot and of slot n - 1; with the
+  // guess the present (hi, 1/gamma^2) and (dbeta, gamma^2), then (hi, lo) of the oldest slot
+  __shared__ float4 s_f[kTile][4];
+  __shared__ double s_acc[6][kBlock];  // per-thread sums of E and B over the tiles
   const long long N = a.N;
   const int D = a.D;
 
   Window win;
-  win.n = a.state->n;
-  win.k0 = a.state->k0;
   win.p0 = a.state->p0;
   win.D = D;
+  win.nw = (int)(a.state->n - a.state->k0) + 1;
   win.err = a.err;
+  const int nw = win.nw;
   const int pn = a.state->pn;
-  const double t = a.state->t;
   const float inv_cdt = PROP != kPropBisect ? (float)(1.0 / (kC * a.state->dt)) : 0.f;
   const float invL = (float)(1.0 / (kC * a.state->dt * D));
-  const int pprev = win.n > win.k0 ? win.phys(win.n - 1) : pn;  // slot n - 1 (or n)
+  const int pprev = nw > 1 ? win.phys(nw - 2) : pn;  // slot n - 1 (or n)
 
   unsigned n_ooh = 0, n_sc = 0, n_bi = 0, n_tests = 0, n_fb = 0;
   double emin = __longlong_as_double(0x7ff0000000000000LL), vmax2 = 0.0;  // adaptive time step (Sec. 2.4)
@@ -138,18 +176,18 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
   const BunchDesc& bd = a.bunches[b];
   const BunchSched& bs = a.sched[b];
   const float3 bref = make_float3((float)bd.beta_ref[0], (float)bd.beta_ref[1], (float)bd.beta_ref[2]);
-  const long long i_loc = (long long)tb * kBlock + threadIdx.x;
+  const int boff = (int)bd.off, bend = boff + bd.n;
+  const int i_loc = tb * kBlock + (int)threadIdx.x;
   const bool active = i_loc < bd.n;
-  const long long i = debug_index<long long>(a.order ? a.order[bd.off + (active ? i_loc : 0)] : bd.off + (active ? i_loc : 0),
-                                            bd.off, bd.off + bd.n, a.err);
-  const long long ic = i;
+  const int t_idx = boff + (active ? i_loc : 0);
+  const int i = debug_index(a.order ? a.order[t_idx] : t_idx, boff, bend, a.err);
 
-  const double* rr = a.rec64 + ((size_t)ic * D + pn) * 6;
+  const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
   const double r0 = rr[0], r1 = rr[1], r2 = rr[2];
   const double vi0 = ADAPT ? rr[3] : 0.0, vi1 = ADAPT ? rr[4] : 0.0, vi2 = ADAPT ? rr[5] : 0.0;  // v_i(t_n)
   // FP32 hi/lo split of the target's position: node tests run in FP32 against the guard-band thresholds
   // of the slot tables and fall back to the FP64 test between them (the decision is the FP64 one)
-  const float* tq = a.rec32 + ((size_t)ic * D + pn) * 12;
+  const float* tq = a.rec32 + ((size_t)i * D + pn) * 12;
   const float rh0 = tq[0], rh1 = tq[1], rh2 = tq[2];
   const float rl0 = tq[4], rl1 = tq[5], rl2 = tq[6];
   const bool far_target = fmaxf(fabsf(rh0), fmaxf(fabsf(rh1), fabsf(rh2))) > 0.5f;
@@ -158,25 +196,36 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
   if (PROP == kPropMlp) rc = mlp::warp_mean(active, rh0, rh1, rh2);
   float fac_lane = 1.f;  // delay factor of source j0 + lane of the current group of 32
 
-  const long long j_begin = bd.off + (long long)chunk_id * bs.chunk;
-  const long long j_end = min(bd.off + bd.n, j_begin + bs.chunk);
+  const int j_begin = boff + chunk_id * bs.chunk;
+  const int j_end = min(bend, j_begin + bs.chunk);
+#pragma unroll
+  for (int c = 0; c < 6; c++) s_acc[c][threadIdx.x] = 0.0;
 
-  double Et[3] = {0, 0, 0}, Bt[3] = {0, 0, 0};
-  double Ep[3] = {0, 0, 0}, Bp[3] = {0, 0, 0};
-  int in_block = 0;
-
-  const double c2 = kC * kC;
-  for (long long j = j_begin; (PROP == kPropMlp || active) && j < j_end; ++j) {
+  for (int tile = j_begin; tile < j_end; tile += kTile) {
+  const int tn = min(kTile, j_end - tile);
+  __syncthreads();
+  for (int q = threadIdx.x; q < tn * (kExt64 / 2); q += kBlock) s_e[q] = __ldg(a.ext64 + (size_t)tile * (kExt64 / 2) + q);
+  for (int q = threadIdx.x; q < tn * 4; q += kBlock) {
+    const int c = q & 3;
+    const int js = debug_index(tile + (q >> 2), boff, bend, a.err);
+    const int slot = PROP == kPropBisect ? (c < 2 ? win.p0 : pprev) : (c < 2 ? pn : win.p0);
+    const int part = PROP == kPropBisect ? (c & 1) : (c == 1 ? 2 : (c & 1));
+    s_f[q >> 2][c] = __ldg(reinterpret_cast<const float4*>(a.rec32) + ((size_t)js * D + slot) * 3 + part);
+  }
+  __syncthreads();
+  double Ep[3] = {0, 0, 0}, Bp[3] = {0, 0, 0};  // sums over this tile's sources
+  for (int jj = 0; (PROP == kPropMlp || active) && jj < tn; ++jj) {
+    const int j = debug_index(tile + jj, boff, bend, a.err);  // tile + jj itself in a release build
     float fac = 1.f;
     if (PROP == kPropMlp) {
       // every 32 sources, the warp evaluates the network for the next 32 (one per lane) at its mean target
       // position; each pair then scales its uniform-motion delay by its source's factor
-      const int l = (int)((j - j_begin) & 31);
+      const int l = jj & 31;
       if (l == 0) {
         __syncwarp();
-        const long long js = j + (threadIdx.x & 31);
-        const bool v = js < j_end;
-        const long long jr = v ? js : j;
+        const int js = jj + (int)(threadIdx.x & 31);
+        const bool v = js < tn;
+        const int jr = v ? tile + js : j;
         const float4* qn = reinterpret_cast<const float4*>(a.rec32 + ((size_t)jr * D + pn) * 12);
         const float4 q0n = __ldg(qn), q2n = __ldg(qn + 2);
         const float4 q2p = __ldg(reinterpret_cast<const float4*>(a.rec32 + ((size_t)jr * D + pprev) * 12) + 2);
@@ -188,12 +237,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
     }
     if (!active) continue;  // and stay in the loop for the next group's evaluation
     if (j == i) continue;
-    const long long jc = debug_index(j, bd.off, bd.off + bd.n, a.err);  // j itself in a release build
-    const double* src = a.rec64 + (size_t)jc * D * 6;
-    const float4* src32 = reinterpret_cast<const float4*>(a.rec32 + (size_t)jc * D * 12);
-    // P(k) at physical slot p: FP32 on the hi/lo split outside the guard band, else the FP64 test
-    auto ntest = [&](int p) -> bool {
-      const float4 q0 = __ldg(src32 + 3 * p), q1 = __ldg(src32 + 3 * p + 1);
+    const double* src = a.rec64 + (size_t)j * D * 6;
+    const float4* src32 = reinterpret_cast<const float4*>(a.rec32 + (size_t)j * D * 12);
+    // P(k) at physical slot p from its FP32 record: on the hi/lo split outside the guard band, else the FP64 test
+    auto test32 = [&](float4 q0, float4 q1, int p) -> bool {
       const float d0 = (rh0 - q0.x) + (rl0 - q1.x), d1 = (rh1 - q0.y) + (rl1 - q1.y), d2 = (rh2 - q0.z) + (rl2 - q1.z);
       const float D2 = d0 * d0 + d1 * d1 + d2 * d2;
       const float4 tb = __ldg(a.tab32 + p);
@@ -204,98 +251,90 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
       n_fb += 1;
       return node_test(r0, r1, r2, src + p * 6, __ldg(a.lhs64 + p));
     };
-    // ---- 1. bracket ------------------------------------------------------------------------
-    long long k1;
-    int br;
-    if (PROP == kPropBisect) {
-      n_tests += 1;
-      if (ntest(win.p0)) {
-        k1 = win.k0;
+    auto ntest = [&](int l) -> bool {
+      const int p = win.phys(l);
+      return test32(__ldg(src32 + 3 * p), __ldg(src32 + 3 * p + 1), p);
+    };
+    // ---- 1. bracket: offset l1 of the older node --------------------------------------------
+    int l1, br;
+    n_tests += 1;
+    if (nw == 1) {
+      // only the present slot exists: every pair is out of history
+      l1 = 0;
+      br = 0;
+    } else if (PROP == kPropBisect) {
+      if (test32(s_f[jj][0], s_f[jj][1], win.p0)) {
+        l1 = 0;
         br = 0;
       } else {
         n_tests += 1;
-        const int pm1 = win.phys(win.n - 1);
-        if (!ntest(pm1)) {
-          k1 = win.n - 1;
+        if (!test32(s_f[jj][2], s_f[jj][3], pprev)) {
+          l1 = nw - 2;
           br = 1;
         } else {
-          long long lo = win.k0, hi = win.n;
+          int lo = 0, hi = nw - 1;
           while (hi - lo > 1) {
-            const long long m = (lo + hi) >> 1;
-            const int pm = win.phys(m);
+            const int m = (lo + hi) >> 1;
             n_tests += 1;
-            if (ntest(pm))
+            if (ntest(m))
               hi = m;
             else
               lo = m;
           }
-          k1 = lo;
+          l1 = lo;
           br = 2;
         }
       }
     } else {
-      // guarded galloping search from the closed-form guess
-      if (win.n == win.k0) {
-        k1 = win.k0;
-        br = 0;
-        n_tests += 1;
+      // guarded galloping search from the uniform-motion delay (scaled by the network's factor with the learned
+      // proposal)
+      const int lg = uniform_motion_guess(rh0, rh1, rh2, s_f[jj][0], s_f[jj][1], bref,
+                                          PROP == kPropMlp ? inv_cdt * fac : inv_cdt, nw);
+      int lo, hi;
+      bool ooh = false;
+      if (lg == 0 ? test32(s_f[jj][2], s_f[jj][3], win.p0) : ntest(lg)) {
+        hi = lg;
+        int s = 1;
+        for (;;) {
+          if (hi == 0) {
+            ooh = true;
+            break;
+          }
+          lo = max(hi - s, 0);
+          n_tests += 1;
+          if (!ntest(lo)) break;
+          hi = lo;
+          s <<= 1;
+        }
       } else {
-        // the uniform-motion delay (scaled by the network's factor with the learned proposal)
-        const float4* qn = reinterpret_cast<const float4*>(a.rec32 + ((size_t)j * D + pn) * 12);
-        const long long kg = uniform_motion_guess(rh0, rh1, rh2, __ldg(qn), __ldg(qn + 2), bref,
-                                                  PROP == kPropMlp ? inv_cdt * fac : inv_cdt, win.k0, win.n);
-        long long lo, hi;
-        bool ooh = false;
-        n_tests += 1;
-        int pg = win.phys(kg);
-        if (ntest(pg)) {
-          hi = kg;
-          long long s = 1;
-          for (;;) {
-            if (hi == win.k0) {
-              ooh = true;
-              break;
-            }
-            lo = hi - s;
-            if (lo < win.k0) lo = win.k0;
-            const int pl = win.phys(lo);
-            n_tests += 1;
-            if (!ntest(pl)) break;
-            hi = lo;
-            s <<= 1;
+        lo = lg;
+        int s = 1;
+        for (;;) {
+          hi = lo + s;
+          if (hi >= nw - 1) {
+            hi = nw - 1;
+            break;
           }
-        } else {
-          lo = kg;
-          long long s = 1;
-          for (;;) {
-            hi = lo + s;
-            if (hi >= win.n) {
-              hi = win.n;
-              break;
-            }
-            const int ph = win.phys(hi);
-            n_tests += 1;
-            if (ntest(ph)) break;
-            lo = hi;
-            s <<= 1;
-          }
+          n_tests += 1;
+          if (ntest(hi)) break;
+          lo = hi;
+          s <<= 1;
         }
-        if (ooh) {
-          k1 = win.k0;
-          br = 0;
-        } else {
-          while (hi - lo > 1) {
-            const long long m = (lo + hi) >> 1;
-            const int pm = win.phys(m);
-            n_tests += 1;
-            if (ntest(pm))
-              hi = m;
-            else
-              lo = m;
-          }
-          k1 = lo;
-          br = (k1 == win.n - 1) ? 1 : 2;
+      }
+      if (ooh) {
+        l1 = 0;
+        br = 0;
+      } else {
+        while (hi - lo > 1) {
+          const int m = (lo + hi) >> 1;
+          n_tests += 1;
+          if (ntest(m))
+            hi = m;
+          else
+            lo = m;
         }
+        l1 = lo;
+        br = (l1 == nw - 2) ? 1 : 2;
       }
     }
     if (br == 0)
@@ -304,159 +343,158 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
       n_sc++;
     else
       n_bi++;
-    if (DUMP) a.dump[(size_t)i * N + j] = 4 * (int)(k1 - win.k0) + br;
+    if (DUMP) a.dump[(size_t)i * N + j] = 4 * l1 + br;
 
-    // ---- 2. reconstruction (eq:dt, eq:linear; eq:mid in the MID variant) ----------------------
-    const int p1 = win.phys(k1);
-    const double2* R1 = reinterpret_cast<const double2*>(src + p1 * 6);
-    const double2 x01 = __ldg(R1), x23 = __ldg(R1 + 1), x45 = __ldg(R1 + 2);
-    const double w10 = x01.x, w11 = x01.y, w12 = x23.x;
-    const double v10 = x23.y, v11 = x45.x, v12 = x45.y;
+    // ---- 2. the source's line at t_n ----------------------------------------------------------
+    const double2* se = s_e + jj * (kExt64 / 2);
+    const double cw = se[5].x;  // c w_j: the charge constant -e / (4 pi eps0) is applied once per target
+    double X0, X1, X2, v10, v11, v12, C2;
+    double2 y01, y23, y45, ts;  // newer record, (t_n - t1, 1 / (t2 - t1))
+    double w10, w11, w12;       // older position (eq:mid)
     if (br == 0) {
-      // ---- out of history (eq:linear2): Heaviside's field of the uniformly moving source -------
-      const double T1 = t - __ldg(a.slot_t + p1);
-      const double X0 = (r0 - w10) - v10 * T1, X1 = (r1 - w11) - v11 * T1, X2 = (r2 - w12) - v12 * T1;
-      const double c2mv2 = c2 - (v10 * v10 + v11 * v11 + v12 * v12);
-      const double XX = X0 * X0 + X1 * X1 + X2 * X2;
-      const double Xv = X0 * v10 + X1 * v11 + X2 * v12;
-      const double Dh = XX * c2mv2 + Xv * Xv;  // c^2 [|X|^2 (1 - beta^2) + (X.beta)^2]
-      if (!(c2mv2 > 0.0)) {
-        errbits |= kErrDisc;
-        continue;
-      }
-      if (!(Dh > 0.0)) {
+      // out of history (eq:linear2): the line through the oldest slot
+      const double2 e0 = se[0], e1 = se[1], e2 = se[2], e3 = se[3], e4 = se[4];
+      X0 = (r0 - e0.x) - e1.y;
+      X1 = (r1 - e0.y) - e2.x;
+      X2 = (r2 - e1.x) - e2.y;
+      v10 = e3.x;
+      v11 = e3.y;
+      v12 = e4.x;
+      C2 = e4.y;
+    } else {
+      const int p1 = win.phys(l1);
+      const int p2 = p1 + 1 == D ? 0 : p1 + 1;
+      const double2* R1 = reinterpret_cast<const double2*>(src + p1 * 6);
+      const double2* R2 = reinterpret_cast<const double2*>(src + p2 * 6);
+      const double2 x01 = __ldg(R1), x23 = __ldg(R1 + 1), x45 = __ldg(R1 + 2);
+      if (MID) y01 = __ldg(R2);
+      y23 = __ldg(R2 + 1);
+      y45 = __ldg(R2 + 2);
+      ts = __ldg(a.tab64 + p1);
+      w10 = x01.x;
+      w11 = x01.y;
+      w12 = x23.x;
+      v10 = x23.y;
+      v11 = x45.x;
+      v12 = x45.y;
+      X0 = fma(-v10, ts.x, r0 - w10);
+      X1 = fma(-v11, ts.x, r1 - w11);
+      X2 = fma(-v12, ts.x, r2 - w12);
+      C2 = fma(-v10, v10, fma(-v11, v11, fma(-v12, v12, kC * kC)));
+    }
+    if (MID && br != 0) {
+      // eq:mid: the midpoint of the bracket stands for the retarded time; eq:LW_E and eq:LW_B as they stand
+      const double idt = ts.y;
+      const double v0 = 0.5 * (v10 + y23.y), v1 = 0.5 * (v11 + y45.x), v2 = 0.5 * (v12 + y45.y);
+      const double a0 = (y23.y - v10) * idt, a1 = (y45.x - v11) * idt, a2 = (y45.y - v12) * idt;
+      const double e0 = r0 - 0.5 * (w10 + y01.x), e1 = r1 - 0.5 * (w11 + y01.y), e2 = r2 - 0.5 * (w12 + y23.x);
+      const double R2s = e0 * e0 + e1 * e1 + e2 * e2;
+      const double invR = rsqrt(R2s);
+      const double R = R2s * invR;
+      const double cinvR = kC * invR;
+      const double vp0 = e0 * cinvR - v0, vp1 = e1 * cinvR - v1, vp2 = e2 * cinvR - v2;
+      const double evp = e0 * vp0 + e1 * vp1 + e2 * vp2;
+      if (!(R2s > 0.0) || !(evp > 0.0)) {
         errbits |= kErrCoincide;
         continue;
       }
-      const double iD = rsqrt(Dh);
-      // E / (-e / (4 pi eps0)): the source's charge constant is applied once per target (kFieldScale)
-      const double pref = (kC * __ldg(a.wts + j)) * c2mv2 * (iD * iD * iD);
-      const double E0 = pref * X0, E1 = pref * X1, E2 = pref * X2;
+      const double c2mv2 = kC * kC - (v0 * v0 + v1 * v1 + v2 * v2);
+      // eta x (v' x a)
+      const double xa0 = vp1 * a2 - vp2 * a1, xa1 = vp2 * a0 - vp0 * a2, xa2 = vp0 * a1 - vp1 * a0;
+      const double ac0 = e1 * xa2 - e2 * xa1, ac1 = e2 * xa0 - e0 * xa2, ac2 = e0 * xa1 - e1 * xa0;
+      const double ievp = recip_refined(evp);
+      const double pref = (cw * (1.0 / kC) * R) * (ievp * ievp * ievp);
+      const double E0 = pref * (c2mv2 * vp0 + ac0), E1 = pref * (c2mv2 * vp1 + ac1), E2 = pref * (c2mv2 * vp2 + ac2);
+      Ep[0] += E0;
+      Ep[1] += E1;
+      Ep[2] += E2;
+      Bp[0] += (e1 * E2 - e2 * E1) * cinvR;
+      Bp[1] += (e2 * E0 - e0 * E2) * cinvR;
+      Bp[2] += (e0 * E1 - e1 * E0) * cinvR;
+      continue;
+    }
+    const double XX = fma(X2, X2, fma(X1, X1, X0 * X0));
+    const double Xv = fma(X2, v12, fma(X1, v11, X0 * v10));
+    const double Dh = fma(Xv, Xv, XX * C2);  // c^2 [|X|^2 (1 - beta1^2) + (X.beta1)^2]
+    if (!(positive_normal(C2) && positive_normal(Dh))) {
+      errbits |= (!positive_normal(C2) || (br != 0 && Dh != Dh)) ? kErrDisc : kErrCoincide;
+      continue;
+    }
+    const Root root(Dh);
+    if (br == 0) {
+      // ---- 3a. Heaviside's field of the uniformly moving source --------------------------------
+      const double iD = root.rsqrt();
       if (ADAPT) {
-        // retarded distance R = c (t - t_r), the positive root of R^2 (c^2 - v^2) - 2 R c (X.v) - c^2 |X|^2
-        // = 0, formed without cancellation; v(t_r) = v1
-        const double sD = Dh * iD;
-        const double R = (Xv >= 0.0) ? kC * (Xv + sD) / c2mv2 : kC * XX / (sD - Xv);
+        const double sD = root.sqrt() + fabs(Xv);
+        const bool pos = Xv >= 0.0;
+        const double R = kC * ((pos ? sD : XX) * recip_refined(pos ? C2 : sD));  // c (t - t_r); v(t_r) = v1
         if (R >= a.eta_allow) {
           emin = fmin(emin, R);
           const double dv0 = vi0 - v10, dv1 = vi1 - v11, dv2 = vi2 - v12;
           vmax2 = fmax(vmax2, dv0 * dv0 + dv1 * dv1 + dv2 * dv2);
         }
       }
-      // c^2 B = v x E (the 1 / c^2 is applied once per target)
+      const double pref = se[5].y * ((iD * iD) * iD);  // c w (c^2 - v1^2) / Dh^{3/2}
+      const double E0 = pref * X0, E1 = pref * X1, E2 = pref * X2;
       Ep[0] += E0;
       Ep[1] += E1;
       Ep[2] += E2;
-      Bp[0] += v11 * E2 - v12 * E1;
-      Bp[1] += v12 * E0 - v10 * E2;
-      Bp[2] += v10 * E1 - v11 * E0;
-      if (++in_block == kSumBlock) {
-        in_block = 0;
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          Et[c] += Ep[c];
-          Bt[c] += Bp[c];
-          Ep[c] = 0.0;
-          Bp[c] = 0.0;
-        }
-      }
+      // c^2 B = v x E (the 1 / c^2 is applied once per target)
+      Bp[0] = fma(v11, E2, fma(-v12, E1, Bp[0]));
+      Bp[1] = fma(v12, E0, fma(-v10, E2, Bp[1]));
+      Bp[2] = fma(v10, E1, fma(-v11, E0, Bp[2]));
       continue;
     }
-    double w0, w1, w2, v0 = v10, v1 = v11, v2 = v12, a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    if (MID && br != 0) {
-      // eq:mid: the midpoint of the bracket stands for the retarded time
-      const int p2 = p1 + 1 == D ? 0 : p1 + 1;
-      const double2* R2 = reinterpret_cast<const double2*>(src + p2 * 6);
-      const double2 y01 = __ldg(R2), y23 = __ldg(R2 + 1), y45 = __ldg(R2 + 2);
-      const double idt = __ldg(a.inv_dtk + p1);
-      w0 = 0.5 * (w10 + y01.x);
-      w1 = 0.5 * (w11 + y01.y);
-      w2 = 0.5 * (w12 + y23.x);
-      v0 = 0.5 * (v10 + y23.y);
-      v1 = 0.5 * (v11 + y45.x);
-      v2 = 0.5 * (v12 + y45.y);
-      a0 = (y23.y - v10) * idt;
-      a1 = (y45.x - v11) * idt;
-      a2 = (y45.y - v12) * idt;
-    } else {
-      const double T1 = t - __ldg(a.slot_t + p1);
-      const double d0 = r0 - w10, d1 = r1 - w11, d2 = r2 - w12;
-      const double C2 = c2 - (v10 * v10 + v11 * v11 + v12 * v12);
-      const double hb = (d0 * v10 + d1 * v11 + d2 * v12) - c2 * T1;  // C1 / 2
-      const double C0 = c2 * T1 * T1 - (d0 * d0 + d1 * d1 + d2 * d2);
-      const double qd = hb * hb - C2 * C0;  // disc / 4
-      if (!(C2 > 0.0) || !(qd >= 0.0)) {
-        errbits |= kErrDisc;
-        continue;
-      }
-      const double sq = qd * rsqrt(fmax(qd, 1e-300));  // sqrt(qd); the reciprocal root costs fewer FP64-pipe operations
-      // smaller root of C2 x^2 + 2 hb x + C0 without cancellation
-      const double dt = (hb <= 0.0) ? C0 * recip_newton(sq - hb) : -(hb + sq) * recip_newton(C2);
-      w0 = w10 + v10 * dt;
-      w1 = w11 + v11 * dt;
-      w2 = w12 + v12 * dt;
-      if (br != 0) {
-        const int p2 = p1 + 1 == D ? 0 : p1 + 1;
-        const double2* R2 = reinterpret_cast<const double2*>(src + p2 * 6);
-        const double2 y23 = __ldg(R2 + 1), y45 = __ldg(R2 + 2);
-        const double idt = __ldg(a.inv_dtk + p1);
-        a0 = (y23.y - v10) * idt;
-        a1 = (y45.x - v11) * idt;
-        a2 = (y45.y - v12) * idt;
-        v0 = v10 + dt * a0;
-        v1 = v11 + dt * a1;
-        v2 = v12 + dt * a2;
-      }
-    }
-    // ---- 3. Lienard-Wiechert fields ----------------------------------------------------------
-    const double e0 = r0 - w0, e1 = r1 - w1, e2 = r2 - w2;
-    const double R2s = e0 * e0 + e1 * e1 + e2 * e2;
-    const double invR = rsqrt(R2s);
-    const double R = R2s * invR;
-    const double cinvR = kC * invR;
-    const double vp0 = e0 * cinvR - v0, vp1 = e1 * cinvR - v1, vp2 = e2 * cinvR - v2;
-    const double evp = e0 * vp0 + e1 * vp1 + e2 * vp2;
-    if (!(R2s > 0.0) || !(evp > 0.0)) {
+    // ---- 3b. retarded state (eq:dt, eq:linear) and Lienard-Wiechert fields ----------------------
+    const double sq = root.sqrt();
+    const double sum = sq + fabs(Xv);
+    const bool pos = __double2hiint(Xv) >= 0;
+    const double tau = (pos ? sum : XX) * recip_refined(pos ? C2 : sum);  // t_n - t_r
+    const double f = (ts.x - tau) * ts.y;                                 // (t_r - t1) / (t2 - t1)
+    const double g0 = y23.y - v10, g1 = y45.x - v11, g2 = y45.y - v12;    // v2 - v1
+    const double e0 = fma(v10, tau, X0), e1 = fma(v11, tau, X1), e2 = fma(v12, tau, X2);  // eta
+    const double v0 = fma(f, g0, v10), v1 = fma(f, g1, v11), v2 = fma(f, g2, v12);
+    const double eg = fma(e2, g2, fma(e1, g1, e0 * g0));
+    const double kappa = fma(-f, eg, sq);
+    if (!positive_normal(kappa)) {
       errbits |= kErrCoincide;
       continue;
     }
-    const double c2mv2 = c2 - (v0 * v0 + v1 * v1 + v2 * v2);
-    // eta x (v' x a)
-    const double xa0 = vp1 * a2 - vp2 * a1, xa1 = vp2 * a0 - vp0 * a2, xa2 = vp0 * a1 - vp1 * a0;
-    const double ac0 = e1 * xa2 - e2 * xa1, ac1 = e2 * xa0 - e0 * xa2, ac2 = e0 * xa1 - e1 * xa0;
-    const double ievp = recip_newton(evp);
-    const double pref = (__ldg(a.wts + j) * R) * (ievp * ievp * ievp);  // charge constant once per target
-    const double E0 = pref * (c2mv2 * vp0 + ac0), E1 = pref * (c2mv2 * vp1 + ac1), E2 = pref * (c2mv2 * vp2 + ac2);
-    const double bs = invR * kC;  // c^2 B = c eta_hat x E
-    if (ADAPT && R >= a.eta_allow) {
-      // interaction scale of the adaptive step: |eta_ij| and |v_i(t_n) - v_j(t_r)|
-      emin = fmin(emin, R);
-      const double dv0 = vi0 - v0, dv1 = vi1 - v1, dv2 = vi2 - v2;
-      vmax2 = fmax(vmax2, dv0 * dv0 + dv1 * dv1 + dv2 * dv2);
-    }
-    Ep[0] += E0;
-    Ep[1] += E1;
-    Ep[2] += E2;
-    Bp[0] += (e1 * E2 - e2 * E1) * bs;
-    Bp[1] += (e2 * E0 - e0 * E2) * bs;
-    Bp[2] += (e0 * E1 - e1 * E0) * bs;
-    if (++in_block == kSumBlock) {
-      in_block = 0;
-#pragma unroll
-      for (int c = 0; c < 3; c++) {
-        Et[c] += Ep[c];
-        Bt[c] += Bp[c];
-        Ep[c] = 0.0;
-        Bp[c] = 0.0;
+    if (ADAPT) {
+      // interaction scale of the adaptive step: |eta_ij| = c tau and |v_i(t_n) - v_j(t_r)|
+      const double R = kC * tau;
+      if (R >= a.eta_allow) {
+        emin = fmin(emin, R);
+        const double dv0 = vi0 - v0, dv1 = vi1 - v1, dv2 = vi2 - v2;
+        vmax2 = fmax(vmax2, dv0 * dv0 + dv1 * dv1 + dv2 * dv2);
       }
     }
-  }
+    const double c2mv2 = fma(-v0, v0, fma(-v1, v1, fma(-v2, v2, kC * kC)));
+    const double ik = recip_refined(kappa);
+    const double s3 = cw * (ik * ik);                       // c w / kappa^2
+    const double s1 = (s3 * ik) * fma(ts.y, eg, c2mv2);     // c w A / kappa^3
+    const double s2 = s3 * ts.y;
+    const double H0 = fma(s1, v0, s2 * g0), H1 = fma(s1, v1, s2 * g1), H2 = fma(s1, v2, s2 * g2);
+    Ep[0] = fma(s1, e0, fma(-tau, H0, Ep[0]));
+    Ep[1] = fma(s1, e1, fma(-tau, H1, Ep[1]));
+    Ep[2] = fma(s1, e2, fma(-tau, H2, Ep[2]));
+    Bp[0] = fma(H1, e2, fma(-H2, e1, Bp[0]));
+    Bp[1] = fma(H2, e0, fma(-H0, e2, Bp[1]));
+    Bp[2] = fma(H0, e1, fma(-H1, e0, Bp[2]));
+  }  // sources of the tile
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    Et[c] = (Et[c] + Ep[c]) * kFieldScale;
-    Bt[c] = (Bt[c] + Bp[c]) * (kFieldScale / (kC * kC));
+    s_acc[c][threadIdx.x] += Ep[c];
+    s_acc[3 + c][threadIdx.x] += Bp[c];
   }
+  }  // tiles
   if (active) {
+    double Et[3], Bt[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+      Et[c] = s_acc[c][threadIdx.x] * kFieldScale;
+      Bt[c] = s_acc[3 + c][threadIdx.x] * (kFieldScale / (kC * kC));
+    }
     if (bs.nchunk == 1) {
       for (int c = 0; c < 3; c++) {
         a.E[3 * i + c] = Et[c];
@@ -560,11 +598,10 @@ cudaError_t launch_pair_fp64(const DeviceState& s, const int* order, int proposa
   PairArgs a;
   a.rec64 = s.rec64;
   a.rec32 = s.rec32;
-  a.slot_t = s.slot_t;
   a.lhs64 = s.tab.lhs64;
   a.tab32 = s.tab.tab32;
-  a.inv_dtk = s.tab.inv_dtk;
-  a.wts = s.wts;
+  a.tab64 = s.tab.tab64;
+  a.ext64 = s.ext64;
   a.state = s.state;
   a.out = s.partial;
   a.E = s.Eself;
@@ -615,7 +652,7 @@ cudaError_t launch_zero_self(const DeviceState& s, cudaStream_t st) {
 namespace {
 __global__ void recip_probe_kernel(const double* __restrict__ x, double* __restrict__ y, long long n) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) y[k] = recip_newton(x[k]);
+  if (k < n) y[k] = recip_refined(x[k]);
 }
 }  // namespace
 

@@ -88,7 +88,7 @@ __global__ void set_state_kernel(DeviceState s, long long n, double t, double dt
 // Slot-table entry of window offset l (slot p0 + l, modulo D) at time t_n (Sec. 2.2): the squared
 // light-travel distance (c (t_n - t_k))^2 in exactly the operation order of the reference evaluation
 // (so that the FP64 node test decides identically), its guard-band thresholds in FP32, c (t_n - t_k) in
-// FP32, and 1 / (t_{k+1} - t_k).
+// FP32, t_n - t_k and 1 / (t_{k+1} - t_k).
 constexpr double kGuardHi = (1.0 + kGuardBand) / (1.0 - kGuardBand), kGuardLo = (1.0 - kGuardBand) / (1.0 + kGuardBand);
 
 // FP32 upper threshold of a slot's (c (t_n - t_k))^2 (the node test is true above it)
@@ -105,10 +105,10 @@ __device__ __forceinline__ void slot_table(const DeviceState& s, int l, int p0, 
   if (l + 1 < nwin) {
     int q = p + 1 == s.D ? 0 : p + 1;
     const double dtk = s.slot_t[q] - tk;
-    s.tab.inv_dtk[p] = 1.0 / dtk;
+    s.tab.tab64[p] = make_double2(t_n - tk, 1.0 / dtk);
     icdt = (float)(1.0 / (kC * dtk));
   } else {
-    s.tab.inv_dtk[p] = 0.0;
+    s.tab.tab64[p] = make_double2(t_n - tk, 0.0);
   }
   s.tab.tab32[p] = make_float4(upper_threshold(lhs), __double2float_rd(lhs * kGuardLo), (float)ct, icdt);
 }
@@ -145,7 +145,9 @@ __global__ void prep_kernel(DeviceState s) {
 //     threshold of slot k0: the oldest-slot bound (kChordMargin), by which an out-of-history pair's
 //     node test of slot k0 needs no record of that slot; and the FP32 record's beta - beta_ref,
 //     1/gamma^2 and gamma^2 of slot k0, which Heaviside's field of that pair reads.
-__global__ void setup_kernel(DeviceState s, int extrap) {
+// For the FP64 path, per source, the out-of-history line of eq:linear2 in FP64 (kExt64): the present position,
+// X_j of the same line, its velocity and the factors of Heaviside's field that no target changes.
+__global__ void setup_kernel(DeviceState s, SetupExt extrap) {
   const long long n = s.state->n;
   const double t_n = s.state->t;
   const long long hs = s.state->hist_start;
@@ -161,10 +163,24 @@ __global__ void setup_kernel(DeviceState s, int extrap) {
   }
   const int nwin = (int)(n - k0 + 1);
   if (gid < nwin) slot_table(s, (int)gid, p0, nwin, t_n);
-  if (!extrap || gid >= s.N) return;
+  if (extrap == SetupExt::none || gid >= s.N) return;
   const long long j = gid;
   const double* rn = s.rec64 + ((size_t)j * s.D + pn) * 6;
   const double* r0 = s.rec64 + ((size_t)j * s.D + p0) * 6;
+  if (extrap == SetupExt::fp64) {
+    const double T0 = t_n - s.slot_t[p0];
+    const double v0 = r0[3], v1 = r0[4], v2 = r0[5];
+    const double C2 = fma(-v0, v0, fma(-v1, v1, fma(-v2, v2, kC * kC)));
+    const double cw = kC * s.wts[j];
+    double2* e = s.ext64 + (size_t)j * (kExt64 / 2);
+    e[0] = make_double2(rn[0], rn[1]);
+    e[1] = make_double2(rn[2], fma(v0, T0, r0[0] - rn[0]));
+    e[2] = make_double2(fma(v1, T0, r0[1] - rn[1]), fma(v2, T0, r0[2] - rn[2]));
+    e[3] = make_double2(v0, v1);
+    e[4] = make_double2(v2, C2);
+    e[5] = make_double2(cw, cw * C2);
+    return;
+  }
   const float* q0 = s.rec32 + ((size_t)j * s.D + p0) * 12;  // FP32 record of slot k0
   float4* ext = s.ext32 + (size_t)j * kExtCount;
   const double dt0 = s.slot_t[pn] - s.slot_t[p0];
@@ -241,11 +257,11 @@ cudaError_t launch_prep(const DeviceState& s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_setup(const DeviceState& s, bool extrap, cudaStream_t st) {
-  const long long n = extrap ? (s.N > s.D ? s.N : s.D) : s.D;
+cudaError_t launch_setup(const DeviceState& s, SetupExt ext, cudaStream_t st) {
+  const long long n = ext != SetupExt::none && s.N > s.D ? s.N : s.D;
   // small blocks: the per-slot and per-source FP64 work spreads over more SMs (an FP64 warp instruction
   // holds an SM's FP64 pipe for 16 cycles)
-  setup_kernel<<<blocks_for(n, 64), 64, 0, st>>>(s, extrap ? 1 : 0);
+  setup_kernel<<<blocks_for(n, 64), 64, 0, st>>>(s, ext);
   return cudaGetLastError();
 }
 

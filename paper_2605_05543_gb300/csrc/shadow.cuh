@@ -37,18 +37,15 @@ __device__ __forceinline__ double gamma2_of_u(double u0, double u1, double u2) {
 
 // Uniform-motion guess of the older bracket node: the source at its present record (q0n, q2n)
 // keeps its velocity; c (t - t_r) = [d.beta + sqrt((d.beta)^2 + (1 - beta^2) d^2)] / (1 - beta^2),
-// d = r - w_n. Returns a slot index clamped to [k0, n - 1] (requires n > k0).
-__device__ __forceinline__ long long uniform_motion_guess(float r0, float r1, float r2, float4 q0n, float4 q2n,
-                                                          float3 bref, float inv_cdt, long long k0, long long n) {
+// d = r - w_n. Returns an offset in the window of nw slots, clamped to [0, nw - 2] (requires nw > 1).
+__device__ __forceinline__ int uniform_motion_guess(float r0, float r1, float r2, float4 q0n, float4 q2n, float3 bref,
+                                                    float inv_cdt, int nw) {
   const float d0 = r0 - q0n.x, d1 = r1 - q0n.y, d2 = r2 - q0n.z;
   const float db = d0 * (bref.x + q2n.x) + d1 * (bref.y + q2n.y) + d2 * (bref.z + q2n.z);
   const float dd = d0 * d0 + d1 * d1 + d2 * d2;
   const float ctau = (db + sqrtf(fmaxf(db * db + q0n.w * dd, 0.f))) * q2n.w;
   const float steps = floorf(ctau * inv_cdt);
-  long long k = n - 1 - (long long)fminf(fmaxf(steps, 0.f), 1e9f);
-  if (k < k0) k = k0;
-  if (k > n - 1) k = n - 1;
-  return k;
+  return max(nw - 2 - (int)fminf(fmaxf(steps, 0.f), 1e9f), 0);
 }
 
 }  // namespace emppp
