@@ -95,6 +95,12 @@ enum { kStatOOH = 0, kStatShortcut = 1, kStatBisect = 2, kStatNodeTests = 3, kSt
 // rounding, so the FP32 decision is the FP64 one; between the thresholds the FP64 test decides.
 constexpr double kGuardBand = 32.0 * 5.9604644775390625e-08;
 
+// The lower threshold from the upper one, which is stored: L^2 (1 - k) / (1 + k) is the upper one's L^2 (1 + k) /
+// (1 - k) times this ratio; 8u covers the roundings of the stored value, the ratio and the product, so the
+// result is never above it.
+constexpr float kLowerRatio = (float)(((1.0 - kGuardBand) / (1.0 + kGuardBand)) * ((1.0 - kGuardBand) / (1.0 + kGuardBand)) *
+                                      (1.0 - 8.0 * 5.9604644775390625e-08));
+
 // Oldest-slot bound of the mixed path. For a pair whose uniform-motion guess lies beyond the history, the
 // node test of slot k0 is |r - w_k0|^2 = |d|^2 + 2 d.c + |c|^2 with d = r - w_n (formed from the staged
 // present records) and the source's chord c = w_n - w_k0. In FP32, |d|^2 carries a relative error below
@@ -124,7 +130,7 @@ constexpr int kExt64 = 12;
 struct SlotTables {
   double* lhs64;    // [D] (c (t_n - t_k))^2, formed as c*(t_n - t_k) then squared (no FMA)
   double2* tab64;   // [D] t_n - t_k and, for k < n, 1 / (t_{k+1} - t_k)
-  // [D] FP32 per slot: (upper threshold of (c (t_n - t_k))^2, lower threshold, c (t_n - t_k),
+  // [D] FP32 per slot: (upper threshold of (c (t_n - t_k))^2, lo and hi of c (t_n - t_k),
   // 1 / (c (t_{k+1} - t_k)))
   float4* tab32;
 };

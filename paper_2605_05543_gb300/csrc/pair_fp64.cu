@@ -72,7 +72,7 @@ struct PairArgs {
   const double* __restrict__ rec64;
   const float* __restrict__ rec32;
   const double* __restrict__ lhs64;
-  const float4* __restrict__ tab32;  // per slot: FP32 guard-band thresholds of (c (t_n - t_k))^2
+  const float4* __restrict__ tab32;  // per slot: FP32 upper guard-band threshold of (c (t_n - t_k))^2
   const double2* __restrict__ tab64;  // per slot: t_n - t_k, 1 / (t_{k+1} - t_k)
   const double2* __restrict__ ext64;  // [N][kExt64 / 2] per source (ring.cu)
   const StepState* __restrict__ state;
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
       const float4 tb = __ldg(a.tab32 + p);
       if (!far_target) {
         if (D2 > tb.x) return true;
-        if (D2 < tb.y) return false;
+        if (D2 < tb.x * kLowerRatio) return false;
       }
       n_fb += 1;
       return node_test(r0, r1, r2, src + p * 6, __ldg(a.lhs64 + p));

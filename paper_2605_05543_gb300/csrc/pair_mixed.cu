@@ -50,6 +50,8 @@ namespace {
 
 // FP64 recomputation of C0 when u L1^2 |s| / (C0 (L1 - s)) exceeds 2e-6: kC0Guard = 2e-6 / u
 constexpr float kC0Guard = 2.0e-6f / 5.9604644775390625e-08f;
+// FP64 separation from the source's line when u L1 / (2 sqrt(Dh)) exceeds 2e-6: kLineGuard = 4e-6 / u
+constexpr float kLineGuard = 4.0e-6f / 5.9604644775390625e-08f;
 // FP64 recomputation of X.beta (out-of-history pairs) when 2 u |X| |X.beta| / denominator exceeds 1.3e-6
 constexpr float kXbGuard = 2.0f * 5.9604644775390625e-08f / 1.3e-6f;
 
@@ -58,7 +60,8 @@ struct MixedArgs {
   const double* __restrict__ rec64;
   const double* __restrict__ lhs64;
   const double* __restrict__ slot_t;  // time stamps of the physical slots
-  const float4* __restrict__ tab32;  // per slot: guard-band thresholds of L^2, c (t - t_k), 1 / (c dt_k)
+  const float4* __restrict__ tab32;  // per slot: upper guard-band threshold of L^2, lo and hi of c (t - t_k), 1 / (c dt_k)
+  const double2* __restrict__ tab64;  // per slot: t - t_k, 1 / dt_k
   const float* __restrict__ kq32;  // -e w_j / (4 pi eps0), FP32
   const int* __restrict__ order;
   const StepState* __restrict__ state;
@@ -158,7 +161,7 @@ __device__ __forceinline__ bool node_test_d(const Target& r, float3 d, float4 ta
   const float D2 = d.x * d.x + d.y * d.y + d.z * d.z;
   if (!r.exact_only) {
     if (D2 > tab.x) return true;
-    if (D2 < tab.y) return false;
+    if (D2 < tab.x * kLowerRatio) return false;
   }
   count_fallback<SH>(n_fb);
   return exact_test(a.rec64 + ((size_t)r.idx * a.D + a.state->pn) * 6, src64 + 6 * p, __ldg(a.lhs64 + p));
@@ -681,6 +684,91 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
                     make_float4(A.q2.x, A.q2.y, A.q2.z, A.q0.w), A.q2.w, pA);
           continue;
         }
+        if (!ADAPT) {
+          // ---- retarded state and fields from the source's line at t_n (light units) ------------------
+          // p is the target's separation from where the line of the older node is at t_n, tau = c (t_n - t_r) = R
+          // the positive root of (1 - beta1^2) tau^2 - 2 (p.beta1) tau - |p|^2 = 0, whose half-discriminant Dh is a
+          // sum of non-negative terms. With f = (t_r - t1) / (t2 - t1), g = beta2 - beta1, eta = p + beta1 tau and
+          // beta = beta1 + f g: kappa = R - eta.beta = sqrt(Dh) - f eta.g, A = 1 - beta^2 + eta.alpha (alpha =
+          // g / (c dt)), H = A beta + kappa alpha, and eq:LW_E, eq:LW_B are E = kq (A eta - tau H) / kappa^3,
+          // c B = kq (H x eta) / kappa^3: no second root, no division by R, no double cross product.
+          // Rounding sequence fixed as below (no packed product feeds a packed sum).
+          const float L1 = tabA.z, icdt = tabA.w;
+          const float ig2 = A.q0.w;
+          const float2 b101 = __fadd2_rn(bref01, make_float2(A.q2.x, A.q2.y));
+          const float b10 = b101.x, b11 = b101.y, b12 = __fadd_rn(bref2, A.q2.z);
+          float2 p01;
+          float p2;
+          if (br == 1) {
+            // near-field shortcut: the end of the last segment, formed per source in FP64 (ext32), since p cancels
+            // when R is far below c (t_n - t_{n-1})
+            const float4* e = a.ext32 + (size_t)j * kExtCount;
+            const float3 dp = separation(r, __ldg(e + kExtSegHi), __ldg(e + kExtSegLo));
+            p01 = make_float2(dp.x, dp.y);
+            p2 = dp.z;
+          } else {
+            // d - beta1 L1 with beta1 = beta_ref + dbeta and L1 in two parts each
+            p01 = __ffma2_rn(make_float2(-bref01.x, -bref01.y), make_float2(L1, L1), make_float2(dA.x, dA.y));
+            p01 = __ffma2_rn(make_float2(-A.q2.x, -A.q2.y), make_float2(L1, L1), p01);
+            p01 = __ffma2_rn(make_float2(-b10, -b11), make_float2(tabA.y, tabA.y), p01);
+            p2 = __fmaf_rn(-b12, tabA.y, __fmaf_rn(-A.q2.z, L1, __fmaf_rn(-bref2, L1, dA.z)));
+          }
+          float pv = dot3(p01.x, p01.y, p2, b10, b11, b12);
+          float pp = dot3(p01.x, p01.y, p2, p01.x, p01.y, p2);
+          float Dh = __fmaf_rn(pp, ig2, __fmul_rn(pv, pv));
+          float sq = __fmul_rn(Dh, rsqrtf(Dh));
+          // The rounding of p (about u L1) moves tau by up to u L1 / (2 sqrt(Dh)) of itself. Where that exceeds 2e-6
+          // (sources moving nearly towards the target at high gamma; below 2 u gamma^2, so never for gamma^2 < 16)
+          // p is formed in FP64 from the FP64 records.
+          if (br == 2 && ig2 < 0.0625f && L1 > __fmul_rn(kLineGuard, sq)) {
+            const double* w64 = src64 + 6 * pA;
+            const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
+            const double T1 = __ldg(a.tab64 + pA).x;
+            p01.x = (float)((__ldg(rr + 0) - __ldg(w64 + 0)) - __ldg(w64 + 3) * T1);
+            p01.y = (float)((__ldg(rr + 1) - __ldg(w64 + 1)) - __ldg(w64 + 4) * T1);
+            p2 = (float)((__ldg(rr + 2) - __ldg(w64 + 2)) - __ldg(w64 + 5) * T1);
+            pv = dot3(p01.x, p01.y, p2, b10, b11, b12);
+            pp = dot3(p01.x, p01.y, p2, p01.x, p01.y, p2);
+            Dh = __fmaf_rn(pp, ig2, __fmul_rn(pv, pv));
+            sq = __fmul_rn(Dh, rsqrtf(Dh));
+            count_fallback<kShared>(n_fb);
+          }
+          const float sum = __fadd_rn(sq, fabsf(pv));
+          const bool pos = pv >= 0.f;
+          const float tau = __fmul_rn(pos ? sum : pp, pos ? A.q2.w : __fdividef(1.f, sum));
+          const float f = __fmul_rn(__fsub_rn(L1, tau), icdt);
+          if (!have_b) q2b = __ldg(src32 + 3 * (pA + 1 == D ? 0 : pA + 1) + 2);
+          const float2 g01 = sub2(make_float2(q2b.x, q2b.y), A.q2);
+          const float g2 = __fsub_rn(q2b.z, A.q2.z);
+          const float2 e01 = __ffma2_rn(b101, make_float2(tau, tau), p01);
+          const float e0 = e01.x, e1 = e01.y, e2 = __fmaf_rn(b12, tau, p2);
+          const float2 v01 = __ffma2_rn(g01, make_float2(f, f), b101);
+          const float v2 = __fmaf_rn(g2, f, b12);
+          const float eg = dot3(e0, e1, e2, g01.x, g01.y, g2);
+          const float kappa = __fmaf_rn(-f, eg, sq);
+          // 1 - beta^2 = (1 - beta1^2) - f g.(beta1 + beta)
+          const float2 t01 = __fadd2_rn(b101, v01);
+          const float Av = __fmaf_rn(icdt, eg, __fmaf_rn(-f, dot3(g01.x, g01.y, g2, t01.x, t01.y, __fadd_rn(b12, v2)), ig2));
+          if (!(ig2 > 0.f && Dh > 0.f && kappa >= 1.17549435e-38f)) {
+            set_err((ig2 > 0.f && Dh >= 0.f) ? kErrCoincide : kErrDisc);
+            continue;
+          }
+          const float ik = __fdividef(1.f, kappa);
+          const float s3 = __fmul_rn(__fmul_rn(s_kq[jj], ik), ik);  // kq / kappa^2
+          const float s1 = __fmul_rn(__fmul_rn(s3, ik), Av);        // kq A / kappa^3
+          const float s2 = __fmul_rn(s3, icdt);
+          const float2 H01 = __ffma2_rn(make_float2(s1, s1), v01, __fmul2_rn(make_float2(s2, s2), g01));
+          const float H2 = __fmaf_rn(s1, v2, __fmul_rn(s2, g2));
+          float2 q01 = __ffma2_rn(make_float2(-tau, -tau), H01, make_float2(P[0], P[1]));
+          q01 = __ffma2_rn(make_float2(s1, s1), e01, q01);
+          P[0] = q01.x;
+          P[1] = q01.y;
+          P[2] = __fmaf_rn(s1, e2, __fmaf_rn(-tau, H2, P[2]));
+          P[3] = __fmaf_rn(H01.y, e2, __fmaf_rn(-H2, e1, P[3]));
+          P[4] = __fmaf_rn(H2, e0, __fmaf_rn(-H01.x, e2, P[4]));
+          P[5] = __fmaf_rn(H01.x, e1, __fmaf_rn(-H01.y, e0, P[5]));
+          continue;
+        }
         // ---- retarded state (light units) --------------------------------------------------------
         // Written with explicit round-to-nearest intrinsics: the compiler may not fuse or regroup any
         // of it, so every search variant (whose own arithmetic shares subexpressions with this code
@@ -950,6 +1038,7 @@ cudaError_t launch_pair_mixed(const DeviceState& s, const int* order, int propos
   a.lhs64 = s.tab.lhs64;
   a.slot_t = s.slot_t;
   a.tab32 = s.tab.tab32;
+  a.tab64 = s.tab.tab64;
   a.kq32 = s.kq32;
   a.order = order;
   a.state = s.state;

@@ -87,9 +87,9 @@ __global__ void set_state_kernel(DeviceState s, long long n, double t, double dt
 
 // Slot-table entry of window offset l (slot p0 + l, modulo D) at time t_n (Sec. 2.2): the squared
 // light-travel distance (c (t_n - t_k))^2 in exactly the operation order of the reference evaluation
-// (so that the FP64 node test decides identically), its guard-band thresholds in FP32, c (t_n - t_k) in
-// FP32, t_n - t_k and 1 / (t_{k+1} - t_k).
-constexpr double kGuardHi = (1.0 + kGuardBand) / (1.0 - kGuardBand), kGuardLo = (1.0 - kGuardBand) / (1.0 + kGuardBand);
+// (so that the FP64 node test decides identically), its upper guard-band threshold in FP32, c (t_n - t_k) in
+// FP32 hi and lo, t_n - t_k and 1 / (t_{k+1} - t_k).
+constexpr double kGuardHi = (1.0 + kGuardBand) / (1.0 - kGuardBand);
 
 // FP32 upper threshold of a slot's (c (t_n - t_k))^2 (the node test is true above it)
 __device__ __forceinline__ float upper_threshold(double lhs) { return __double2float_ru(lhs * kGuardHi); }
@@ -110,7 +110,7 @@ __device__ __forceinline__ void slot_table(const DeviceState& s, int l, int p0, 
   } else {
     s.tab.tab64[p] = make_double2(t_n - tk, 0.0);
   }
-  s.tab.tab32[p] = make_float4(upper_threshold(lhs), __double2float_rd(lhs * kGuardLo), (float)ct, icdt);
+  s.tab.tab32[p] = make_float4(upper_threshold(lhs), (float)(ct - (double)(float)ct), (float)ct, icdt);
 }
 
 // Per-step slot tables over the usable window k0..n alone (used before the delay sampler).
