@@ -9,10 +9,14 @@
 //             the FP64 one. Search: the paper's bisection, or the guarded galloping
 //             search from the uniform-motion guess; with the guess, the records of the one or two slots
 //             the guess points at are loaded together, so a correct guess needs a single gather round.
-//             A pair the guess places beyond the history first tries the oldest-slot bound (kChordMargin,
-//             emppp_internal.cuh): from the staged present separation and the source's chord, it shows the
-//             oldest slot's FP32 test true at its first comparison without loading that slot's record.
-//   retarded  in light units (lengths in m, velocities as beta = v/c): with L1 = c (t - t1) and d = r - w1,
+//             Before any guess a pair tries the oldest-slot bound (kChordMargin, emppp_internal.cuh): from the
+//             staged present separation and the source's chord, it shows the oldest slot's FP32 test true at
+//             its first comparison without loading that slot's record. It decides most pairs beyond the
+//             history, whose field reads staged vectors alone, so that they need no guess (with the guess
+//             first: 32.6 against 30.8 ms at N = 65536, 251 slots).
+//   retarded  and fields, fixed step: from the source's line at t_n (at the code below).
+//   retarded  adaptive step: the textbook forms, kept because the last bit of |eta| and v_j(t_r) decides the
+//             step and with it every later time stamp: in light units (lengths in m, velocities as beta = v/c): with L1 = c (t - t1) and d = r - w1,
 //             (1 - beta1^2) s^2 + 2 (d.beta1 - L1) s + (L1^2 - |d|^2) = 0 for s = c (t_r - t1) (eq:dt),
 //             smaller root without cancellation; eta = d - beta1 s (eq:linear, retarded position w1 + v1 dt);
 //             in the near-field shortcut bracket the same point is formed from the segment's end
@@ -21,7 +25,7 @@
 //             beta = beta1 + (s / (c dt)) (beta2 - beta1), alpha = a / c^2 = (beta2 - beta1) / (c dt)
 //             (eq:linear2 out of history: beta = beta1, alpha = 0); 1 - beta^2 = 1/gamma1^2 - dbeta.(2 beta1
 //             + dbeta), so 1 - beta^2 is never formed by cancellation.
-//   fields    with u' = eta_hat - beta: E = (q / 4 pi eps0) R [(1 - beta^2) u' + eta x (u' x alpha)] / (eta.u')^3
+//   fields    (adaptive step) with u' = eta_hat - beta: E = (q / 4 pi eps0) R [(1 - beta^2) u' + eta x (u' x alpha)] / (eta.u')^3
 //             (eq:LW_E with v' = c u', a = c^2 alpha), B = eta_hat x E / c (eq:LW_B). eta.u' = R - eta.beta
 //             cancels for a source moving towards the target; there it is formed as
 //             [R^2 (1 - beta^2) + |eta x beta|^2] / (R + eta.beta), a sum of non-negative terms.
@@ -174,24 +178,18 @@ __device__ __forceinline__ bool node_test(const Target& r, const float4* __restr
                          p, a, n_fb);
 }
 
-// uniform-motion guess of the retarded delay, from the staged present record of the source:
-// c tau = gamma^2 [d.beta + sqrt((d.beta)^2 + |d|^2 / gamma^2)] with d from the hi parts only (g2.w is
-// gamma^2, times the learned delay factor with that proposal)
-__device__ __forceinline__ float closed_form_ctau(const Target& r, float4 g0, float4 g2) {
-  const float2 x01 = sub2(r.h01, g0);
-  const float x0 = x01.x, x1 = x01.y, x2 = r.h2 - g0.z;
-  const float db = x0 * g2.x + x1 * g2.y + x2 * g2.z;
-  const float dd = x0 * x0 + x1 * x1 + x2 * x2;
-  const float x = fmaxf(fmaf(db, db, g0.w * dd), 0.f);
-  return (db + x * rsqrtf(fmaxf(x, 1e-37f))) * g2.w;
+// uniform-motion guess of the retarded delay in steps, from the separation d = r - w_n and the staged present
+// record of the source: gamma^2 [d.beta + sqrt((d.beta)^2 + |d|^2 / gamma^2)] / (c dt) (g2.w is gamma^2 / (c dt),
+// times the learned delay factor with that proposal; a zero root, of coincident particles, gives a NaN)
+__device__ __forceinline__ float guessed_steps(float3 d, float dd, float ig2, float4 g2) {
+  const float db = d.x * g2.x + d.y * g2.y + d.z * g2.z;
+  const float x = fmaf(db, db, ig2 * dd);
+  return fmaf(x, rsqrtf(x), db) * g2.w;
 }
 
-// offset of the guessed older node for a delay of sc steps: (nw - 2) - floor(sc); -1 ("older than the
-// history") when floor(sc) > nw - 2, i.e. sc >= nw - 1, decided before any rounding; a negative or NaN
-// delay guesses the newest bracket
-__device__ __forceinline__ int guessed_offset(float sc, int nw, float nw1) {
-  return (sc >= nw1) ? -1 : (nw - 2) - (int)fmaxf(sc, 0.f);
-}
+// offset of the guessed older node for a delay of sc steps: (nw - 2) - floor(sc), negative ("older than the history")
+// when sc >= nw - 1 (the conversion saturates); a negative or NaN delay guesses the newest bracket
+__device__ __forceinline__ int guessed_offset(float sc, int nw) { return (nw - 2) - __float2int_rz(fmaxf(sc, 0.f)); }
 
 // bisection between offsets lo (P false) and hi (P true); returns lo
 template <bool SH>
@@ -237,15 +235,20 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
   __shared__ float4 s_q2[kTile];
   __shared__ float s_kq[kTile];
   __shared__ float4 s_q1[kTile];  // present record (lo, 0) of the tile's sources
-  __shared__ float4 s_x[kTile];   // out-of-history line at t_n, relative to the present position; gamma^2 of slot k0
-  // with the uniform-motion guess: the chord w_n - w_k0 and the oldest-slot bound's threshold, and slot k0's
-  // (beta - beta_ref, 1/gamma^2) (ext32)
+  // out of history: the line at t_n relative to the present position, and slot k0's velocity (ext32). s_x.w is
+  // kq / gamma^2 and s_k0 (beta, 1/gamma^2) of slot k0; for the adaptive step, which also needs dbeta and gamma^2 there,
+  // gamma^2 and (dbeta, 1/gamma^2)
+  __shared__ float4 s_x[kTile];
+  __shared__ float4 s_k0[kTile];
+  // with the uniform-motion guess: twice the chord w_n - w_k0 and the oldest-slot bound's threshold (ext32)
   constexpr int kTileG = PROP != kPropBisect ? kTile : 1;
   __shared__ float4 s_ck[kTileG];
-  __shared__ float4 s_k0[kTileG];
   __shared__ float s_acc[12][kBlock];  // per-thread compensated sums
 
   __shared__ int s_item;
+  // block constants read only when a tile is staged: shared memory instead of registers live across the pairs
+  __shared__ float s_inv_cdt;  // 1 / (c dt)
+  __shared__ int s_fac;        // first delay factor of the item's target group (learned proposal)
   const int N = a.N;
   const int D = a.D;
 
@@ -257,8 +260,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
   win.err = a.err;
   win.nw = (int)(n_abs - k0_abs) + 1;
   const int pn = a.state->pn;
-  const float inv_cdt = (float)(1.0 / (kC * a.state->dt));
-  const float nw1 = (float)(win.nw - 1);  // a guessed delay of at least nw - 1 steps is out of history
 
   // Counts and error bits. Node tests are counted per thread. The branch counts (added once per tile), the
   // FP64 fallbacks and the error bits (both rare) are kept in shared memory by the guessed-search
@@ -271,8 +272,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
     s_cnt[0] = s_cnt[1] = s_cnt[2] = 0;
     s_fallbacks = 0;
     s_err = 0;
+    s_inv_cdt = (float)(1.0 / (kC * a.state->dt));
   }
-  unsigned n_tests = 0, n_ooh = 0, n_sc = 0, n_bi = 0, n_fb = 0;
+  unsigned n_tests = 0;  // node tests beyond the first of each pair, which the branch counts hold
+  unsigned n_ooh = 0, n_sc = 0, n_bi = 0, n_fb = 0;
   int errbits = 0;
   auto set_err = [&](int bits) {
     if (kShared)
@@ -326,11 +329,13 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
   // learned proposal: the delay factors of this target tile's group (kFacGroup targets, a multiple of the
   // tile), one per source of the bunch
   // (as an index of a.fac relative to the bunch's first particle: the table has fewer than 2^31 entries)
-  const int fac_row = PROP == kPropMlp ? (int)(bd.fac_off + (long long)((tb * kBlock) / kFacGroup) * bd.n) - boff : 0;
-  // the lane's guessed older-node offset for staged source jj of the tile (-1: predicted out of history)
+  if (PROP == kPropMlp && threadIdx.x == 0)
+    s_fac = (int)(bd.fac_off + (long long)((tb * kBlock) / kFacGroup) * bd.n) - boff;
+  // the lane's guessed older-node offset for staged source jj of the tile (negative: predicted out of history)
   auto guess_of = [&](int jj) -> int {
-    const float sc = closed_form_ctau(r, s_q0[jj], s_q2[jj]) * inv_cdt;
-    return guessed_offset(sc, win.nw, nw1);
+    const float4 g0 = s_q0[jj];
+    const float3 d = separation(r, g0, s_q1[jj]);
+    return guessed_offset(guessed_steps(d, d.x * d.x + d.y * d.y + d.z * d.z, g0.w, s_q2[jj]), win.nw);
   };
   // beta_i(t_n) - beta_ref of the target (adaptive time step; target and sources share the bunch's beta_ref,
   // so relative velocities are formed from these small differences at full FP32 relative precision)
@@ -360,14 +365,21 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
       s_q0[threadIdx.x] = q[0];
       const float4 q2 = q[2];
       s_q2[threadIdx.x] = make_float4(bref01.x + q2.x, bref01.y + q2.y, bref2 + q2.z,
-                                      PROP == kPropMlp ? q2.w * __ldg(a.fac + (fac_row + j)) : q2.w);
-      s_kq[threadIdx.x] = a.kq32[j];
+                                      (PROP == kPropMlp ? q2.w * __ldg(a.fac + (s_fac + j)) : q2.w) * s_inv_cdt);
+      const float kq = a.kq32[j];
+      s_kq[threadIdx.x] = kq;
       s_q1[threadIdx.x] = q[1];
       const float4* e = a.ext32 + (size_t)j * kExtCount;
-      s_x[threadIdx.x] = __ldg(e + kExtLine);
+      float4 line = __ldg(e + kExtLine), old = __ldg(e + kExtOldest);
+      if (!ADAPT) {
+        line.w = __fmul_rn(kq, old.w);
+        old = make_float4(__fadd_rn(bref01.x, old.x), __fadd_rn(bref01.y, old.y), __fadd_rn(bref2, old.z), old.w);
+      }
+      s_x[threadIdx.x] = line;
+      s_k0[threadIdx.x] = old;
       if (PROP != kPropBisect) {
-        s_ck[threadIdx.x] = __ldg(e + kExtChord);
-        s_k0[threadIdx.x] = __ldg(e + kExtOldest);
+        const float4 ck = __ldg(e + kExtChord);
+        s_ck[threadIdx.x] = make_float4(2.f * ck.x, 2.f * ck.y, 2.f * ck.z, ck.w);
       }
     }
     __syncthreads();
@@ -434,20 +446,21 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           }
         }
         if (WIN && !active) continue;
-        if (j == i) continue;
+        // the target itself: d = 0 never passes the oldest-slot bound, so the guess's instances look after it
+        if ((PROP == kPropBisect || win.nw == 1) && j == i) continue;
         const float4* src32 = a.rec32 + (size_t)j * D * 3;
         const double* src64 = a.rec64 + (size_t)j * D * 6;
-        auto heaviside = [&](float2 dn01, float dn2, float4 o, float g2, int pk) {
+        auto heaviside = [&](float2 dn01, float dn2) {
           // ---- out of history (eq:linear2): the source moves uniformly with beta1 along the line through
           // w1; its Lienard-Wiechert field is Heaviside's field about the line's point at t_n,
           //   E = kq (1 - beta^2) X / [X^2 (1 - beta^2) + (X.beta)^2]^{3/2},  c B = beta x E,
           // with X = (r - w_n) - (line at t_n - w_n) from the staged present record and line offset.
-          const float4 gx = s_x[jj];
+          const float4 gx = s_x[jj], o = s_k0[jj];
           const float2 X01 = sub2(dn01, gx);
           float X0 = X01.x, X1 = X01.y;
           float X2 = __fsub_rn(dn2, gx.z);
-          const float2 b101 = __fadd2_rn(bref01, make_float2(o.x, o.y));
-          const float b10 = b101.x, b11 = b101.y, b12 = __fadd_rn(bref2, o.z);
+          const float b10 = ADAPT ? __fadd_rn(bref01.x, o.x) : o.x, b11 = ADAPT ? __fadd_rn(bref01.y, o.y) : o.y;
+          const float b12 = ADAPT ? __fadd_rn(bref2, o.z) : o.z;
           const float ig2 = o.w;
           float Xb = dot3(X0, X1, X2, b10, b11, b12);
           float XX = dot3(X0, X1, X2, X0, X1, X2);
@@ -456,8 +469,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           // near perpendicular to beta) X and X.beta are formed in FP64 from the FP64 records instead.
           // (as the shift is at most u gamma, sources with gamma^2 < 100 never need it)
           if (ig2 < 0.01f && __fmul_rn(kXbGuard, __fmul_rn(sqrtf(XX), fabsf(Xb))) > __fmaf_rn(XX, ig2, __fmul_rn(Xb, Xb))) {
-            const double* w0 = src64 + 6 * pk;  // FP64 record of slot k0: X = r - w_k0 - v_k0 (t_n - t_k0)
-            const double ct = kC * (a.state->t - __ldg(a.slot_t + pk));  // c (t_n - t_k0)
+            const double* w0 = src64 + 6 * win.p0;  // FP64 record of slot k0: X = r - w_k0 - v_k0 (t_n - t_k0)
+            const double ct = kC * (a.state->t - __ldg(a.slot_t + win.p0));  // c (t_n - t_k0)
             const double ic = 1.0 / kC;
             const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
             const double y0 = (__ldg(rr + 0) - __ldg(w0 + 0)) - __ldg(w0 + 3) * ic * ct;
@@ -476,11 +489,11 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
             set_err((ig2 > 0.f) ? kErrCoincide : kErrDisc);
             return;
           }
-          const float pref = __fmul_rn(__fmul_rn(s_kq[jj], ig2), __fmul_rn(__fmul_rn(iD, iD), iD));
+          const float pref = __fmul_rn(ADAPT ? __fmul_rn(s_kq[jj], ig2) : gx.w, __fmul_rn(__fmul_rn(iD, iD), iD));
           if (ADAPT) {
             // retarded distance c (t - t_r) = gamma^2 [X.beta + sqrt(Dh)], and v(t_r) = v1
             const float sD = __fmul_rn(Dh, iD);
-            const float R = (Xb >= 0.f) ? __fmul_rn(__fadd_rn(Xb, sD), g2)
+            const float R = (Xb >= 0.f) ? __fmul_rn(__fadd_rn(Xb, sD), gx.w)
                                         : __fdividef(dot3(X0, X1, X2, X0, X1, X2), __fsub_rn(sD, Xb));
             if (R >= a.eta_allow) {
               emin = fminf(emin, R);
@@ -492,13 +505,11 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           P[0] = p01.x;
           P[1] = p01.y;
           P[2] = __fmaf_rn(pref, X2, P[2]);
-          // c B = beta x E = pref (beta x X)
-          const float2 p34 = __ffma2_rn(make_float2(pref, pref),
-                                        make_float2(cross1(b11, b12, X1, X2), cross1(b12, b10, X2, X0)),
-                                        make_float2(P[3], P[4]));
-          P[3] = p34.x;
-          P[4] = p34.y;
-          P[5] = __fmaf_rn(pref, cross1(b10, b11, X0, X1), P[5]);
+          // c B = beta x E = (pref beta) x X
+          const float h0 = __fmul_rn(pref, b10), h1 = __fmul_rn(pref, b11), h2 = __fmul_rn(pref, b12);
+          P[3] = __fmaf_rn(h1, X2, __fmaf_rn(-h2, X1, P[3]));
+          P[4] = __fmaf_rn(h2, X0, __fmaf_rn(-h0, X2, P[4]));
+          P[5] = __fmaf_rn(h0, X1, __fmaf_rn(-h1, X0, P[5]));
         };
         // ---- bracket: offset l1 of the older node, its slot pA, record A, separation dA and table -------
         int l1;
@@ -512,7 +523,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
         bool fast = true;  // pA, A, dA and tabA already belong to l1
         if (win.nw == 1) {
           // n = k0: only the present slot exists; every pair is out of history
-          n_tests += 1;
           l1 = 0;
           br = 0;
           pA = win.phys(0);
@@ -520,7 +530,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           dA = separation(r, A.q0, A.q1);
           tabA = __ldg(a.tab32 + pA);
         } else if (PROP == kPropBisect) {
-          n_tests += 1;
           pA = win.phys(0);
           A = load_rec(src32, pA);
           dA = separation(r, A.q0, A.q1);
@@ -540,24 +549,25 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
             fast = (l1 == 0);
           }
         } else {
-          // the uniform-motion delay (with the learned proposal scaled by the network's factor for the
-          // block's target group and this source, staged in s_q2)
-          const int lraw = WIN ? g_cur : guess_of(jj);
-          // predicted out of history: the oldest-slot bound (kChordMargin) from the present separation and
-          // the staged chord; where it holds, slot k0's node test is true without its record
-          if (lraw < 0 && !r.exact_only) {
+          // The oldest-slot bound (kChordMargin) first, from the present separation and the staged chord: where it
+          // holds, slot k0's node test is true without its record, and no guess is needed.
+          const float4 g0 = s_q0[jj];
+          const float3 dn = separation(r, g0, s_q1[jj]);
+          const float dd = dn.x * dn.x + dn.y * dn.y + dn.z * dn.z;
+          {
             const float4 ck = s_ck[jj];
-            const float3 dn = separation(r, s_q0[jj], s_q1[jj]);
-            const float dd = dn.x * dn.x + dn.y * dn.y + dn.z * dn.z;
-            const float dc = dn.x * ck.x + dn.y * ck.y + dn.z * ck.z;
-            if (fmaf(2.f, dc, dd * kChordLo) > ck.w) {
-              n_tests += 1;
+            const float dc2 = dn.x * ck.x + dn.y * ck.y + dn.z * ck.z;
+            if (!r.exact_only && fmaf(dd, kChordLo, dc2) > ck.w) {
               brc += 1u;
               if (DUMP) a.dump[(size_t)i * N + j] = 0;
-              heaviside(make_float2(dn.x, dn.y), dn.z, s_k0[jj], s_x[jj].w, win.phys(0));
+              heaviside(make_float2(dn.x, dn.y), dn.z);
               continue;
             }
           }
+          if (j == i) continue;
+          // the uniform-motion delay (with the learned proposal scaled by the network's factor for the
+          // block's target group and this source, staged in s_q2)
+          const int lraw = WIN ? g_cur : guessed_offset(guessed_steps(dn, dd, g0.w, s_q2[jj]), win.nw);
           const int lg = max(lraw, 0);
           pA = win.phys(lg);
           // records of the guessed bracket: from the staged window when both lie in it
@@ -575,7 +585,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           tabA = __ldg(a.tab32 + pA);
           if (lraw < 0) {
             // predicted out of history: the only record needed is the oldest slot's
-            n_tests += 1;
             if (node_test_d<kShared>(r, dA, tabA, src64, pA, a, n_fb)) {
               l1 = 0;
               br = 0;
@@ -609,7 +618,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
             } else {
               Bn = load_rec(src32, pg1);
             }
-            n_tests += 1;
             const bool tA = node_test_d<kShared>(r, dA, tabA, src64, pA, a, n_fb);
             if (!tA) {
               bool tB = true;  // P(n) is always true
@@ -679,9 +687,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
         if (DUMP) a.dump[(size_t)i * N + j] = 4 * l1 + br;
 
         if (br == 0) {
-          const float4 g0 = s_q0[jj], g1 = s_q1[jj];
-          heaviside(__fadd2_rn(sub2(r.h01, g0), sub2(r.l01, g1)), __fadd_rn(__fsub_rn(r.h2, g0.z), __fsub_rn(r.l2, g1.z)),
-                    make_float4(A.q2.x, A.q2.y, A.q2.z, A.q0.w), A.q2.w, pA);
+          const float3 dn = separation(r, s_q0[jj], s_q1[jj]);
+          heaviside(make_float2(dn.x, dn.y), dn.z);
           continue;
         }
         if (!ADAPT) {
@@ -988,6 +995,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
     if (s_cnt[0]) atomicAdd(a.stats + kStatOOH, s_cnt[0]);
     if (s_cnt[1]) atomicAdd(a.stats + kStatShortcut, s_cnt[1]);
     if (s_cnt[2]) atomicAdd(a.stats + kStatBisect, s_cnt[2]);
+    const unsigned long long pairs = s_cnt[0] + s_cnt[1] + s_cnt[2];
+    if (pairs) atomicAdd(a.stats + kStatNodeTests, pairs);
     if (s_fallbacks) atomicAdd(a.stats + kStatGuard, s_fallbacks);
     if (s_err) atomicOr(a.err, s_err);
   }

@@ -142,8 +142,8 @@ __global__ void prep_kernel(DeviceState s) {
 //     source moves uniformly, so its field is Heaviside's field about the point w_{j,n} + X_j; the
 //     separation from a target is then (r - w_{j,n}) - X_j, formed without cancellation.
 //   c_j = w_{j,n} - w_{j,k0} and T (1 + 32u) - |c_j|^2 (1 - 32u), rounded up, with T the FP32 upper
-//     threshold of slot k0: the oldest-slot bound (kChordMargin), by which an out-of-history pair's
-//     node test of slot k0 needs no record of that slot; and the FP32 record's beta - beta_ref,
+//     threshold of slot k0 (and at least 0, so that d = 0 never passes): the oldest-slot bound (kChordMargin),
+//     by which an out-of-history pair's node test of slot k0 needs no record of that slot; and the FP32 record's beta - beta_ref,
 //     1/gamma^2 and gamma^2 of slot k0, which Heaviside's field of that pair reads.
 // For the FP64 path, per source, the out-of-history line of eq:linear2 in FP64 (kExt64): the present position,
 // X_j of the same line, its velocity and the factors of Heaviside's field that no target changes.
@@ -193,7 +193,7 @@ __global__ void setup_kernel(DeviceState s, SetupExt extrap) {
     const double cc = c0 * c0 + c1 * c1 + c2 * c2;
     const double rhs = (double)upper_threshold(__dmul_rn(ct, ct)) * (1.0 + kChordMargin) - cc * (1.0 - kChordMargin);
     const float inf = __int_as_float(0x7f800000);
-    ext[kExtChord] = make_float4((float)c0, (float)c1, (float)c2, n > k0 ? __double2float_ru(rhs) : inf);
+    ext[kExtChord] = make_float4((float)c0, (float)c1, (float)c2, n > k0 ? fmaxf(__double2float_ru(rhs), 0.f) : inf);
   }
   if (n <= k0) return;  // no segment [n-1, n] in the window
   const int p1 = pn == 0 ? s.D - 1 : pn - 1;
