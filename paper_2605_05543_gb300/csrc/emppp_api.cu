@@ -781,21 +781,19 @@ EMPPP_API emppp_status emppp_set_history(emppp_handle h, int64_t n, int32_t nslo
   const double* Vlast = V + (size_t)(nslots - 1) * N * 3;
   if ((st = set_bunch_frames(h, Wlast, Vlast, false, is_device_ptr)) != EMPPP_OK) return st;
   std::vector<double> ht((size_t)h->D, 0.0);
-  for (int s = 0; s < nslots; s++) {
-    const int64_t k = n - nslots + 1 + s;
-    const int p = (int)(k % h->D);
-    ht[p] = hT[s];
-    const double* Ws = W + (size_t)s * N * 3;
-    const double* Vs = V + (size_t)s * N * 3;
-    if (!is_device_ptr) {
-      if ((st = to_device(h, h->staging, Ws, 3 * N, 0)) != EMPPP_OK) return st;
-      if ((st = to_device(h, h->staging + 3 * N, Vs, 3 * N, 0)) != EMPPP_OK) return st;
-      Ws = h->staging;
-      Vs = h->staging + 3 * N;
-    }
-    CU(launch_scatter_slot(h->ds, p, Ws, Vs, h->stream));
+  const int p_first = (int)((n - nslots + 1) % h->D);
+  for (int s = 0; s < nslots; s++) ht[(p_first + s) % h->D] = hT[s];
+  if (is_device_ptr) {
+    CU(launch_scatter_history(h->ds, p_first, nslots, W, V, h->stream));
     h->launches += 1;
-    if (!is_device_ptr) CU(cudaStreamSynchronize(h->stream));  // staging is reused by the next slot
+  } else {
+    for (int s = 0; s < nslots; s++) {
+      if ((st = to_device(h, h->staging, W + (size_t)s * N * 3, 3 * N, 0)) != EMPPP_OK) return st;
+      if ((st = to_device(h, h->staging + 3 * N, V + (size_t)s * N * 3, 3 * N, 0)) != EMPPP_OK) return st;
+      CU(launch_scatter_slot(h->ds, (p_first + s) % h->D, h->staging, h->staging + 3 * N, h->stream));
+      h->launches += 1;
+      CU(cudaStreamSynchronize(h->stream));  // staging is reused by the next slot
+    }
   }
   CU(cudaMemcpyAsync(h->ds.slot_t, ht.data(), sizeof(double) * h->D, cudaMemcpyHostToDevice, h->stream));
   const double* du = u;

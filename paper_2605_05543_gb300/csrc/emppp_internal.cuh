@@ -290,6 +290,8 @@ __device__ __forceinline__ void decode_item(const BunchSched* __restrict__ sched
 cudaError_t launch_init_slot0(const DeviceState& s, const double* x, const double* u, const double* w,
                               cudaStream_t st);
 cudaError_t launch_scatter_slot(const DeviceState& s, int p, const double* W, const double* V, cudaStream_t st);
+cudaError_t launch_scatter_history(const DeviceState& s, int p_first, int nslots, const double* W, const double* V,
+                                   cudaStream_t st);
 cudaError_t launch_gather_slot(const DeviceState& s, int p, double* W, double* V, cudaStream_t st);
 cudaError_t launch_set_state(const DeviceState& s, long long n, double t, double dt, long long hist_start,
                              const double* u, const double* w, cudaStream_t st);

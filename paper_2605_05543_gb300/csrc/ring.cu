@@ -1,24 +1,31 @@
 // History ring (Sec. 2.2: positions and velocities stored at discrete steps; the acceleration is not
 // stored) and per-step slot tables.
 #include "emppp_internal.cuh"
+#include "fp64_roots.cuh"
 #include "shadow.cuh"
 
 namespace emppp {
 
-// Writes record (j, p) of both rings from an FP64 position and velocity.
-__device__ __forceinline__ void write_record(const DeviceState& s, long long j, int p, double w0, double w1,
-                                             double w2, double v0, double v1, double v2) {
+// Writes record (j, p) of both rings from an FP64 position and velocity, gamma^2 and its inverse.
+__device__ __forceinline__ void write_record(const DeviceState& s, long long j, int p, double w0, double w1, double w2,
+                                             double v0, double v1, double v2, double gamma2, double inv_gamma2) {
   double* r = s.rec64 + ((size_t)j * s.D + p) * 6;
   reinterpret_cast<double2*>(r)[0] = make_double2(w0, w1);
   reinterpret_cast<double2*>(r)[1] = make_double2(w2, v0);
   reinterpret_cast<double2*>(r)[2] = make_double2(v1, v2);
   float4 q[3];
   const BunchDesc& bd = s.bunches[s.bunch_of[j]];
-  shadow_record(bd.origin, bd.beta_ref, w0, w1, w2, v0, v1, v2, gamma2_of_v(v0, v1, v2), q);
+  shadow_record(bd.origin, bd.beta_ref, w0, w1, w2, v0, v1, v2, gamma2, inv_gamma2, q);
   float4* o = reinterpret_cast<float4*>(s.rec32 + ((size_t)j * s.D + p) * 12);
   o[0] = q[0];
   o[1] = q[1];
   o[2] = q[2];
+}
+
+__device__ __forceinline__ void write_record(const DeviceState& s, long long j, int p, double w0, double w1, double w2,
+                                             double v0, double v1, double v2) {
+  const double gamma2 = gamma2_of_v(v0, v1, v2);
+  write_record(s, j, p, w0, w1, w2, v0, v1, v2, gamma2, 1.0 / gamma2);
 }
 
 // v = u / gamma with gamma = sqrt(1 + u.u / c^2), in the operation order of a plain FP64 evaluation
@@ -53,6 +60,33 @@ __global__ void scatter_slot_kernel(DeviceState s, int p, const double* __restri
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= s.N) return;
   write_record(s, j, p, W[3 * j], W[3 * j + 1], W[3 * j + 2], V[3 * j], V[3 * j + 1], V[3 * j + 2]);
+}
+
+// All slots of a history held on the device (W, V [nslots][N][3], the layout of emppp_set_history) in one launch:
+// slot s goes to physical slot (p_first + s) mod D. What bounds it is memory (24 + 24 bytes read and 96 written per
+// record) and, close behind, the FP64 operations of the FP32 record. A thread takes kScatterSlots consecutive slots of
+// one particle: the reads of a warp are contiguous over its particles, and the 48-byte records that one thread writes
+// follow one another, so that their sectors fill in L2. N = 8192, 301 slots: 0.22 ms instead of 1.85 ms for one launch
+// per slot.
+constexpr int kScatterSlots = 8;
+
+__global__ void __launch_bounds__(256) scatter_history_kernel(DeviceState s, int p_first, int nslots,
+                                                              const double* __restrict__ W,
+                                                              const double* __restrict__ V) {
+  const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= s.N) return;
+  const int s0 = blockIdx.y * kScatterSlots, s1 = min(nslots, s0 + kScatterSlots);
+  int p = p_first + s0;
+  if (p >= s.D) p -= s.D;
+  for (int k = s0; k < s1; k++) {
+    const double* w = W + ((size_t)k * s.N + j) * 3;
+    const double* v = V + ((size_t)k * s.N + j) * 3;
+    const double v0 = __ldg(v), v1 = __ldg(v + 1), v2 = __ldg(v + 2);
+    // 1 / gamma^2 = 1 - v.v / c^2 and its reciprocal without divisions (both are rounded to FP32)
+    const double ig2 = 1.0 - (v0 * v0 + v1 * v1 + v2 * v2) * (1.0 / (kC * kC));
+    write_record(s, j, p, __ldg(w), __ldg(w + 1), __ldg(w + 2), v0, v1, v2, recip_refined(ig2), ig2);
+    p = p + 1 == s.D ? 0 : p + 1;
+  }
 }
 
 __global__ void gather_slot_kernel(DeviceState s, int p, double* __restrict__ W, double* __restrict__ V) {
@@ -238,6 +272,18 @@ cudaError_t launch_init_slot0(const DeviceState& s, const double* x, const doubl
 
 cudaError_t launch_scatter_slot(const DeviceState& s, int p, const double* W, const double* V, cudaStream_t st) {
   scatter_slot_kernel<<<blocks_for(s.N, 256), 256, 0, st>>>(s, p, W, V);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_scatter_history(const DeviceState& s, int p_first, int nslots, const double* W, const double* V,
+                                   cudaStream_t st) {
+  // blockIdx.y counts groups of slots: at most 65535 of them per launch
+  constexpr int kMost = 65535 * kScatterSlots;
+  for (int k = 0; k < nslots; k += kMost) {
+    const int m = nslots - k < kMost ? nslots - k : kMost;
+    scatter_history_kernel<<<dim3(blocks_for(s.N, 256), blocks_for(m, kScatterSlots)), 256, 0, st>>>(
+        s, (int)(((long long)p_first + k) % s.D), m, W + (size_t)k * s.N * 3, V + (size_t)k * s.N * 3);
+  }
   return cudaGetLastError();
 }
 

@@ -15,14 +15,20 @@
 namespace emppp {
 
 __device__ __forceinline__ void shadow_record(const double origin[3], const double beta_ref[3], double w0, double w1,
-                                              double w2, double v0, double v1, double v2, double gamma2, float4 q[3]) {
+                                              double w2, double v0, double v1, double v2, double gamma2, double inv_gamma2,
+                                              float4 q[3]) {
   const double d0 = w0 - origin[0], d1 = w1 - origin[1], d2 = w2 - origin[2];
   const float h0 = (float)d0, h1 = (float)d1, h2 = (float)d2;
   const double ic = 1.0 / kC;
-  q[0] = make_float4(h0, h1, h2, (float)(1.0 / gamma2));
+  q[0] = make_float4(h0, h1, h2, (float)inv_gamma2);
   q[1] = make_float4((float)(d0 - (double)h0), (float)(d1 - (double)h1), (float)(d2 - (double)h2), 0.f);
   q[2] = make_float4((float)(v0 * ic - beta_ref[0]), (float)(v1 * ic - beta_ref[1]), (float)(v2 * ic - beta_ref[2]),
                      (float)gamma2);
+}
+
+__device__ __forceinline__ void shadow_record(const double origin[3], const double beta_ref[3], double w0, double w1,
+                                              double w2, double v0, double v1, double v2, double gamma2, float4 q[3]) {
+  shadow_record(origin, beta_ref, w0, w1, w2, v0, v1, v2, gamma2, 1.0 / gamma2, q);
 }
 
 // gamma^2 of a stored velocity: 1 / (1 - v.v / c^2)
