@@ -783,6 +783,7 @@ EMPPP_API emppp_status emppp_set_history(emppp_handle h, int64_t n, int32_t nslo
   std::vector<double> ht((size_t)h->D, 0.0);
   const int p_first = (int)((n - nslots + 1) % h->D);
   for (int s = 0; s < nslots; s++) ht[(p_first + s) % h->D] = hT[s];
+  CU(cudaMemcpyAsync(h->ds.slot_t, ht.data(), sizeof(double) * h->D, cudaMemcpyHostToDevice, h->stream));
   if (is_device_ptr) {
     CU(launch_scatter_history(h->ds, p_first, nslots, W, V, h->stream));
     h->launches += 1;
@@ -790,12 +791,12 @@ EMPPP_API emppp_status emppp_set_history(emppp_handle h, int64_t n, int32_t nslo
     for (int s = 0; s < nslots; s++) {
       if ((st = to_device(h, h->staging, W + (size_t)s * N * 3, 3 * N, 0)) != EMPPP_OK) return st;
       if ((st = to_device(h, h->staging + 3 * N, V + (size_t)s * N * 3, 3 * N, 0)) != EMPPP_OK) return st;
-      CU(launch_scatter_slot(h->ds, (p_first + s) % h->D, h->staging, h->staging + 3 * N, h->stream));
+      CU(launch_scatter_slot(h->ds, (p_first + s) % h->D, s > 0 ? hT[s] - hT[s - 1] : 0.0, h->staging, h->staging + 3 * N,
+                             h->stream));
       h->launches += 1;
       CU(cudaStreamSynchronize(h->stream));  // staging is reused by the next slot
     }
   }
-  CU(cudaMemcpyAsync(h->ds.slot_t, ht.data(), sizeof(double) * h->D, cudaMemcpyHostToDevice, h->stream));
   const double* du = u;
   const double* dw = w;
   if (!is_device_ptr) {

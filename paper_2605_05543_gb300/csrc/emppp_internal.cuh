@@ -9,7 +9,7 @@
 //                             w (3) and velocity v (3) at the time slot_t[p]; slots are used
 //                             modulo D, so one particle's whole history is one contiguous 48*D-byte
 //                             run (pair gathers of one source stay within a few cache lines).
-//   rec32  [N][D][12] float   FP32 shadow of rec64 (shadow.cuh): hi(3) 1/gamma^2 | lo(3) 0 |
+//   rec32  [N][D][12] float   FP32 shadow of rec64 (shadow.cuh): hi(3) 1/gamma^2 | lo(3) dev |
 //                             beta - beta_ref (3) gamma^2; 48-byte records, three 16-byte loads each;
 //                             origin and beta_ref are per bunch.
 //   slot_t [D]                time stamp of each physical slot.
@@ -112,6 +112,20 @@ constexpr float kLowerRatio = (float)(((1.0 - kGuardBand) / (1.0 + kGuardBand)) 
 // rounded up (setup_kernel); kChordLo is 1 - 32u.
 constexpr double kChordMargin = 32.0 * 5.9604644775390625e-08;
 constexpr float kChordLo = 1.0f - 32.0f * 5.9604644775390625e-08f;
+
+// Newer-node bound of the mixed path. A pair whose guessed older node A tests false solves the line w_A + v_A (t - t_A)
+// for tau = c (t_n - t_r) with half-discriminant sq. phi(s) = |p + beta s| - s (p the separation from the line at
+// t_n) is convex with phi(tau) = 0 and slope -sq / tau there, so at L_B = c (t_n - t_B) < tau, phi(L_B) >= (sq /
+// tau) (tau - L_B); the stored node B lies within dev of the line, so |r - w_B| >= L_B + phi(L_B) - dev. In FP32 p
+// carries an absolute error below 7u L_A (two roundings of each component of d, three fused products), beta one of
+// 1.5u, phi(tau) as computed one below 12u tau and (1 - f) sq, with 1 - f = (tau - L_B) / (c dt), one below 6u tau
+// in units of c dt: 27u L_A in all; the slope is off by less than 3 % for gamma^2 up to kDevGamma2. So if
+//   (1 - f) sq  >  tau / (c dt) [33u L_A + 1.03 dev]
+// as computed, the exact |r - w_B| exceeds L_B by more than 5u L_A, far above the FP64 test's rounding: P(B) is
+// true. The FP32 record of A holds 1.03 dev in q1.w (rounded up), +inf while it has no newer node or above
+// kDevGamma2, which leaves the test to the node itself.
+constexpr float kNewerMargin = 33.0f * 5.9604644775390625e-08f;
+constexpr double kDevGamma2 = 16384.0;
 
 // per-source float4s of ext32 (mixed path)
 enum {
@@ -289,7 +303,7 @@ __device__ __forceinline__ void decode_item(const BunchSched* __restrict__ sched
 // ring.cu
 cudaError_t launch_init_slot0(const DeviceState& s, const double* x, const double* u, const double* w,
                               cudaStream_t st);
-cudaError_t launch_scatter_slot(const DeviceState& s, int p, const double* W, const double* V, cudaStream_t st);
+cudaError_t launch_scatter_slot(const DeviceState& s, int p, double dt, const double* W, const double* V, cudaStream_t st);
 cudaError_t launch_scatter_history(const DeviceState& s, int p_first, int nslots, const double* W, const double* V,
                                    cudaStream_t st);
 cudaError_t launch_gather_slot(const DeviceState& s, int p, double* W, double* V, cudaStream_t st);

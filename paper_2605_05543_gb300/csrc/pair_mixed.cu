@@ -7,16 +7,19 @@
 //             (kGuardBand, emppp_internal.cuh); beyond them the FP32 decision is the FP64 one, between
 //             them the FP64 test itself (reference operation order) decides. The bracket is therefore
 //             the FP64 one. Search: the paper's bisection, or the guarded galloping
-//             search from the uniform-motion guess; with the guess, the records of the one or two slots
-//             the guess points at are loaded together, so a correct guess needs a single gather round.
+//             search from the uniform-motion guess. With the guess and a fixed step, the older node's record and the
+//             newer one's velocity are loaded together; the line solve then mostly shows the newer node's test
+//             true without its position (newer-node bound, kNewerMargin in emppp_internal.cuh), which saves
+//             three of a pair's eight gathers: 31.0 to 29.0 ms at N = 65536, where the L1 wavefronts of the
+//             gathers (19 lines per 16-byte load of a warp) weigh as much as the instructions.
 //             Before any guess a pair tries the oldest-slot bound (kChordMargin, emppp_internal.cuh): from the
 //             staged present separation and the source's chord, it shows the oldest slot's FP32 test true at
 //             its first comparison without loading that slot's record. It decides most pairs beyond the
 //             history, whose field reads staged vectors alone, so that they need no guess (with the guess
 //             first: 32.6 against 30.8 ms at N = 65536, 251 slots).
 //   retarded  and fields, fixed step: from the source's line at t_n (at the code below).
-//   retarded  adaptive step: the textbook forms, kept because the last bit of |eta| and v_j(t_r) decides the
-//             step and with it every later time stamp: in light units (lengths in m, velocities as beta = v/c): with L1 = c (t - t1) and d = r - w1,
+//   retarded  adaptive step: the textbook forms, whose every rounding is kept: the last bit of |eta| and v_j(t_r)
+//             decides the step and with it every later time stamp: in light units (lengths in m, velocities as beta = v/c): with L1 = c (t - t1) and d = r - w1,
 //             (1 - beta1^2) s^2 + 2 (d.beta1 - L1) s + (L1^2 - |d|^2) = 0 for s = c (t_r - t1) (eq:dt),
 //             smaller root without cancellation; eta = d - beta1 s (eq:linear, retarded position w1 + v1 dt);
 //             in the near-field shortcut bracket the same point is formed from the segment's end
@@ -51,6 +54,13 @@ namespace {
 #ifndef EMPPP_MIXED_MIN_BLOCKS
 #define EMPPP_MIXED_MIN_BLOCKS 8  // resident blocks per SM the register budget is fitted to (64 registers)
 #endif
+
+// Resident blocks per SM, of 128 threads: 8 at 64 registers (N = 32768: 7.69 ms; 7 at 72 registers 8.08, 9 at 56 with
+// spills 10.0). The history-window shape holds more state across a pair and spills 132 bytes at 64 registers: 7 blocks
+// (N = 16384: 3.21 ms against 3.88 at 8 and 3.41 at 6).
+constexpr int mixed_min_blocks(int shape) {
+  return (shape_win(shape) > 0 ? EMPPP_MIXED_MIN_BLOCKS - 1 : EMPPP_MIXED_MIN_BLOCKS) * 128 / shape_block(shape);
+}
 
 // FP64 recomputation of C0 when u L1^2 |s| / (C0 (L1 - s)) exceeds 2e-6: kC0Guard = 2e-6 / u
 constexpr float kC0Guard = 2.0e-6f / 5.9604644775390625e-08f;
@@ -212,7 +222,7 @@ __device__ __forceinline__ int bisect(const Target& r, const float4* __restrict_
 // SHAPE: targets per block (kBlock), sources per FP32 partial sum (kSub); the
 // register budget stays at 64 per thread for every block size
 template <int PROP, bool ADAPT, bool DUMP, int SHAPE>
-__global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 128 / shape_block(SHAPE))
+__global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
     pair_mixed_kernel(MixedArgs a) {
   constexpr int kBlock = shape_block(SHAPE);
   // sources per staged tile: half a block's targets, which keeps 8 blocks of the (128, *) shapes within the
@@ -505,11 +515,112 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           P[0] = p01.x;
           P[1] = p01.y;
           P[2] = __fmaf_rn(pref, X2, P[2]);
-          // c B = beta x E = (pref beta) x X
-          const float h0 = __fmul_rn(pref, b10), h1 = __fmul_rn(pref, b11), h2 = __fmul_rn(pref, b12);
-          P[3] = __fmaf_rn(h1, X2, __fmaf_rn(-h2, X1, P[3]));
-          P[4] = __fmaf_rn(h2, X0, __fmaf_rn(-h0, X2, P[4]));
-          P[5] = __fmaf_rn(h0, X1, __fmaf_rn(-h1, X0, P[5]));
+          if (ADAPT) {
+            // c B = beta x E = pref (beta x X), in the sequence that adaptive runs have always had: a last place of a field
+            // moves the particles, and with them now and then the last place of |eta|, which is the step
+            const float2 p34 = __ffma2_rn(make_float2(pref, pref),
+                                          make_float2(cross1(b11, b12, X1, X2), cross1(b12, b10, X2, X0)),
+                                          make_float2(P[3], P[4]));
+            P[3] = p34.x;
+            P[4] = p34.y;
+            P[5] = __fmaf_rn(pref, cross1(b10, b11, X0, X1), P[5]);
+          } else {
+            // c B = beta x E = (pref beta) x X
+            const float h0 = __fmul_rn(pref, b10), h1 = __fmul_rn(pref, b11), h2 = __fmul_rn(pref, b12);
+            P[3] = __fmaf_rn(h1, X2, __fmaf_rn(-h2, X1, P[3]));
+            P[4] = __fmaf_rn(h2, X0, __fmaf_rn(-h0, X2, P[4]));
+            P[5] = __fmaf_rn(h0, X1, __fmaf_rn(-h1, X0, P[5]));
+          }
+        };
+        // ---- the fields of a bracketed pair (fixed step) from its older record A, separation dA, table entry and the
+        // newer node's velocity; with check_b false (and nothing added) unless the newer-node bound holds
+        auto line_fields = [&](const Rec& A, float3 dA, float4 tabA, float4 q2b, int pA, int br, bool check_b) -> bool {
+          // ---- retarded state and fields from the source's line at t_n (light units) ------------------
+          // p is the target's separation from where the line of the older node is at t_n, tau = c (t_n - t_r) = R
+          // the positive root of (1 - beta1^2) tau^2 - 2 (p.beta1) tau - |p|^2 = 0, whose half-discriminant Dh is a
+          // sum of non-negative terms. With f = (t_r - t1) / (t2 - t1), g = beta2 - beta1, eta = p + beta1 tau and
+          // beta = beta1 + f g: kappa = R - eta.beta = sqrt(Dh) - f eta.g, A = 1 - beta^2 + eta.alpha (alpha =
+          // g / (c dt)), H = A beta + kappa alpha, and eq:LW_E, eq:LW_B are E = kq (A eta - tau H) / kappa^3,
+          // c B = kq (H x eta) / kappa^3: no second root, no division by R, no double cross product.
+          // Rounding sequence fixed as below (no packed product feeds a packed sum).
+          const float L1 = tabA.z, icdt = tabA.w;
+          const float ig2 = A.q0.w;
+          const float2 b101 = __fadd2_rn(bref01, make_float2(A.q2.x, A.q2.y));
+          const float b10 = b101.x, b11 = b101.y, b12 = __fadd_rn(bref2, A.q2.z);
+          float2 p01;
+          float p2;
+          if (br == 1) {
+            // near-field shortcut: the end of the last segment, formed per source in FP64 (ext32), since p cancels
+            // when R is far below c (t_n - t_{n-1})
+            const float4* e = a.ext32 + (size_t)j * kExtCount;
+            const float3 dp = separation(r, __ldg(e + kExtSegHi), __ldg(e + kExtSegLo));
+            p01 = make_float2(dp.x, dp.y);
+            p2 = dp.z;
+          } else {
+            // d - beta1 L1 with beta1 = beta_ref + dbeta and L1 in two parts each
+            p01 = __ffma2_rn(make_float2(-bref01.x, -bref01.y), make_float2(L1, L1), make_float2(dA.x, dA.y));
+            p01 = __ffma2_rn(make_float2(-A.q2.x, -A.q2.y), make_float2(L1, L1), p01);
+            p01 = __ffma2_rn(make_float2(-b10, -b11), make_float2(tabA.y, tabA.y), p01);
+            p2 = __fmaf_rn(-b12, tabA.y, __fmaf_rn(-A.q2.z, L1, __fmaf_rn(-bref2, L1, dA.z)));
+          }
+          float pv = dot3(p01.x, p01.y, p2, b10, b11, b12);
+          float pp = dot3(p01.x, p01.y, p2, p01.x, p01.y, p2);
+          float Dh = __fmaf_rn(pp, ig2, __fmul_rn(pv, pv));
+          float sq = __fmul_rn(Dh, rsqrtf(Dh));
+          // The rounding of p (about u L1) moves tau by up to u L1 / (2 sqrt(Dh)) of itself. Where that exceeds 2e-6
+          // (sources moving nearly towards the target at high gamma; below 2 u gamma^2, so never for gamma^2 < 16)
+          // p is formed in FP64 from the FP64 records.
+          if (br == 2 && ig2 < 0.0625f && L1 > __fmul_rn(kLineGuard, sq)) {
+            const double* w64 = src64 + 6 * pA;
+            const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
+            const double T1 = __ldg(a.tab64 + pA).x;
+            p01.x = (float)((__ldg(rr + 0) - __ldg(w64 + 0)) - __ldg(w64 + 3) * T1);
+            p01.y = (float)((__ldg(rr + 1) - __ldg(w64 + 1)) - __ldg(w64 + 4) * T1);
+            p2 = (float)((__ldg(rr + 2) - __ldg(w64 + 2)) - __ldg(w64 + 5) * T1);
+            pv = dot3(p01.x, p01.y, p2, b10, b11, b12);
+            pp = dot3(p01.x, p01.y, p2, p01.x, p01.y, p2);
+            Dh = __fmaf_rn(pp, ig2, __fmul_rn(pv, pv));
+            sq = __fmul_rn(Dh, rsqrtf(Dh));
+            count_fallback<kShared>(n_fb);
+          }
+          const float sum = __fadd_rn(sq, fabsf(pv));
+          const bool pos = pv >= 0.f;
+          const float tau = __fmul_rn(pos ? sum : pp, pos ? A.q2.w : __fdividef(1.f, sum));
+          const float f = __fmul_rn(__fsub_rn(L1, tau), icdt);
+          // The newer-node bound (kNewerMargin, emppp_internal.cuh): the solve shows the newer node's test true without
+          // that node's position
+          if (check_b && !(__fmaf_rn(-f, sq, sq) > __fmul_rn(__fmul_rn(tau, icdt), __fmaf_rn(kNewerMargin, L1, A.q1.w))))
+            return false;
+          const float2 g01 = sub2(make_float2(q2b.x, q2b.y), A.q2);
+          const float g2 = __fsub_rn(q2b.z, A.q2.z);
+          const float2 e01 = __ffma2_rn(b101, make_float2(tau, tau), p01);
+          const float e0 = e01.x, e1 = e01.y, e2 = __fmaf_rn(b12, tau, p2);
+          const float2 v01 = __ffma2_rn(g01, make_float2(f, f), b101);
+          const float v2 = __fmaf_rn(g2, f, b12);
+          const float eg = dot3(e0, e1, e2, g01.x, g01.y, g2);
+          const float kappa = __fmaf_rn(-f, eg, sq);
+          // 1 - beta^2 = (1 - beta1^2) - f g.(beta1 + beta)
+          const float2 t01 = __fadd2_rn(b101, v01);
+          const float Av = __fmaf_rn(icdt, eg, __fmaf_rn(-f, dot3(g01.x, g01.y, g2, t01.x, t01.y, __fadd_rn(b12, v2)), ig2));
+          if (!(ig2 > 0.f && Dh > 0.f && kappa >= 1.17549435e-38f)) {
+            set_err((ig2 > 0.f && Dh >= 0.f) ? kErrCoincide : kErrDisc);
+            return true;
+          }
+          const float ik = __fdividef(1.f, kappa);
+          const float s3 = __fmul_rn(__fmul_rn(s_kq[jj], ik), ik);  // kq / kappa^2
+          const float s1 = __fmul_rn(__fmul_rn(s3, ik), Av);        // kq A / kappa^3
+          const float s2 = __fmul_rn(s3, icdt);
+          const float2 H01 = __ffma2_rn(make_float2(s1, s1), v01, __fmul2_rn(make_float2(s2, s2), g01));
+          const float H2 = __fmaf_rn(s1, v2, __fmul_rn(s2, g2));
+          float2 q01 = __ffma2_rn(make_float2(-tau, -tau), H01, make_float2(P[0], P[1]));
+          q01 = __ffma2_rn(make_float2(s1, s1), e01, q01);
+          P[0] = q01.x;
+          P[1] = q01.y;
+          P[2] = __fmaf_rn(s1, e2, __fmaf_rn(-tau, H2, P[2]));
+          P[3] = __fmaf_rn(H01.y, e2, __fmaf_rn(-H2, e1, P[3]));
+          P[4] = __fmaf_rn(H2, e0, __fmaf_rn(-H01.x, e2, P[4]));
+          P[5] = __fmaf_rn(H01.x, e1, __fmaf_rn(-H01.y, e0, P[5]));
+          return true;
         };
         // ---- bracket: offset l1 of the older node, its slot pA, record A, separation dA and table -------
         int l1;
@@ -607,29 +718,26 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
               fast = (l1 == 0);
             }
           } else {
-            // predicted bracket [lg, lg + 1]: both records are loaded at once
+            // predicted bracket [lg, lg + 1]; of the newer record mostly the velocity alone is needed
             const int pg1 = pA + 1 == D ? 0 : pA + 1;  // slot of offset lg + 1
-            Rec Bn;
-            if (WIN) {
-              const float4* rb = inw ? ra + 3 : src32 + 3 * pg1;
-              Bn.q0 = rb[0];
-              Bn.q1 = rb[1];
-              Bn.q2 = rb[2];
-            } else {
-              Bn = load_rec(src32, pg1);
-            }
+            const float4* rb = WIN && inw ? ra + 3 : src32 + 3 * pg1;
+            q2b = WIN ? rb[2] : __ldg(rb + 2);
+            have_b = true;
             const bool tA = node_test_d<kShared>(r, dA, tabA, src64, pA, a, n_fb);
             if (!tA) {
-              bool tB = true;  // P(n) is always true
-              if (lg + 1 < win.nw - 1) {
-                n_tests += 1;
-                tB = node_test_d<kShared>(r, separation(r, Bn.q0, Bn.q1), __ldg(a.tab32 + pg1), src64, pg1, a, n_fb);
+              const bool last = lg == win.nw - 2;  // the newer node is the present slot: P(n) is always true
+              if (!last) n_tests += 1;
+              if (!ADAPT && line_fields(A, dA, tabA, q2b, pA, last ? 1 : 2, !last)) {
+                brc += last ? 1u << 10 : 1u << 20;
+                if (DUMP) a.dump[(size_t)i * N + j] = 4 * lg + (last ? 1 : 2);
+                continue;
               }
-              if (tB) {
+              // the bound does not hold: the newer node's test itself, and the records again from the ring (they need
+              // not stay in registers through the bound)
+              if (!ADAPT) fast = have_b = false;
+              if (last || node_test<kShared>(r, src32, src64, pg1, a, n_fb)) {
                 l1 = lg;
-                br = (l1 == win.nw - 2) ? 1 : 2;
-                q2b = Bn.q2;
-                have_b = true;
+                br = last ? 1 : 2;
               } else {
                 // gallop up from lo = lg + 1 (P false)
                 int lo = lg + 1, hi, st = 1;
@@ -646,7 +754,7 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
                 }
                 l1 = bisect<kShared>(r, src32, src64, win, lo, hi, a, n_tests, n_fb);
                 br = (l1 == win.nw - 2) ? 1 : 2;
-                fast = false;
+                fast = have_b = false;
               }
             } else if (lg == 0) {
               l1 = 0;
@@ -673,7 +781,7 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
                 l1 = bisect<kShared>(r, src32, src64, win, lo, hi, a, n_tests, n_fb);
                 br = (l1 == win.nw - 2) ? 1 : 2;
               }
-              fast = false;
+              fast = have_b = false;
             }
           }
         }
@@ -692,88 +800,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), EMPPP_MIXED_MIN_BLOCKS * 1
           continue;
         }
         if (!ADAPT) {
-          // ---- retarded state and fields from the source's line at t_n (light units) ------------------
-          // p is the target's separation from where the line of the older node is at t_n, tau = c (t_n - t_r) = R
-          // the positive root of (1 - beta1^2) tau^2 - 2 (p.beta1) tau - |p|^2 = 0, whose half-discriminant Dh is a
-          // sum of non-negative terms. With f = (t_r - t1) / (t2 - t1), g = beta2 - beta1, eta = p + beta1 tau and
-          // beta = beta1 + f g: kappa = R - eta.beta = sqrt(Dh) - f eta.g, A = 1 - beta^2 + eta.alpha (alpha =
-          // g / (c dt)), H = A beta + kappa alpha, and eq:LW_E, eq:LW_B are E = kq (A eta - tau H) / kappa^3,
-          // c B = kq (H x eta) / kappa^3: no second root, no division by R, no double cross product.
-          // Rounding sequence fixed as below (no packed product feeds a packed sum).
-          const float L1 = tabA.z, icdt = tabA.w;
-          const float ig2 = A.q0.w;
-          const float2 b101 = __fadd2_rn(bref01, make_float2(A.q2.x, A.q2.y));
-          const float b10 = b101.x, b11 = b101.y, b12 = __fadd_rn(bref2, A.q2.z);
-          float2 p01;
-          float p2;
-          if (br == 1) {
-            // near-field shortcut: the end of the last segment, formed per source in FP64 (ext32), since p cancels
-            // when R is far below c (t_n - t_{n-1})
-            const float4* e = a.ext32 + (size_t)j * kExtCount;
-            const float3 dp = separation(r, __ldg(e + kExtSegHi), __ldg(e + kExtSegLo));
-            p01 = make_float2(dp.x, dp.y);
-            p2 = dp.z;
-          } else {
-            // d - beta1 L1 with beta1 = beta_ref + dbeta and L1 in two parts each
-            p01 = __ffma2_rn(make_float2(-bref01.x, -bref01.y), make_float2(L1, L1), make_float2(dA.x, dA.y));
-            p01 = __ffma2_rn(make_float2(-A.q2.x, -A.q2.y), make_float2(L1, L1), p01);
-            p01 = __ffma2_rn(make_float2(-b10, -b11), make_float2(tabA.y, tabA.y), p01);
-            p2 = __fmaf_rn(-b12, tabA.y, __fmaf_rn(-A.q2.z, L1, __fmaf_rn(-bref2, L1, dA.z)));
-          }
-          float pv = dot3(p01.x, p01.y, p2, b10, b11, b12);
-          float pp = dot3(p01.x, p01.y, p2, p01.x, p01.y, p2);
-          float Dh = __fmaf_rn(pp, ig2, __fmul_rn(pv, pv));
-          float sq = __fmul_rn(Dh, rsqrtf(Dh));
-          // The rounding of p (about u L1) moves tau by up to u L1 / (2 sqrt(Dh)) of itself. Where that exceeds 2e-6
-          // (sources moving nearly towards the target at high gamma; below 2 u gamma^2, so never for gamma^2 < 16)
-          // p is formed in FP64 from the FP64 records.
-          if (br == 2 && ig2 < 0.0625f && L1 > __fmul_rn(kLineGuard, sq)) {
-            const double* w64 = src64 + 6 * pA;
-            const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
-            const double T1 = __ldg(a.tab64 + pA).x;
-            p01.x = (float)((__ldg(rr + 0) - __ldg(w64 + 0)) - __ldg(w64 + 3) * T1);
-            p01.y = (float)((__ldg(rr + 1) - __ldg(w64 + 1)) - __ldg(w64 + 4) * T1);
-            p2 = (float)((__ldg(rr + 2) - __ldg(w64 + 2)) - __ldg(w64 + 5) * T1);
-            pv = dot3(p01.x, p01.y, p2, b10, b11, b12);
-            pp = dot3(p01.x, p01.y, p2, p01.x, p01.y, p2);
-            Dh = __fmaf_rn(pp, ig2, __fmul_rn(pv, pv));
-            sq = __fmul_rn(Dh, rsqrtf(Dh));
-            count_fallback<kShared>(n_fb);
-          }
-          const float sum = __fadd_rn(sq, fabsf(pv));
-          const bool pos = pv >= 0.f;
-          const float tau = __fmul_rn(pos ? sum : pp, pos ? A.q2.w : __fdividef(1.f, sum));
-          const float f = __fmul_rn(__fsub_rn(L1, tau), icdt);
           if (!have_b) q2b = __ldg(src32 + 3 * (pA + 1 == D ? 0 : pA + 1) + 2);
-          const float2 g01 = sub2(make_float2(q2b.x, q2b.y), A.q2);
-          const float g2 = __fsub_rn(q2b.z, A.q2.z);
-          const float2 e01 = __ffma2_rn(b101, make_float2(tau, tau), p01);
-          const float e0 = e01.x, e1 = e01.y, e2 = __fmaf_rn(b12, tau, p2);
-          const float2 v01 = __ffma2_rn(g01, make_float2(f, f), b101);
-          const float v2 = __fmaf_rn(g2, f, b12);
-          const float eg = dot3(e0, e1, e2, g01.x, g01.y, g2);
-          const float kappa = __fmaf_rn(-f, eg, sq);
-          // 1 - beta^2 = (1 - beta1^2) - f g.(beta1 + beta)
-          const float2 t01 = __fadd2_rn(b101, v01);
-          const float Av = __fmaf_rn(icdt, eg, __fmaf_rn(-f, dot3(g01.x, g01.y, g2, t01.x, t01.y, __fadd_rn(b12, v2)), ig2));
-          if (!(ig2 > 0.f && Dh > 0.f && kappa >= 1.17549435e-38f)) {
-            set_err((ig2 > 0.f && Dh >= 0.f) ? kErrCoincide : kErrDisc);
-            continue;
-          }
-          const float ik = __fdividef(1.f, kappa);
-          const float s3 = __fmul_rn(__fmul_rn(s_kq[jj], ik), ik);  // kq / kappa^2
-          const float s1 = __fmul_rn(__fmul_rn(s3, ik), Av);        // kq A / kappa^3
-          const float s2 = __fmul_rn(s3, icdt);
-          const float2 H01 = __ffma2_rn(make_float2(s1, s1), v01, __fmul2_rn(make_float2(s2, s2), g01));
-          const float H2 = __fmaf_rn(s1, v2, __fmul_rn(s2, g2));
-          float2 q01 = __ffma2_rn(make_float2(-tau, -tau), H01, make_float2(P[0], P[1]));
-          q01 = __ffma2_rn(make_float2(s1, s1), e01, q01);
-          P[0] = q01.x;
-          P[1] = q01.y;
-          P[2] = __fmaf_rn(s1, e2, __fmaf_rn(-tau, H2, P[2]));
-          P[3] = __fmaf_rn(H01.y, e2, __fmaf_rn(-H2, e1, P[3]));
-          P[4] = __fmaf_rn(H2, e0, __fmaf_rn(-H01.x, e2, P[4]));
-          P[5] = __fmaf_rn(H01.x, e1, __fmaf_rn(-H01.y, e0, P[5]));
+          line_fields(A, dA, tabA, q2b, pA, br, false);
           continue;
         }
         // ---- retarded state (light units) --------------------------------------------------------

@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
     double u[3] = {s.u[3 * i], s.u[3 * i + 1], s.u[3 * i + 2]};
     const double E[3] = {s.Eself[3 * i], s.Eself[3 * i + 1], s.Eself[3 * i + 2]};
     const double Bs[3] = {s.Bself[3 * i], s.Bself[3 * i + 1], s.Bself[3 * i + 2]};
+    const double vn[3] = {rec[3], rec[4], rec[5]}, xn[3] = {rec[0], rec[1], rec[2]};
     double v[3], B[3];
     push_particle(x, u, E, Bs, bp, dt, v, B);
     const double x0 = x[0], x1 = x[1], x2 = x[2], v0 = v[0], v1 = v[1], v2 = v[2];
@@ -196,6 +197,9 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
     o[0] = q[0];
     o[1] = q[1];
     o[2] = q[2];
+    // how far slot n + 1 lies from slot n's line (newer-node bound of the mixed path)
+    s.rec32[((size_t)i * s.D + pfrom) * 12 + 7] =
+        line_deviation(xn[0], xn[1], xn[2], vn[0], vn[1], vn[2], x0, x1, x2, (t_n + dt) - t_n);
   }
   // the last block to finish advances the clock and resets the reduction for the next step (and, with
   // ep.on, evaluates the energy monitor of every bunch on the pushed state)

@@ -56,21 +56,29 @@ __global__ void init_slot0_kernel(DeviceState s, const double* __restrict__ x, c
   s.kq32[i] = (float)(-kQe * s.wts[i] / (4.0 * kPi * kEps0));
 }
 
-__global__ void scatter_slot_kernel(DeviceState s, int p, const double* __restrict__ W, const double* __restrict__ V) {
+// slot p of every particle; dt > 0: the time since the slot before it, whose deviation (shadow.cuh) it completes
+__global__ void scatter_slot_kernel(DeviceState s, int p, double dt, const double* __restrict__ W,
+                                    const double* __restrict__ V) {
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= s.N) return;
+  if (dt > 0.0) {
+    const size_t q = (size_t)j * s.D + (p == 0 ? s.D - 1 : p - 1);
+    const double* r = s.rec64 + q * 6;
+    s.rec32[q * 12 + 7] =
+        line_deviation(r[0], r[1], r[2], r[3], r[4], r[5], W[3 * j], W[3 * j + 1], W[3 * j + 2], dt);
+  }
   write_record(s, j, p, W[3 * j], W[3 * j + 1], W[3 * j + 2], V[3 * j], V[3 * j + 1], V[3 * j + 2]);
 }
 
 // All slots of a history held on the device (W, V [nslots][N][3], the layout of emppp_set_history) in one launch:
-// slot s goes to physical slot (p_first + s) mod D. What bounds it is memory (24 + 24 bytes read and 96 written per
+// slot s goes to physical slot (p_first + s) mod D (last: these end with the present slot). What bounds it is memory (24 + 24 bytes read and 96 written per
 // record) and, close behind, the FP64 operations of the FP32 record. A thread takes kScatterSlots consecutive slots of
 // one particle: the reads of a warp are contiguous over its particles, and the 48-byte records that one thread writes
 // follow one another, so that their sectors fill in L2. N = 8192, 301 slots: 0.22 ms instead of 1.85 ms for one launch
 // per slot.
 constexpr int kScatterSlots = 8;
 
-__global__ void __launch_bounds__(256) scatter_history_kernel(DeviceState s, int p_first, int nslots,
+__global__ void __launch_bounds__(256) scatter_history_kernel(DeviceState s, int p_first, int nslots, int last,
                                                               const double* __restrict__ W,
                                                               const double* __restrict__ V) {
   const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -78,14 +86,27 @@ __global__ void __launch_bounds__(256) scatter_history_kernel(DeviceState s, int
   const int s0 = blockIdx.y * kScatterSlots, s1 = min(nslots, s0 + kScatterSlots);
   int p = p_first + s0;
   if (p >= s.D) p -= s.D;
+  const size_t stride = (size_t)s.N * 3;
+  const double* w = W + (size_t)s0 * stride + 3 * j;
+  const double* v = V + (size_t)s0 * stride + 3 * j;
+  double w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2);
   for (int k = s0; k < s1; k++) {
-    const double* w = W + ((size_t)k * s.N + j) * 3;
-    const double* v = V + ((size_t)k * s.N + j) * 3;
     const double v0 = __ldg(v), v1 = __ldg(v + 1), v2 = __ldg(v + 2);
     // 1 / gamma^2 = 1 - v.v / c^2 and its reciprocal without divisions (both are rounded to FP32)
     const double ig2 = 1.0 - (v0 * v0 + v1 * v1 + v2 * v2) * (1.0 / (kC * kC));
-    write_record(s, j, p, __ldg(w), __ldg(w + 1), __ldg(w + 2), v0, v1, v2, recip_refined(ig2), ig2);
-    p = p + 1 == s.D ? 0 : p + 1;
+    write_record(s, j, p, w0, w1, w2, v0, v1, v2, recip_refined(ig2), ig2);
+    const int pnext = p + 1 == s.D ? 0 : p + 1;
+    w += stride;
+    v += stride;
+    if (!last || k + 1 < nslots) {  // the next slot, which may be another thread's
+      const double x0 = __ldg(w), x1 = __ldg(w + 1), x2 = __ldg(w + 2);
+      s.rec32[((size_t)j * s.D + p) * 12 + 7] =
+          line_deviation(w0, w1, w2, v0, v1, v2, x0, x1, x2, s.slot_t[pnext] - s.slot_t[p]);
+      w0 = x0;
+      w1 = x1;
+      w2 = x2;
+    }
+    p = pnext;
   }
 }
 
@@ -270,8 +291,9 @@ cudaError_t launch_init_slot0(const DeviceState& s, const double* x, const doubl
   return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_slot(const DeviceState& s, int p, const double* W, const double* V, cudaStream_t st) {
-  scatter_slot_kernel<<<blocks_for(s.N, 256), 256, 0, st>>>(s, p, W, V);
+cudaError_t launch_scatter_slot(const DeviceState& s, int p, double dt, const double* W, const double* V,
+                                cudaStream_t st) {
+  scatter_slot_kernel<<<blocks_for(s.N, 256), 256, 0, st>>>(s, p, dt, W, V);
   return cudaGetLastError();
 }
 
@@ -282,7 +304,7 @@ cudaError_t launch_scatter_history(const DeviceState& s, int p_first, int nslots
   for (int k = 0; k < nslots; k += kMost) {
     const int m = nslots - k < kMost ? nslots - k : kMost;
     scatter_history_kernel<<<dim3(blocks_for(s.N, 256), blocks_for(m, kScatterSlots)), 256, 0, st>>>(
-        s, (int)(((long long)p_first + k) % s.D), m, W + (size_t)k * s.N * 3, V + (size_t)k * s.N * 3);
+        s, (int)(((long long)p_first + k) % s.D), m, k + m == nslots, W + (size_t)k * s.N * 3, V + (size_t)k * s.N * 3);
   }
   return cudaGetLastError();
 }

@@ -1,7 +1,9 @@
 // FP32 shadow record of one history slot, used by the mixed-precision pair path and by the FP32
 // delay guess. Three float4 per (particle, slot):
 //   q0 = (hi.x, hi.y, hi.z, 1/gamma^2)   hi = fl32(w - origin)
-//   q1 = (lo.x, lo.y, lo.z, 0)           lo = fl32((w - origin) - hi), so hi + lo carries ~48 bits
+//   q1 = (lo.x, lo.y, lo.z, dev)         lo = fl32((w - origin) - hi), so hi + lo carries ~48 bits; dev: 1.03 times
+//                                        the next slot's distance from this slot's line (kNewerMargin), +inf
+//                                        until that slot is written
 //   q2 = (dbeta.x, dbeta.y, dbeta.z, gamma^2)  dbeta = v/c - beta_ref
 // 1/gamma^2 = 1 - beta^2 is formed in FP64, so the FP32 path never subtracts beta^2 from 1. Velocities
 // are stored relative to a reference velocity beta_ref (the velocity of one particle of the bunch when
@@ -21,7 +23,8 @@ __device__ __forceinline__ void shadow_record(const double origin[3], const doub
   const float h0 = (float)d0, h1 = (float)d1, h2 = (float)d2;
   const double ic = 1.0 / kC;
   q[0] = make_float4(h0, h1, h2, (float)inv_gamma2);
-  q[1] = make_float4((float)(d0 - (double)h0), (float)(d1 - (double)h1), (float)(d2 - (double)h2), 0.f);
+  q[1] = make_float4((float)(d0 - (double)h0), (float)(d1 - (double)h1), (float)(d2 - (double)h2),
+                     __int_as_float(0x7f800000));
   q[2] = make_float4((float)(v0 * ic - beta_ref[0]), (float)(v1 * ic - beta_ref[1]), (float)(v2 * ic - beta_ref[2]),
                      (float)gamma2);
 }
@@ -29,6 +32,17 @@ __device__ __forceinline__ void shadow_record(const double origin[3], const doub
 __device__ __forceinline__ void shadow_record(const double origin[3], const double beta_ref[3], double w0, double w1,
                                               double w2, double v0, double v1, double v2, double gamma2, float4 q[3]) {
   shadow_record(origin, beta_ref, w0, w1, w2, v0, v1, v2, gamma2, 1.0 / gamma2, q);
+}
+
+// dev of a slot at w0 with velocity v0 whose next slot, dt later, is at w1 (rounded up: the FP32 norm is within 4u, and
+// the added 1e-20 m covers squares that underflow)
+__device__ __forceinline__ float line_deviation(double w00, double w01, double w02, double v00, double v01, double v02,
+                                                double w10, double w11, double w12, double dt) {
+  const float d0 = (float)((w10 - w00) - v00 * dt), d1 = (float)((w11 - w01) - v01 * dt),
+              d2 = (float)((w12 - w02) - v02 * dt);
+  const float up = fmaf(sqrtf(d0 * d0 + d1 * d1 + d2 * d2), 1.0302f, 1e-20f);
+  const double c2mv2 = kC * kC - (v00 * v00 + v01 * v01 + v02 * v02);
+  return c2mv2 >= kC * kC / kDevGamma2 ? up : __int_as_float(0x7f800000);
 }
 
 // gamma^2 of a stored velocity: 1 / (1 - v.v / c^2)

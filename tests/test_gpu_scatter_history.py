@@ -1,5 +1,5 @@
 """emppp_set_history from device arrays (one launch over all slots) against the same history from host arrays (a launch
-per slot): the stored history comes back bit for bit, the FP64 fields are equal, and the mixed ones agree within its
+per slot): the stored history comes back bit for bit, every pair's bracket is the oracle's, the FP64 fields are equal, and the mixed ones agree within its
 FP32 records' last place (their 1 / gamma^2 is formed without a division). Slot counts around the launch's groups of
 8 slots, rings that wrap and rings that do not fill, two bunches."""
 import numpy as np
@@ -32,6 +32,8 @@ def test_device_history_equals_host_history(N, n, D, bunches):
                 _, T2, W2, V2, u2 = s.get_history()
                 for a, b in ((T, T2), (W, W2), (V, V2), (u, u2)):
                     assert np.array_equal(a, b)
+                if bunches is None:
+                    assert np.array_equal(s.bracket_dump()[0], oracle.bracket_table(h.T, h.W, h.n, D))
                 s.step(1)
                 out[precision, where] = s.get_fields()
     for a, b in zip(out["fp64", "host"], out["fp64", "device"]):
