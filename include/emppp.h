@@ -288,7 +288,7 @@ EMPPP_API emppp_status emppp_synchronize(emppp_handle h);
  *     nslots - 1 is the present one and every slot is usable (the history depth is nslots).
  *   w [n] optional weights (NULL: 1); E, B [n][3] device outputs (B is the self field only).
  *   cuda_stream: cudaStream_t the work is enqueued on (NULL: legacy default stream); asynchronous.
- * The FP64 path with the paper's search (out-of-history test, shortcut, bisection) is used. Its working
+ * The fields are the FP64 path's (same brackets: the search starts from the uniform-motion guess). Its working
  * memory is one fixed 16 MiB device array inside the library (held by every GPU that loads the
  * library until the process exits), which limits n to 348160 and nslots to 4096: larger sizes are
  * rejected with EMPPP_ERR_ARG. All calls share that array, so calls whose work overlaps on the GPU

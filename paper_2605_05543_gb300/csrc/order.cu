@@ -31,23 +31,47 @@ __host__ __device__ __forceinline__ int cell_bits(int n) {
   return b < 2 ? 2 : (b > kMaxBits ? kMaxBits : b);
 }
 
-__global__ void __launch_bounds__(kThreads) order_kernel(DeviceState s, unsigned* __restrict__ key,
+// where the particles to order stand: the bunch of a block and the FP32 position of its particle k
+struct RingPositions {  // present positions of a solver's bunches (hi parts about their origins)
+  DeviceState s;
+  const float4* rec;
+  int pn;
+  __device__ __forceinline__ void begin() {
+    rec = reinterpret_cast<const float4*>(s.rec32);
+    pn = (int)(s.state->n % s.D);
+  }
+  __device__ __forceinline__ int count() const { return s.bunches[blockIdx.x].n; }
+  __device__ __forceinline__ long long offset() const { return s.bunches[blockIdx.x].off; }
+  // one record per particle's ring run, so every particle is its own cache line
+  __device__ __forceinline__ float4 at(long long k) const { return __ldg(rec + ((size_t)k * s.D + pn) * 3); }
+};
+struct ArrayPositions {  // x [n][3], about the first particle
+  const double* x;
+  int n;
+  __device__ __forceinline__ void begin() {}
+  __device__ __forceinline__ int count() const { return n; }
+  __device__ __forceinline__ long long offset() const { return 0; }
+  __device__ __forceinline__ float4 at(long long k) const {
+    return make_float4((float)(__ldg(x + 3 * k) - __ldg(x)), (float)(__ldg(x + 3 * k + 1) - __ldg(x + 1)),
+                       (float)(__ldg(x + 3 * k + 2) - __ldg(x + 2)), 0.f);
+  }
+};
+
+template <class Positions>
+__global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsigned* __restrict__ key,
                                                          int* __restrict__ order) {
   extern __shared__ int hist[];
   __shared__ float s_lo[3][32], s_hi[3][32];
   __shared__ int s_warp[32];
-  const BunchDesc bd = s.bunches[blockIdx.x];
-  const int n = bd.n;
-  const long long off = bd.off;
+  where.begin();
+  const int n = where.count();
+  const long long off = where.offset();
   const int bits = cell_bits(n);
   const int cells = 1 << (3 * bits);
-  const int pn = (int)(s.state->n % s.D);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
-  // present FP32 position (hi part) of particle k of the bunch: one record per particle's ring run, so
-  // every particle is its own cache line; kUnroll of them are loaded before any is used
-  const float4* __restrict__ rec = reinterpret_cast<const float4*>(s.rec32);
-  auto position = [&](int k) { return __ldg(rec + ((size_t)(off + k) * s.D + pn) * 3); };
+  // position of particle k of the bunch; kUnroll of them are loaded before any is used
+  auto position = [&](int k) { return where.at(off + k); };
   // bounding box of the present FP32 positions
   float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
   for (int k0 = tid; k0 < n; k0 += kUnroll * kThreads) {
@@ -160,13 +184,21 @@ constexpr size_t kSmem = sizeof(int) << (3 * kMaxBits);
 
 // allows the kernel its shared-memory histogram on the current device (call before launching)
 cudaError_t prepare_target_order() {
-  return cudaFuncSetAttribute(order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  cudaError_t e =
+      cudaFuncSetAttribute(order_kernel<RingPositions>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(order_kernel<ArrayPositions>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+}
+
+cudaError_t launch_array_order(const double* x, int n, unsigned* key, int* order, cudaStream_t st) {
+  order_kernel<<<1, kThreads, sizeof(int) << (3 * cell_bits(n)), st>>>(ArrayPositions{x, n}, key, order);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_target_order(const DeviceState& s, unsigned* key, int* order, long long max_bunch, cudaStream_t st) {
   // histogram of the largest bunch's cells only: a small system does not reserve 128 KB of shared memory
   const size_t smem = sizeof(int) << (3 * cell_bits((int)(max_bunch < (1LL << 30) ? max_bunch : (1LL << 30))));
-  order_kernel<<<s.nbunch, kThreads, smem, st>>>(s, key, order);
+  order_kernel<<<s.nbunch, kThreads, smem, st>>>(RingPositions{s, nullptr, 0}, key, order);
   return cudaGetLastError();
 }
 

@@ -25,18 +25,13 @@
 // (the guess, the node tests outside the guard band, indices, loads) runs on the FP32/INT pipes beside it.
 #include "../../include/emppp.h"
 #include "emppp_internal.cuh"
-#include "fp64_roots.cuh"
+#include "fp64_fields.cuh"
 #include "mlp.cuh"
 #include "shadow.cuh"
 
 namespace emppp {
 
 namespace {
-
-constexpr double kCoulomb = 1.0 / (4.0 * kPi * kEps0);
-// the sums run over w_j-weighted fields without the electron's charge constant -e / (4 pi eps0), and over
-// c^2 B; both are scaled once per target
-constexpr double kFieldScale = -kQe * kCoulomb;
 
 struct PairArgs {
   const double* __restrict__ rec64;
@@ -183,7 +178,7 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
     s_f[q >> 2][c] = __ldg(reinterpret_cast<const float4*>(a.rec32) + ((size_t)js * D + slot) * 3 + part);
   }
   __syncthreads();
-  double Ep[3] = {0, 0, 0}, Bp[3] = {0, 0, 0};  // sums over this tile's sources
+  FieldSums sum;  // over this tile's sources
   for (int jj = 0; (PROP == kPropMlp || active) && jj < tn; ++jj) {
     const int j = debug_index(tile + jj, boff, bend, a.err);  // tile + jj itself in a release build
     float fac = 1.f;
@@ -318,19 +313,19 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
     // ---- 2. the source's line at t_n ----------------------------------------------------------
     const double2* se = s_e + jj * (kExt64 / 2);
     const double cw = se[5].x;  // c w_j: the charge constant -e / (4 pi eps0) is applied once per target
-    double X0, X1, X2, v10, v11, v12, C2;
+    Line ln;
     double2 y01, y23, y45, ts;  // newer record, (t_n - t1, 1 / (t2 - t1))
     double w10, w11, w12;       // older position (eq:mid)
     if (br == 0) {
       // out of history (eq:linear2): the line through the oldest slot
       const double2 e0 = se[0], e1 = se[1], e2 = se[2], e3 = se[3], e4 = se[4];
-      X0 = (r0 - e0.x) - e1.y;
-      X1 = (r1 - e0.y) - e2.x;
-      X2 = (r2 - e1.x) - e2.y;
-      v10 = e3.x;
-      v11 = e3.y;
-      v12 = e4.x;
-      C2 = e4.y;
+      ln.X0 = (r0 - e0.x) - e1.y;
+      ln.X1 = (r1 - e0.y) - e2.x;
+      ln.X2 = (r2 - e1.x) - e2.y;
+      ln.v0 = e3.x;
+      ln.v1 = e3.y;
+      ln.v2 = e4.x;
+      ln.C2 = e4.y;
     } else {
       const int p1 = win.phys(l1);
       const int p2 = p1 + 1 == D ? 0 : p1 + 1;
@@ -344,19 +339,19 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
       w10 = x01.x;
       w11 = x01.y;
       w12 = x23.x;
-      v10 = x23.y;
-      v11 = x45.x;
-      v12 = x45.y;
-      X0 = fma(-v10, ts.x, r0 - w10);
-      X1 = fma(-v11, ts.x, r1 - w11);
-      X2 = fma(-v12, ts.x, r2 - w12);
-      C2 = fma(-v10, v10, fma(-v11, v11, fma(-v12, v12, kC * kC)));
+      ln.v0 = x23.y;
+      ln.v1 = x45.x;
+      ln.v2 = x45.y;
+      ln.X0 = fma(-ln.v0, ts.x, r0 - w10);
+      ln.X1 = fma(-ln.v1, ts.x, r1 - w11);
+      ln.X2 = fma(-ln.v2, ts.x, r2 - w12);
+      ln.set_c2();
     }
     if (MID && br != 0) {
       // eq:mid: the midpoint of the bracket stands for the retarded time; eq:LW_E and eq:LW_B as they stand
       const double idt = ts.y;
-      const double v0 = 0.5 * (v10 + y23.y), v1 = 0.5 * (v11 + y45.x), v2 = 0.5 * (v12 + y45.y);
-      const double a0 = (y23.y - v10) * idt, a1 = (y45.x - v11) * idt, a2 = (y45.y - v12) * idt;
+      const double v0 = 0.5 * (ln.v0 + y23.y), v1 = 0.5 * (ln.v1 + y45.x), v2 = 0.5 * (ln.v2 + y45.y);
+      const double a0 = (y23.y - ln.v0) * idt, a1 = (y45.x - ln.v1) * idt, a2 = (y45.y - ln.v2) * idt;
       const double e0 = r0 - 0.5 * (w10 + y01.x), e1 = r1 - 0.5 * (w11 + y01.y), e2 = r2 - 0.5 * (w12 + y23.x);
       const double R2s = e0 * e0 + e1 * e1 + e2 * e2;
       const double invR = rsqrt(R2s);
@@ -375,87 +370,43 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
       const double ievp = recip_refined(evp);
       const double pref = (cw * (1.0 / kC) * R) * (ievp * ievp * ievp);
       const double E0 = pref * (c2mv2 * vp0 + ac0), E1 = pref * (c2mv2 * vp1 + ac1), E2 = pref * (c2mv2 * vp2 + ac2);
-      Ep[0] += E0;
-      Ep[1] += E1;
-      Ep[2] += E2;
-      Bp[0] += (e1 * E2 - e2 * E1) * cinvR;
-      Bp[1] += (e2 * E0 - e0 * E2) * cinvR;
-      Bp[2] += (e0 * E1 - e1 * E0) * cinvR;
+      sum.E[0] += E0;
+      sum.E[1] += E1;
+      sum.E[2] += E2;
+      sum.B[0] += (e1 * E2 - e2 * E1) * cinvR;
+      sum.B[1] += (e2 * E0 - e0 * E2) * cinvR;
+      sum.B[2] += (e0 * E1 - e1 * E0) * cinvR;
       continue;
     }
-    const double XX = fma(X2, X2, fma(X1, X1, X0 * X0));
-    const double Xv = fma(X2, v12, fma(X1, v11, X0 * v10));
-    const double Dh = fma(Xv, Xv, XX * C2);  // c^2 [|X|^2 (1 - beta1^2) + (X.beta1)^2]
-    if (!(positive_normal(C2) && positive_normal(Dh))) {
-      errbits |= (!positive_normal(C2) || (br != 0 && Dh != Dh)) ? kErrDisc : kErrCoincide;
+    const double XX = ln.XX(), Xv = ln.Xv();
+    const double Dh = fma(Xv, Xv, XX * ln.C2);  // c^2 [|X|^2 (1 - beta1^2) + (X.beta1)^2]
+    if (!(positive_normal(ln.C2) && positive_normal(Dh))) {
+      errbits |= (!positive_normal(ln.C2) || (br != 0 && Dh != Dh)) ? kErrDisc : kErrCoincide;
       continue;
     }
+    // ---- 3. fields, and the adaptive step's interaction scale |eta_ij| = c tau, |v_i(t_n) - v_j(t_r)| ------
     const Root root(Dh);
+    Retarded ret{0.0, ln.v0, ln.v1, ln.v2};
     if (br == 0) {
-      // ---- 3a. Heaviside's field of the uniformly moving source --------------------------------
-      const double iD = root.rsqrt();
-      if (ADAPT) {
-        const double sD = root.sqrt() + fabs(Xv);
-        const bool pos = Xv >= 0.0;
-        const double R = kC * ((pos ? sD : XX) * recip_refined(pos ? C2 : sD));  // c (t - t_r); v(t_r) = v1
-        if (R >= a.eta_allow) {
-          emin = fmin(emin, R);
-          const double dv0 = vi0 - v10, dv1 = vi1 - v11, dv2 = vi2 - v12;
-          vmax2 = fmax(vmax2, dv0 * dv0 + dv1 * dv1 + dv2 * dv2);
-        }
-      }
-      const double pref = se[5].y * ((iD * iD) * iD);  // c w (c^2 - v1^2) / Dh^{3/2}
-      const double E0 = pref * X0, E1 = pref * X1, E2 = pref * X2;
-      Ep[0] += E0;
-      Ep[1] += E1;
-      Ep[2] += E2;
-      // c^2 B = v x E (the 1 / c^2 is applied once per target)
-      Bp[0] = fma(v11, E2, fma(-v12, E1, Bp[0]));
-      Bp[1] = fma(v12, E0, fma(-v10, E2, Bp[1]));
-      Bp[2] = fma(v10, E1, fma(-v11, E0, Bp[2]));
-      continue;
-    }
-    // ---- 3b. retarded state (eq:dt, eq:linear) and Lienard-Wiechert fields ----------------------
-    const double sq = root.sqrt();
-    const double sum = sq + fabs(Xv);
-    const bool pos = __double2hiint(Xv) >= 0;
-    const double tau = (pos ? sum : XX) * recip_refined(pos ? C2 : sum);  // t_n - t_r
-    const double f = (ts.x - tau) * ts.y;                                 // (t_r - t1) / (t2 - t1)
-    const double g0 = y23.y - v10, g1 = y45.x - v11, g2 = y45.y - v12;    // v2 - v1
-    const double e0 = fma(v10, tau, X0), e1 = fma(v11, tau, X1), e2 = fma(v12, tau, X2);  // eta
-    const double v0 = fma(f, g0, v10), v1 = fma(f, g1, v11), v2 = fma(f, g2, v12);
-    const double eg = fma(e2, g2, fma(e1, g1, e0 * g0));
-    const double kappa = fma(-f, eg, sq);
-    if (!positive_normal(kappa)) {
+      if (ADAPT) ret.tau = line_delay(ln, XX, Xv, root.sqrt());
+      heaviside_fields(ln, se[5].y, root, sum);
+    } else if (!bracket_fields(ln, XX, Xv, root, ts.x, ts.y, y23.y, y45.x, y45.y, cw, sum, ret)) {
       errbits |= kErrCoincide;
       continue;
     }
     if (ADAPT) {
-      // interaction scale of the adaptive step: |eta_ij| = c tau and |v_i(t_n) - v_j(t_r)|
-      const double R = kC * tau;
+      const double R = kC * ret.tau;
       if (R >= a.eta_allow) {
         emin = fmin(emin, R);
-        const double dv0 = vi0 - v0, dv1 = vi1 - v1, dv2 = vi2 - v2;
+        const double dv0 = vi0 - ret.v0, dv1 = vi1 - ret.v1, dv2 = vi2 - ret.v2;
         vmax2 = fmax(vmax2, dv0 * dv0 + dv1 * dv1 + dv2 * dv2);
       }
     }
-    const double c2mv2 = fma(-v0, v0, fma(-v1, v1, fma(-v2, v2, kC * kC)));
-    const double ik = recip_refined(kappa);
-    const double s3 = cw * (ik * ik);                       // c w / kappa^2
-    const double s1 = (s3 * ik) * fma(ts.y, eg, c2mv2);     // c w A / kappa^3
-    const double s2 = s3 * ts.y;
-    const double H0 = fma(s1, v0, s2 * g0), H1 = fma(s1, v1, s2 * g1), H2 = fma(s1, v2, s2 * g2);
-    Ep[0] = fma(s1, e0, fma(-tau, H0, Ep[0]));
-    Ep[1] = fma(s1, e1, fma(-tau, H1, Ep[1]));
-    Ep[2] = fma(s1, e2, fma(-tau, H2, Ep[2]));
-    Bp[0] = fma(H1, e2, fma(-H2, e1, Bp[0]));
-    Bp[1] = fma(H2, e0, fma(-H0, e2, Bp[1]));
-    Bp[2] = fma(H0, e1, fma(-H1, e0, Bp[2]));
   }  // sources of the tile
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    s_acc[c][threadIdx.x] += Ep[c];
-    s_acc[3 + c][threadIdx.x] += Bp[c];
+    s_acc[c][threadIdx.x] += sum.E[c];
+    s_acc[3 + c][threadIdx.x] += sum.B[c];
   }
   }  // tiles
   if (active) {
