@@ -1342,12 +1342,13 @@ EMPPP_API emppp_status emppp_mlp_gradient(const float* params, const float* feat
                                           int64_t m, float* grad, double* loss, void* cuda_stream) {
   if (!params || !features || !targets || !grad || m < 1) return fail(EMPPP_ERR_ARG, "bad arguments");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  DevBuf img, dl;
-  if (!img.alloc(mlp_image_bytes()) || !dl.alloc(sizeof(float))) return fail(EMPPP_ERR_OOM, "network buffers");
-  CU(launch_build_image(params, img.p, s));
-  CU(cudaMemsetAsync(grad, 0, sizeof(float) * EMPPP_MLP_NUM_PARAMS, s));
+  const int sms = device_sms();
+  DevBuf buf, dl;
+  if (!buf.alloc(train_buffer_bytes(m, sms)) || !dl.alloc(sizeof(float))) return fail(EMPPP_ERR_OOM, "network buffers");
+  CU(launch_train_image(params, buf.p, s));
   CU(cudaMemsetAsync(dl.p, 0, sizeof(float), s));
-  CU(launch_mlp_train_pass(img.p, features, targets, 0, m, (float)m, grad, static_cast<float*>(dl.p), device_sms(), s));
+  CU(launch_train_pass(buf.p, params, features, targets, 0, m, (float)m, static_cast<float*>(dl.p), sms, false, s));
+  CU(launch_gradient(buf.p, m, sms, grad, s));
   float hl = 0.f;
   CU(cudaMemcpyAsync(&hl, dl.p, sizeof(float), cudaMemcpyDeviceToHost, s));
   CU(cudaStreamSynchronize(s));
@@ -1360,34 +1361,35 @@ EMPPP_API emppp_status emppp_mlp_train(float* params, const float* features, con
   if (!params || !features || !targets || !cfg || m < 1) return fail(EMPPP_ERR_ARG, "bad arguments");
   if (cfg->epochs < 0 || cfg->batch < 16 || !(cfg->lr > 0.f)) return fail(EMPPP_ERR_ARG, "bad training config");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  DevBuf img, grad, m1, m2, dl;
-  const size_t P = sizeof(float) * EMPPP_MLP_NUM_PARAMS;
-  if (!img.alloc(mlp_image_bytes()) || !grad.alloc(P) || !m1.alloc(P) || !m2.alloc(P) || !dl.alloc(sizeof(float)))
-    return fail(EMPPP_ERR_OOM, "training buffers");
-  CU(cudaMemsetAsync(m1.p, 0, P, s));
-  CU(cudaMemsetAsync(m2.p, 0, P, s));
   const int sms = device_sms();
+  // one buffer: operands and partial gradients, Adam's moments, the epoch's loss
+  const size_t P = sizeof(float) * EMPPP_MLP_NUM_PARAMS;
+  const size_t work = (train_buffer_bytes(cfg->batch < m ? cfg->batch : m, sms) + 255) / 256 * 256;
+  DevBuf buf;
+  if (!buf.alloc(work + 2 * P + sizeof(float))) return fail(EMPPP_ERR_OOM, "training buffers");
+  float* m1 = reinterpret_cast<float*>(static_cast<char*>(buf.p) + work);
+  float* m2 = m1 + EMPPP_MLP_NUM_PARAMS;
+  float* dl = m2 + EMPPP_MLP_NUM_PARAMS;
+  CU(cudaMemsetAsync(m1, 0, 2 * P, s));
+  CU(launch_train_image(params, buf.p, s));
   int step = 0;
   const long long batches = (m + cfg->batch - 1) / cfg->batch;
   const long long total = batches * cfg->epochs;
   const bool decay = cfg->lr_final > 0.f && cfg->lr_final < cfg->lr && total > 1;
   for (int ep = 0; ep < cfg->epochs; ep++) {
-    CU(cudaMemsetAsync(dl.p, 0, sizeof(float), s));
+    CU(cudaMemsetAsync(dl, 0, sizeof(float), s));
     for (int64_t r0 = 0; r0 < m; r0 += cfg->batch) {
       const int64_t rows = (m - r0 < cfg->batch) ? m - r0 : cfg->batch;
-      CU(launch_build_image(params, img.p, s));
-      CU(cudaMemsetAsync(grad.p, 0, P, s));
-      CU(launch_mlp_train_pass(img.p, features, targets, r0, rows, (float)rows, static_cast<float*>(grad.p),
-                               static_cast<float*>(dl.p), sms, s));
+      // every pass but an epoch's first follows an Adam step, whose end it may overlap
+      CU(launch_train_pass(buf.p, params, features, targets, r0, rows, (float)rows, dl, sms, r0 > 0, s));
       // cosine schedule from lr (first step) to lr_final (last step)
       const double frac = decay ? (double)step / (double)(total - 1) : 0.0;
       const float lr = decay ? (float)(cfg->lr_final + 0.5 * (cfg->lr - cfg->lr_final) * (1.0 + cos(3.14159265358979323846 * frac)))
                              : cfg->lr;
-      CU(launch_adam(params, static_cast<float*>(grad.p), static_cast<float*>(m1.p), static_cast<float*>(m2.p), lr,
-                     cfg->beta1, cfg->beta2, cfg->eps, ++step, s));
+      CU(launch_adam(params, buf.p, rows, sms, m1, m2, lr, cfg->beta1, cfg->beta2, cfg->eps, ++step, s));
     }
     float hl = 0.f;
-    CU(cudaMemcpyAsync(&hl, dl.p, sizeof(float), cudaMemcpyDeviceToHost, s));
+    CU(cudaMemcpyAsync(&hl, dl, sizeof(float), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
     if (loss_per_epoch) loss_per_epoch[ep] = hl / (float)m;
   }

@@ -347,10 +347,16 @@ cudaError_t launch_sample(const DeviceState& s, const int* pairs, long long m, f
 cudaError_t launch_mlp_forward(const void* image, const float* X, long long m, float* z, int mode, cudaStream_t st);
 // delay factors of the learned proposal (mixed path) for the present state, targets in `order` (or index order)
 cudaError_t launch_mlp_factors(const DeviceState& s, const int* order, cudaStream_t st);
-cudaError_t launch_mlp_train_pass(const void* image, const float* X, const float* T, long long row0, long long rows,
-                                  float norm, float* grad, float* loss, int num_sms, cudaStream_t st);
-cudaError_t launch_adam(float* p, const float* grad, float* m1, float* m2, float lr, float b1, float b2, float eps,
-                        int step, cudaStream_t st);
+// mlp_train.cu: num_sms bounds the blocks of a pass, and with them the partial gradients of the buffer
+size_t train_buffer_bytes(long long batch_rows, int num_sms);
+cudaError_t launch_train_image(const float* params, void* buffer, cudaStream_t st);
+// overlap: the launch may start while the one before it in the stream drains
+cudaError_t launch_train_pass(void* buffer, const float* params, const float* X, const float* T, long long row0,
+                              long long rows, float norm, float* loss, int num_sms, bool overlap, cudaStream_t st);
+// Adam step on the sum of the pass's gradients, after launch_train_pass of as many rows
+cudaError_t launch_adam(float* p, void* buffer, long long rows, int num_sms, float* m1, float* m2, float lr, float b1,
+                        float b2, float eps, int step, cudaStream_t st);
+cudaError_t launch_gradient(const void* buffer, long long rows, int num_sms, float* grad, cudaStream_t st);
 // energy.cu
 cudaError_t launch_energy(const DeviceState& s, const EnergyParams& ep, EnergyMon* mon, bool reset, cudaStream_t st);
 constexpr int kEnergyThreads = 256;  // block size of the energy monitor (and of the post-pair launch)

@@ -48,11 +48,9 @@ constexpr int kNumParams = kOffB3 + 1;  // 4929
 // Network image for the tensor-core passes (BF16 pairs packed in uint32, k contiguous per column):
 //   w1f[n][k/2]: layer-1 weights as the B operand (n = hidden unit, k = feature)
 //   w2f[n][k/2]: layer-2 weights as the B operand (n = output unit, k = input unit)
-//   w2b[n][k/2]: layer-2 weights transposed, the B operand of the input-gradient pass
 struct __align__(16) NetImage {  // copied with 16-byte vector loads and stores
   uint32_t w1f[kH][kInPad / 2];
   uint32_t w2f[kH][kH / 2];
-  uint32_t w2b[kH][kH / 2];
   float b1[kH], b2[kH], w3[kH];
   float b3;
   float pad_[3];
