@@ -1,6 +1,5 @@
 // Per-particle arithmetic of the Higuera-Cary push (Sec. 2.3, Ripperda form) and of the background
-// field (Sec. 2.6), shared by the stage-1 push and the stage-2 transport kernels so that both advance a
-// particle with the same operations.
+// field (Sec. 2.6) of the stage-1 push; the stage-2 transport (stage2.cu) has the same kick reduced to E = 0.
 #pragma once
 
 #include "emppp_internal.cuh"
@@ -27,14 +26,11 @@ __device__ __forceinline__ void background_b(const BextParams& b, double x0, dou
   }
 }
 
-// One Higuera-Cary update of the proper velocity u with fields E, B and h = q dt / (2 m). With
-// HAS_E = false the electric half-kicks are left out: for E = 0 they add a zero, so the values are the
-// same.
-template <bool HAS_E = true>
+// One Higuera-Cary update of the proper velocity u with fields E, B and h = q dt / (2 m).
 __device__ __forceinline__ void hc_kick(double u[3], const double E[3], const double B[3], double h) {
-  const double um0 = HAS_E ? u[0] + h * E[0] : u[0];
-  const double um1 = HAS_E ? u[1] + h * E[1] : u[1];
-  const double um2 = HAS_E ? u[2] + h * E[2] : u[2];
+  const double um0 = u[0] + h * E[0];
+  const double um1 = u[1] + h * E[1];
+  const double um2 = u[2] + h * E[2];
   const double ic2 = 1.0 / (kC * kC);
   const double gm2 = 1.0 + (um0 * um0 + um1 * um1 + um2 * um2) * ic2;
   const double ta0 = h * B[0], ta1 = h * B[1], ta2 = h * B[2];
@@ -49,20 +45,13 @@ __device__ __forceinline__ void hc_kick(double u[3], const double E[3], const do
   const double up0 = s * (um0 + umt * t0 + (um1 * t2 - um2 * t1));
   const double up1 = s * (um1 + umt * t1 + (um2 * t0 - um0 * t2));
   const double up2 = s * (um2 + umt * t2 + (um0 * t1 - um1 * t0));
-  if (HAS_E) {
-    u[0] = up0 + h * E[0] + (up1 * t2 - up2 * t1);
-    u[1] = up1 + h * E[1] + (up2 * t0 - up0 * t2);
-    u[2] = up2 + h * E[2] + (up0 * t1 - up1 * t0);
-  } else {
-    u[0] = up0 + (up1 * t2 - up2 * t1);
-    u[1] = up1 + (up2 * t0 - up0 * t2);
-    u[2] = up2 + (up0 * t1 - up1 * t0);
-  }
+  u[0] = up0 + h * E[0] + (up1 * t2 - up2 * t1);
+  u[1] = up1 + h * E[1] + (up2 * t0 - up0 * t2);
+  u[2] = up2 + h * E[2] + (up0 * t1 - up1 * t0);
 }
 
 // One full push of a particle (x, u): half drift, kick with E and B_self + B_ext(x^{n+1/2}), half drift.
-// Returns the new velocity in v and the total B used in Btot. HAS_E = false: E = 0 (stage 2).
-template <bool HAS_E = true>
+// Returns the new velocity in v and the total B used in Btot.
 __device__ __forceinline__ void push_particle(double x[3], double u[3], const double E[3], const double Bself[3],
                                               const BextParams& bp, double dt, double v[3], double Btot[3]) {
   // 1 / gamma = 1 / sqrt(1 + u.u / c^2), then v = u / gamma as three products (FP64 throughout; each
@@ -75,7 +64,7 @@ __device__ __forceinline__ void push_particle(double x[3], double u[3], const do
   background_b(bp, xh0, xh1, xh2, Bg);
   for (int c = 0; c < 3; c++) Btot[c] = Bself[c] + Bg[c];
   const double h = -kQe * dt / (2.0 * kMe);
-  hc_kick<HAS_E>(u, E, Btot, h);
+  hc_kick(u, E, Btot, h);
   const double ig1 = rsqrt(1.0 + (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) * ic2);
   v[0] = u[0] * ig1;
   v[1] = u[1] * ig1;
