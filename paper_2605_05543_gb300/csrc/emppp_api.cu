@@ -288,15 +288,6 @@ bool any_chunked(const emppp_ctx* c) {
   return false;
 }
 
-// the post-pair launch reads the per-chunk partial sums with a warp per particle when a small system is
-// split into many chunks (a thread per particle would read them one after another)
-bool wide_reduction(const emppp_ctx* c) {
-  if (c->N > 16384) return false;
-  for (int b = 0; b < c->nbunch; b++)
-    if (c->hs[b].nchunk >= 8) return true;
-  return false;
-}
-
 emppp_status read_err(emppp_handle h) {
   int herr = 0;
   CU(cudaMemcpyAsync(&herr, h->ds.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -458,8 +449,7 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
   // launch evaluates the bunches in parallel, one block each)
   const bool fused_energy = h->energy.on && h->N <= 16384 && h->nbunch <= 8;
   NvtxRange r_post("emppp:push_append");
-  CU(launch_step_post(h->ds, bp, h->adapt, chunked, half, chunked && wide_reduction(h),
-                      fused_energy ? &h->energy : nullptr, h->d_mon, h->stream));
+  CU(launch_step_post(h->ds, bp, h->adapt, chunked, half, fused_energy ? &h->energy : nullptr, h->d_mon, h->stream));
   k += 1;
   if (h->energy.on && !fused_energy) {
     // mean energy of the new state and the switch criterion (Sec. 2.7)

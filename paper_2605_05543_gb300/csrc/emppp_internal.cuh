@@ -323,11 +323,11 @@ int max_blocks_pair_fp64(int proposal, int variant, int shape);
 // 4 (k1 - k0) + branch (emppp_bracket_dump)
 cudaError_t launch_pair_fp64(const DeviceState& s, const int* order, int proposal, int reconstruction,
                              const AdaptParams& ap, const PairLaunch& pl, cudaStream_t st, int* dump = nullptr);
-cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_zero_self(const DeviceState& s, cudaStream_t st);
 // push.cu
 cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked,
-                             bool half, bool wide, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st);
+                             bool half, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st);
+cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_half_slot(const DeviceState& s, cudaStream_t st);
 // stage2.cu
 cudaError_t launch_bunch_sums(const DeviceState& s, cudaStream_t st);

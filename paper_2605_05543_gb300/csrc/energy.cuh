@@ -21,8 +21,8 @@ __device__ __forceinline__ double kinetic_term(double u0, double u1, double u2, 
 // kinetic_term values when already formed (by the pushing threads of the same launch), else nullptr.
 // Reads of the particles go to L2 (__ldcg): they were written by other blocks of the same launch.
 __device__ __forceinline__ void energy_block(const DeviceState& s, const EnergyParams& ep, EnergyMon* __restrict__ mon,
-                                             int reset, int b, long long n, double t, const double* terms,
-                                             double* s_num, double* s_den) {
+                                             int reset, int b, long long n, double t, const double* terms) {
+  __shared__ double s_sum[2][kEnergyThreads];
   const BunchDesc& bd = s.bunches[b];
   double num = 0.0, den = 0.0;
   for (long long i = bd.off + threadIdx.x; i < bd.off + bd.n; i += kEnergyThreads) {
@@ -34,18 +34,24 @@ __device__ __forceinline__ void energy_block(const DeviceState& s, const EnergyP
     }
     den += w;
   }
-  s_num[threadIdx.x] = num;
-  s_den[threadIdx.x] = den;
+  // fixed tree, halving the distance: across the warps (by the first two warps, one sum each), then over their lanes
+  s_sum[0][threadIdx.x] = num;
+  s_sum[1][threadIdx.x] = den;
   __syncthreads();
-  for (int h = kEnergyThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-      s_num[threadIdx.x] += s_num[threadIdx.x + h];
-      s_den[threadIdx.x] += s_den[threadIdx.x + h];
-    }
-    __syncthreads();
+  if (threadIdx.x < 64) {
+    const int l = threadIdx.x & 31;
+    const double* v = s_sum[threadIdx.x >> 5];
+    static_assert(kEnergyThreads == 256, "the tree below adds eight warps");
+    double t = ((v[l] + v[l + 128]) + (v[l + 64] + v[l + 192])) + ((v[l + 32] + v[l + 160]) + (v[l + 96] + v[l + 224]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+    if (l == 0) s_sum[threadIdx.x >> 5][0] = t;
   }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const double ebar = s_num[0] / s_den[0] * (kMe * kC * kC);
+    num = s_sum[0][0];
+    den = s_sum[1][0];
+    const double ebar = num / den * (kMe * kC * kC);
     EnergyMon m = mon[b];
     if (reset) {
       m.ebar = ebar;

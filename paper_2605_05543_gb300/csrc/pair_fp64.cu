@@ -453,26 +453,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
   }
 }
 
-// E_i = sum over the source chunks c of partial[c][i] (fixed order), for bunches split in chunks
-__global__ void reduce_partials_kernel(const double* __restrict__ part, const BunchSched* __restrict__ sched,
-                                       const int* __restrict__ bunch_of, long long N, double* __restrict__ E,
-                                       double* __restrict__ B) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const int S = sched[bunch_of[i]].nchunk;
-  if (S == 1) return;  // written directly by the pair kernel
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int c = 0; c < S; c++) {
-    const double* o = part + ((size_t)c * N + i) * 6;
-#pragma unroll
-    for (int k = 0; k < 6; k++) acc[k] += o[k];
-  }
-  for (int c = 0; c < 3; c++) {
-    E[3 * i + c] = acc[c];
-    B[3 * i + c] = acc[3 + c];
-  }
-}
-
 __global__ void zero_kernel(double* __restrict__ a, double* __restrict__ b, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
@@ -556,12 +536,6 @@ cudaError_t launch_pair_fp64(const DeviceState& s, const int* order, int proposa
     launch_fp64<false, false, false, 2>(proposal, pl, a, st);
   else
     launch_fp64<false, false, false, 0>(proposal, pl, a, st);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st) {
-  reduce_partials_kernel<<<(unsigned)((s.N + 255) / 256), 256, 0, st>>>(s.partial, s.sched, s.bunch_of, s.N, s.Eself,
-                                                                          s.Bself);
   return cudaGetLastError();
 }
 

@@ -83,99 +83,173 @@ __global__ void half_slot_kernel(DeviceState s) {
   }
 }
 
+// ---- the sum of each target's per-chunk partial fields ----------------------------------------------------
+// A block of kEnergyThreads threads takes P particles. The chunks fall in eight classes (c mod 8); kSumThreads threads
+// each own one 16-byte word of a particle's six sums and some of the classes, so that the reads of neighbouring
+// threads follow one another and a thread has several in flight; the classes are then added in order. The result is
+// the same whatever P, so a bunch's sums do not depend on what else the solver holds.
+// What bounds it: memory for large systems, one round of L2 latency for small ones. (A thread per particle, which read
+// its chunks one after another, and a warp per particle, whose lanes read 48 bytes N * 48 apart, took 95 us at
+// N = 65536 and 82 us at 16381, with the push; a step of the paper's 400 macroparticles went from 53 to 47 us.)
+constexpr int kClasses = 8;
+constexpr int kSumThreads = 192;
+
+template <int P>
+struct ChunkSums {
+  static constexpr int kWords = 3 * P;                         // 16-byte words of the block's sums
+  static constexpr int kGroups = kSumThreads / kWords;         // threads that share a word
+  static constexpr int kPerThread = kClasses / kGroups;        // classes of a thread
+  static_assert(kGroups * kWords == kSumThreads && kPerThread * kGroups == kClasses, "words and classes divide the threads");
+  double2 part[kClasses][kWords];
+  double2 sum[kWords];
+  int chunks[P];  // chunks of the particle's bunch; at most 1: the pair kernel wrote its fields itself
+
+  // fills sum, and the solver's Eself and Bself, for particles i0 .. i0 + P - 1 (whole block; ends with a barrier)
+  __device__ __forceinline__ void run(const DeviceState& s, long long i0) {
+    if (threadIdx.x < P) {
+      const long long i = i0 + threadIdx.x;
+      chunks[threadIdx.x] = i < s.N ? s.sched[s.bunch_of[i]].nchunk : 0;
+    }
+    __syncthreads();
+    if (threadIdx.x < kSumThreads) {
+      const int w = threadIdx.x % kWords, g = threadIdx.x / kWords;
+      const int S = chunks[w / 3];
+      const size_t stride = (size_t)s.N * 3;
+      const double2* src = reinterpret_cast<const double2*>(s.partial) + i0 * 3 + w;
+      double2 acc[kPerThread];
+#pragma unroll
+      for (int k = 0; k < kPerThread; k++) acc[k] = make_double2(0.0, 0.0);
+      if (S > 1) {
+#pragma unroll 4
+        for (int c0 = g * kPerThread; c0 < S; c0 += kClasses) {
+#pragma unroll
+          for (int k = 0; k < kPerThread; k++) {
+            if (c0 + k < S) {
+              const double2 v = __ldcg(src + (size_t)(c0 + k) * stride);
+              acc[k].x += v.x;
+              acc[k].y += v.y;
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < kPerThread; k++) part[g * kPerThread + k][w] = acc[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < kWords) {
+      const int w = threadIdx.x;
+      if (chunks[w / 3] > 1) {
+        double2 t = part[0][w];
+#pragma unroll
+        for (int k = 1; k < kClasses; k++) {
+          t.x += part[k][w].x;
+          t.y += part[k][w].y;
+        }
+        sum[w] = t;
+        // words: (E0, E1), (E2, B0), (B1, B2)
+        const long long i = i0 + w / 3;
+        const int c = w % 3;
+        if (c == 0) {
+          s.Eself[3 * i] = t.x;
+          s.Eself[3 * i + 1] = t.y;
+        } else if (c == 1) {
+          s.Eself[3 * i + 2] = t.x;
+          s.Bself[3 * i] = t.y;
+        } else {
+          s.Bself[3 * i + 1] = t.x;
+          s.Bself[3 * i + 2] = t.y;
+        }
+      }
+    }
+    __syncthreads();
+  }
+};
+
+// particles per block: few for small systems, whose push then spreads over more SMs (an FP64 warp instruction holds an
+// SM's FP64 pipe for 16 cycles however few of its lanes are active), a full warp of pushers for large ones
+int post_particles(long long n) { return n <= 2432 ? 8 : (n <= 4864 ? 16 : 32); }
+
+template <int P>
+__global__ void __launch_bounds__(kEnergyThreads) reduce_partials_kernel(DeviceState s) {
+  __shared__ ChunkSums<P> sums;
+  sums.run(s, (long long)blockIdx.x * P);
+}
+
+cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st) {
+  const int p = post_particles(s.N);
+  const unsigned blocks = (unsigned)((s.N + p - 1) / p);
+  if (p == 8)
+    reduce_partials_kernel<8><<<blocks, kEnergyThreads, 0, st>>>(s);
+  else if (p == 16)
+    reduce_partials_kernel<16><<<blocks, kEnergyThreads, 0, st>>>(s);
+  else
+    reduce_partials_kernel<32><<<blocks, kEnergyThreads, 0, st>>>(s);
+  return cudaGetLastError();
+}
+
 // The rest of a step after the pair kernel, in one launch: the sum of each target's per-chunk partial
-// fields (fixed chunk order), the adaptive step size, the push of every particle and the append of slot
+// fields, the adaptive step size, the push of every particle and the append of slot
 // n+1, then (by the last block to finish) the clock advance n -> n+1, t -> t + dt and the reset of the
 // interaction-scale reduction. The last block is found with a counter that every block increments once
 // after its work; nothing waits on it. With half = 1 (half-step field point) the clock already stands at
 // the provisional slot n+1: the push starts from slot n, the provisional slot is overwritten and the
 // clock moves from t_n + dt/2 to t_n + dt (formed from t_n, as without the variant).
+template <int P>
 __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s, BextParams bp, AdaptParams ap,
-                                                                   int chunked, int half, int wide, EnergyParams ep,
+                                                                   int chunked, int half, EnergyParams ep,
                                                                    EnergyMon* __restrict__ mon) {
-  // wide = 1: one warp per particle, whose lanes read the per-chunk partial sums in parallel (small
-  // systems, where a bunch is split into many short chunks); else one thread per particle
-  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long i = wide ? (g >> 5) : g;
-  const int lane = threadIdx.x & 31;
-  const bool owner = !wide || lane == 0;
+  __shared__ ChunkSums<P> sums;
+  __shared__ double s_step[3];
+  const long long i0 = (long long)blockIdx.x * P;
   const StepState st = *s.state;
-  double dt = st.dt, eta_rep = 0.0, v_rep = 0.0;
-  if (ap.on) {
-    // the step size, once per block (FP64 root and division) and shared
-    __shared__ double s_step[3];
-    if (threadIdx.x == 0) {
-      s_step[0] = adaptive_step(s, ap, s_step[1], s_step[2]);
-    }
-    __syncthreads();
-    dt = s_step[0];
-    eta_rep = s_step[1];
-    v_rep = s_step[2];
-  }
   // slot of x^n, the slot the push writes and t_n
   const int pfrom = half ? (st.pn == 0 ? s.D - 1 : st.pn - 1) : st.pn;
   const int pnext = half ? st.pn : (st.pn + 1 == s.D ? 0 : st.pn + 1);
   const double t_n = half ? s.slot_t[pfrom] : st.t;
-  if (g == 0) {
+  // the adaptive step size (FP64 root and division), by a warp that sums no chunks
+  if (ap.on && threadIdx.x == kSumThreads) s_step[0] = adaptive_step(s, ap, s_step[1], s_step[2]);
+  // the particle this thread pushes, its state loaded before the sums are there
+  const long long i = i0 + threadIdx.x;
+  const bool pusher = threadIdx.x < P && i < s.N;
+  double x[3], u[3], vn[3];
+  if (pusher) {
+    const double* rec = s.rec64 + ((size_t)i * s.D + pfrom) * 6;
+    for (int c = 0; c < 3; c++) {
+      x[c] = rec[c];
+      vn[c] = rec[3 + c];
+      u[c] = s.u[3 * i + c];
+    }
+  }
+  if (chunked)
+    sums.run(s, i0);
+  else if (ap.on)
+    __syncthreads();  // s_step
+  const double dt = ap.on ? s_step[0] : st.dt;
+  if (i == 0) {
     s.slot_t[pnext] = t_n + dt;
     if (ap.on) {
       s.adapt_info[0] = dt;
-      s.adapt_info[1] = eta_rep;
-      s.adapt_info[2] = v_rep;
+      s.adapt_info[1] = s_step[1];
+      s.adapt_info[2] = s_step[2];
     }
-  }
-  if (i < s.N) {
-    if (chunked) {
-      // E_i = sum over the source chunks c of partial[c][i], in a fixed order
-      const int S = s.sched[s.bunch_of[i]].nchunk;
-      if (S > 1) {
-        double acc[6] = {0, 0, 0, 0, 0, 0};
-        if (wide) {
-          // lane l adds chunks l, l + 32, ... in order; then a butterfly over the lanes, which leaves the
-          // same sum in every lane (each step adds two equal-order partial sums, a commutative operation)
-          for (int c = lane; c < S; c += 32) {
-            const double* o = s.partial + ((size_t)c * s.N + i) * 6;
-#pragma unroll
-            for (int k = 0; k < 6; k++) acc[k] += o[k];
-          }
-#pragma unroll
-          for (int m = 16; m >= 1; m >>= 1) {
-#pragma unroll
-            for (int k = 0; k < 6; k++) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], m);
-          }
-        } else {
-          for (int c = 0; c < S; c++) {
-            const double* o = s.partial + ((size_t)c * s.N + i) * 6;
-#pragma unroll
-            for (int k = 0; k < 6; k++) acc[k] += o[k];
-          }
-        }
-        if (owner) {
-          for (int c = 0; c < 3; c++) {
-            s.Eself[3 * i + c] = acc[c];
-            s.Bself[3 * i + c] = acc[3 + c];
-          }
-        }
-      }
-    }
-  }
-  // the particle this thread pushes: its own, or (wide) one of the block's particles by the lanes of the
-  // first warp, so that the FP64 push occupies one warp per block rather than one lane of each warp
-  long long ip = i;
-  bool pusher = i < s.N && owner;
-  if (wide) {
-    __syncthreads();  // the block's field sums are written
-    ip = (long long)blockIdx.x * (blockDim.x >> 5) + threadIdx.x;
-    pusher = threadIdx.x < (blockDim.x >> 5) && ip < s.N;
   }
   if (pusher) {
-    const long long i = ip;
-    const double* rec = s.rec64 + ((size_t)i * s.D + pfrom) * 6;
-    double x[3] = {rec[0], rec[1], rec[2]};
-    double u[3] = {s.u[3 * i], s.u[3 * i + 1], s.u[3 * i + 2]};
-    const double E[3] = {s.Eself[3 * i], s.Eself[3 * i + 1], s.Eself[3 * i + 2]};
-    const double Bs[3] = {s.Bself[3 * i], s.Bself[3 * i + 1], s.Bself[3 * i + 2]};
-    const double vn[3] = {rec[3], rec[4], rec[5]}, xn[3] = {rec[0], rec[1], rec[2]};
+    double E[3], Bs[3];
+    if (chunked && sums.chunks[threadIdx.x] > 1) {
+      const double2 a = sums.sum[3 * threadIdx.x], b = sums.sum[3 * threadIdx.x + 1], c = sums.sum[3 * threadIdx.x + 2];
+      E[0] = a.x;
+      E[1] = a.y;
+      E[2] = b.x;
+      Bs[0] = b.y;
+      Bs[1] = c.x;
+      Bs[2] = c.y;
+    } else {
+      for (int c = 0; c < 3; c++) {
+        E[c] = s.Eself[3 * i + c];
+        Bs[c] = s.Bself[3 * i + c];
+      }
+    }
+    const double xn[3] = {x[0], x[1], x[2]};
     double v[3], B[3];
     push_particle(x, u, E, Bs, bp, dt, v, B);
     const double x0 = x[0], x1 = x[1], x2 = x[2], v0 = v[0], v1 = v[1], v2 = v[2];
@@ -204,7 +278,6 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
   // the last block to finish advances the clock and resets the reduction for the next step (and, with
   // ep.on, evaluates the energy monitor of every bunch on the pushed state)
   __shared__ bool s_last;
-  __shared__ double s_num[kEnergyThreads], s_den[kEnergyThreads];
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -227,17 +300,23 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
   if (ep.on && s_last) {
     __threadfence();
     for (int b = 0; b < s.nbunch; b++)
-      energy_block(s, ep, mon, 0, b, half ? st.n : st.n + 1, t_n + dt, s.ke, s_num, s_den);
+      energy_block(s, ep, mon, 0, b, half ? st.n : st.n + 1, t_n + dt, s.ke);
   }
 }
 
 cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked,
-                             bool half, bool wide, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st) {
-  const long long threads = wide ? 32 * s.N : s.N;
+                             bool half, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st) {
   EnergyParams e{0, 1, 0.0};
   if (ep) e = *ep;  // the energy monitor in the last block (small systems)
-  step_post_kernel<<<(unsigned)((threads + kEnergyThreads - 1) / kEnergyThreads), kEnergyThreads, 0, st>>>(
-      s, b, ap, chunked ? 1 : 0, half ? 1 : 0, wide ? 1 : 0, e, mon);
+  const int p = post_particles(s.N);
+  const unsigned blocks = (unsigned)((s.N + p - 1) / p);
+  const int c = chunked ? 1 : 0, h = half ? 1 : 0;
+  if (p == 8)
+    step_post_kernel<8><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, e, mon);
+  else if (p == 16)
+    step_post_kernel<16><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, e, mon);
+  else
+    step_post_kernel<32><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, e, mon);
   return cudaGetLastError();
 }
 
