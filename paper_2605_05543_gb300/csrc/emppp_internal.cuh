@@ -282,6 +282,13 @@ struct PairLaunch {
   int wait_limit = 1 << 16;  // probes of a bounded wait on a staged history window (window shapes)
 };
 
+// the work item a block takes after `item` (-1: its first): from the counter, or, with a block for every item (small
+// systems), its own and no other, without the counter's round trips
+__device__ __forceinline__ int next_item(int item, int nitems, int* work) {
+  if (nitems <= (int)gridDim.x) return item < 0 ? (int)blockIdx.x : nitems;
+  return atomicAdd(work, 1);
+}
+
 // item -> (bunch, chunk, target tile): bunches are searched by their first item
 __device__ __forceinline__ void decode_item(const BunchSched* __restrict__ sched, int nbunch, int item, int& b,
                                             int& chunk_id, int& tb) {

@@ -24,6 +24,8 @@ __device__ __forceinline__ void energy_block(const DeviceState& s, const EnergyP
                                              int reset, int b, long long n, double t, const double* terms) {
   __shared__ double s_sum[2][kEnergyThreads];
   const BunchDesc& bd = s.bunches[b];
+  EnergyMon m;
+  if (threadIdx.x == 0) m = mon[b];
   double num = 0.0, den = 0.0;
   for (long long i = bd.off + threadIdx.x; i < bd.off + bd.n; i += kEnergyThreads) {
     const double w = __ldcg(s.wts + i);
@@ -52,7 +54,6 @@ __device__ __forceinline__ void energy_block(const DeviceState& s, const EnergyP
     num = s_sum[0][0];
     den = s_sum[1][0];
     const double ebar = num / den * (kMe * kC * kC);
-    EnergyMon m = mon[b];
     if (reset) {
       m.ebar = ebar;
       m.rate = 0.0;

@@ -130,9 +130,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs 
   int errbits = 0;
 
   // persistent blocks pull (source chunk, target tile) items, chunk-major, until none is left
+  if (threadIdx.x == 0) s_item = -1;
   for (;;) {
   __syncthreads();
-  if (threadIdx.x == 0) s_item = atomicAdd(a.work, 1);
+  if (threadIdx.x == 0) s_item = next_item(s_item, a.nitems, a.work);
   __syncthreads();
   const int item = s_item;
   if (item >= a.nitems) break;

@@ -307,9 +307,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
   }
 
   // persistent blocks pull (source chunk, target tile) items, chunk-major, until none is left
+  if (threadIdx.x == 0) s_item = -1;
   for (;;) {
   __syncthreads();
-  if (threadIdx.x == 0) s_item = atomicAdd(a.work, 1);
+  if (threadIdx.x == 0) s_item = next_item(s_item, a.nitems, a.work);
   __syncthreads();
   const int item = s_item;
   if (item >= a.nitems) break;

@@ -13,6 +13,7 @@
 // pair kernel is one launch.
 #include "emppp_internal.cuh"
 #include "energy.cuh"
+#include "fp64_roots.cuh"
 #include "push_math.cuh"
 #include "shadow.cuh"
 
@@ -108,7 +109,7 @@ struct ChunkSums {
   __device__ __forceinline__ void run(const DeviceState& s, long long i0) {
     if (threadIdx.x < P) {
       const long long i = i0 + threadIdx.x;
-      chunks[threadIdx.x] = i < s.N ? s.sched[s.bunch_of[i]].nchunk : 0;
+      chunks[threadIdx.x] = i < s.N ? s.sched[s.nbunch == 1 ? 0 : s.bunch_of[i]].nchunk : 0;
     }
     __syncthreads();
     if (threadIdx.x < kSumThreads) {
@@ -200,6 +201,7 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
                                                                    EnergyMon* __restrict__ mon) {
   __shared__ ChunkSums<P> sums;
   __shared__ double s_step[3];
+  __shared__ double s_new[P][12];  // pushed particles: x, u, and the slot before, x and v
   const long long i0 = (long long)blockIdx.x * P;
   const StepState st = *s.state;
   // slot of x^n, the slot the push writes and t_n
@@ -249,31 +251,52 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
         Bs[c] = s.Bself[3 * i + c];
       }
     }
-    const double xn[3] = {x[0], x[1], x[2]};
+    double* out = s_new[threadIdx.x];
+    for (int c = 0; c < 3; c++) {
+      out[6 + c] = x[c];
+      out[9 + c] = vn[c];
+    }
     double v[3], B[3];
     push_particle(x, u, E, Bs, bp, dt, v, B);
-    const double x0 = x[0], x1 = x[1], x2 = x[2], v0 = v[0], v1 = v[1], v2 = v[2];
-    if (!isfinite(x0 + x1 + x2 + u[0] + u[1] + u[2])) atomicOr(s.err, kErrNonFinite);
-    s.u[3 * i] = u[0];
-    s.u[3 * i + 1] = u[1];
-    s.u[3 * i + 2] = u[2];
-    if (ep.on) s.ke[i] = kinetic_term(u[0], u[1], u[2], s.wts[i]);  // for the monitor in the last block
-    for (int c = 0; c < 3; c++) s.Bout[3 * i + c] = B[c];
-    // append slot n+1 (both rings)
+    for (int c = 0; c < 3; c++) {
+      out[c] = x[c];
+      out[3 + c] = u[c];
+      s.u[3 * i + c] = u[c];
+      s.Bout[3 * i + c] = B[c];
+    }
+    if (!isfinite(x[0] + x[1] + x[2] + u[0] + u[1] + u[2])) atomicOr(s.err, kErrNonFinite);
+    // append slot n+1 to the FP64 ring
     double* r = s.rec64 + ((size_t)i * s.D + pnext) * 6;
-    reinterpret_cast<double2*>(r)[0] = make_double2(x0, x1);
-    reinterpret_cast<double2*>(r)[1] = make_double2(x2, v0);
-    reinterpret_cast<double2*>(r)[2] = make_double2(v1, v2);
-    float4 q[3];
-    const BunchDesc& bd = s.bunches[s.bunch_of[i]];
-    shadow_record(bd.origin, bd.beta_ref, x0, x1, x2, v0, v1, v2, gamma2_of_u(u[0], u[1], u[2]), q);
-    float4* o = reinterpret_cast<float4*>(s.rec32 + ((size_t)i * s.D + pnext) * 12);
-    o[0] = q[0];
-    o[1] = q[1];
-    o[2] = q[2];
-    // how far slot n + 1 lies from slot n's line (newer-node bound of the mixed path)
-    s.rec32[((size_t)i * s.D + pfrom) * 12 + 7] =
-        line_deviation(xn[0], xn[1], xn[2], vn[0], vn[1], vn[2], x0, x1, x2, (t_n + dt) - t_n);
+    reinterpret_cast<double2*>(r)[0] = make_double2(x[0], x[1]);
+    reinterpret_cast<double2*>(r)[1] = make_double2(x[2], v[0]);
+    reinterpret_cast<double2*>(r)[2] = make_double2(v[1], v[2]);
+    vn[0] = v[0];
+    vn[1] = v[1];
+    vn[2] = v[2];
+  }
+  __syncthreads();
+  // What follows from the pushed state, by a warp each: the FP32 record, the monitor's term, and how far slot n + 1
+  // lies from slot n's line (newer-node bound of the mixed path)
+  const int task = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long it = i0 + lane;
+  if (task < 3 && lane < P && it < s.N) {
+    const double* o = s_new[lane];
+    if (task == 0) {
+      const BunchDesc& bd = s.bunches[s.nbunch == 1 ? 0 : s.bunch_of[it]];
+      // gamma^2 = 1 + u.u / c^2 and its inverse without divisions (both are rounded to FP32)
+      const double gamma2 = 1.0 + (o[3] * o[3] + o[4] * o[4] + o[5] * o[5]) * (1.0 / (kC * kC));
+      float4 q[3];
+      shadow_record(bd.origin, bd.beta_ref, o[0], o[1], o[2], vn[0], vn[1], vn[2], gamma2, recip_refined(gamma2), q);
+      float4* w = reinterpret_cast<float4*>(s.rec32 + ((size_t)it * s.D + pnext) * 12);
+      w[0] = q[0];
+      w[1] = q[1];
+      w[2] = q[2];
+    } else if (task == 1) {
+      if (ep.on) s.ke[it] = kinetic_term(o[3], o[4], o[5], s.wts[it]);
+    } else {
+      s.rec32[((size_t)it * s.D + pfrom) * 12 + 7] =
+          line_deviation(o[6], o[7], o[8], o[9], o[10], o[11], o[0], o[1], o[2], (t_n + dt) - t_n);
+    }
   }
   // the last block to finish advances the clock and resets the reduction for the next step (and, with
   // ep.on, evaluates the energy monitor of every bunch on the pushed state)

@@ -160,8 +160,9 @@ __device__ __forceinline__ void slot_table(const DeviceState& s, int l, int p0, 
   if (l + 1 < nwin) {
     int q = p + 1 == s.D ? 0 : p + 1;
     const double dtk = s.slot_t[q] - tk;
-    s.tab.tab64[p] = make_double2(t_n - tk, 1.0 / dtk);
-    icdt = (float)(1.0 / (kC * dtk));
+    const double idt = recip_refined(dtk);
+    s.tab.tab64[p] = make_double2(t_n - tk, idt);
+    icdt = (float)(idt * (1.0 / kC));
   } else {
     s.tab.tab64[p] = make_double2(t_n - tk, 0.0);
   }
