@@ -69,6 +69,13 @@ struct emppp_ctx {
   double t = 0.0;          // host mirror of t_n
   int64_t hist_start = 0;  // host mirror of the earliest stored slot
   double* staging = nullptr;  // [7N] doubles for host transfers
+  // page-locked host words that a call's small reads from the device land in, so that one wait serves all of them
+  struct HostPage {
+    int err;
+    StepState state;
+  };
+  HostPage* page = nullptr;
+  double* frames = nullptr;  // page-locked: first positions and velocities of the bunches [nbunch][6], then [D]
   std::vector<void*> allocs;
   // bunches
   int nbunch = 1;
@@ -189,7 +196,9 @@ void invalidate_graph(emppp_handle h) {
 // cost of the items (the branch mix differs across a bunch) evens out; systems too small for that get
 // one round of items with short chunks instead. At most max_split chunks per bunch. Uploaded when the
 // configuration changes.
-constexpr long long kMinChunk = 4;  // fewest sources per chunk
+// fewest sources per chunk: 4 on the mixed path, 2 on the FP64 path, whose pairs are a longer chain (N = 256: 127 us with 4,
+// 115 with 2, a call that takes one step and reads the state back)
+constexpr long long kMinChunkMixed = 4, kMinChunkFp64 = 2;
 
 emppp_status update_schedule(emppp_handle c) {
   const bool mixed = c->opt.precision == EMPPP_MIXED;
@@ -232,8 +241,9 @@ emppp_status update_schedule(emppp_handle c) {
   }();
   // chunking of one bunch: about items_per_block items per resident block over all bunches (counted in
   // 128-target tiles), in whole tiles of TB sources and at least 256 sources (small == false); or, for a
-  // system too small to fill the resident blocks that way, one round of items with chunks of 4k sources
+  // system too small to fill the resident blocks that way, one round of items with short chunks
   // (small == true), since then each block's time is its own chunk length
+  const long long kMin = mixed ? kMinChunkMixed : kMinChunkFp64;
   auto chunks = [&](long long n, bool small) -> long long {
     long long nchunk;
     if (c->opt.source_split > 0) {
@@ -246,13 +256,13 @@ emppp_status update_schedule(emppp_handle c) {
       if (nchunk > by_size) nchunk = by_size;
     } else {
       nchunk = Rreal / total_tiles > 1 ? Rreal / total_tiles : 1;
-      const long long by_size = (n + kMinChunk - 1) / kMinChunk;
+      const long long by_size = (n + kMin - 1) / kMin;
       if (nchunk > by_size) nchunk = by_size;
     }
     if (nchunk > c->ds.max_split) nchunk = c->ds.max_split;
     if (nchunk < 1) nchunk = 1;
     long long chunk = (n + nchunk - 1) / nchunk;
-    return chunk >= TB ? (chunk + TB - 1) / TB * TB : (chunk + kMinChunk - 1) / kMinChunk * kMinChunk;
+    return chunk >= TB ? (chunk + TB - 1) / TB * TB : (chunk + kMin - 1) / kMin * kMin;
   };
   long long items_large = 0;
   for (int b = 0; b < c->nbunch; b++) {
@@ -288,10 +298,14 @@ bool any_chunked(const emppp_ctx* c) {
   return false;
 }
 
-emppp_status read_err(emppp_handle h) {
-  int herr = 0;
-  CU(cudaMemcpyAsync(&herr, h->ds.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-  CU(cudaStreamSynchronize(h->stream));
+// the device error word: request_err enqueues its copy to the host, check_err reports it after the stream is waited for
+emppp_status request_err(emppp_handle h) {
+  CU(cudaMemcpyAsync(&h->page->err, h->ds.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  return EMPPP_OK;
+}
+
+emppp_status check_err(emppp_handle h) {
+  const int herr = h->page->err;
   if (herr == kErrTimeout) {
     CU(cudaMemsetAsync(h->ds.err, 0, sizeof(int), h->stream));
     CU(cudaStreamSynchronize(h->stream));
@@ -307,14 +321,32 @@ emppp_status read_err(emppp_handle h) {
   return EMPPP_OK;
 }
 
-// with the adaptive time step the device chooses each step's size: refresh the host mirror of t_n
+emppp_status read_err(emppp_handle h) {
+  emppp_status st = request_err(h);
+  if (st != EMPPP_OK) return st;
+  CU(cudaStreamSynchronize(h->stream));
+  return check_err(h);
+}
+
+// with the adaptive time step the device chooses each step's size: refresh the host mirror of t_n (request_time enqueues the
+// copy, take_time reads it after the stream is waited for)
+emppp_status request_time(emppp_handle h) {
+  if (h->t_stale)
+    CU(cudaMemcpyAsync(&h->page->state, h->ds.state, sizeof(StepState), cudaMemcpyDeviceToHost, h->stream));
+  return EMPPP_OK;
+}
+
+void take_time(emppp_handle h) {
+  if (h->t_stale) h->t = h->page->state.t;
+  h->t_stale = false;
+}
+
 emppp_status sync_time(emppp_handle h) {
   if (!h->t_stale) return EMPPP_OK;
-  StepState hs;
-  CU(cudaMemcpyAsync(&hs, h->ds.state, sizeof(StepState), cudaMemcpyDeviceToHost, h->stream));
+  emppp_status st = request_time(h);
+  if (st != EMPPP_OK) return st;
   CU(cudaStreamSynchronize(h->stream));
-  h->t = hs.t;
-  h->t_stale = false;
+  take_time(h);
   return EMPPP_OK;
 }
 
@@ -331,27 +363,24 @@ emppp_status from_device(emppp_handle h, double* dst, const double* src, size_t 
   return EMPPP_OK;
 }
 
-// reads 3 doubles at element 3*i of a caller array (host or device)
-emppp_status read3(emppp_handle h, const double* a, long long i, int is_dev, double out[3]) {
-  if (is_dev) {
-    CU(cudaMemcpyAsync(out, a + 3 * i, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CU(cudaStreamSynchronize(h->stream));
-  } else {
-    memcpy(out, a + 3 * i, 3 * sizeof(double));
-  }
-  return EMPPP_OK;
-}
-
 // Origin of each bunch's FP32 position split and reference velocity of its FP32 velocities: those of
 // the bunch's first particle when the state is set. x and v_or_u index the present positions and
-// velocities (or proper velocities).
+// velocities (or proper velocities). Device arrays are read with one wait, which also serves what the caller enqueued.
 emppp_status set_bunch_frames(emppp_handle h, const double* x, const double* v_or_u, bool is_u, int is_dev) {
+  double* f = h->frames;
   for (int b = 0; b < h->nbunch; b++) {
-    double x0[3], v0[3];
-    emppp_status st = read3(h, x, h->hb[b].off, is_dev, x0);
-    if (st != EMPPP_OK) return st;
-    st = read3(h, v_or_u, h->hb[b].off, is_dev, v0);
-    if (st != EMPPP_OK) return st;
+    const long long i = h->hb[b].off;
+    if (is_dev) {
+      CU(cudaMemcpyAsync(f + 6 * b, x + 3 * i, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+      CU(cudaMemcpyAsync(f + 6 * b + 3, v_or_u + 3 * i, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    } else {
+      memcpy(f + 6 * b, x + 3 * i, 3 * sizeof(double));
+      memcpy(f + 6 * b + 3, v_or_u + 3 * i, 3 * sizeof(double));
+    }
+  }
+  if (is_dev) CU(cudaStreamSynchronize(h->stream));
+  for (int b = 0; b < h->nbunch; b++) {
+    const double *x0 = f + 6 * b, *v0 = x0 + 3;
     double g = 1.0;
     if (is_u) g = sqrt(1.0 + (v0[0] * v0[0] + v0[1] * v0[1] + v0[2] * v0[2]) / (kC * kC));
     for (int c = 0; c < 3; c++) {
@@ -360,8 +389,7 @@ emppp_status set_bunch_frames(emppp_handle h, const double* x, const double* v_o
     }
   }
   CU(cudaMemcpyAsync(h->d_bunches, h->hb.data(), sizeof(BunchDesc) * h->nbunch, cudaMemcpyHostToDevice, h->stream));
-  CU(cudaStreamSynchronize(h->stream));
-  return EMPPP_OK;
+  return EMPPP_OK;  // the caller waits for the stream before it returns
 }
 
 emppp_status ensure_events(emppp_handle h) {
@@ -628,6 +656,14 @@ emppp_status create_impl(int32_t nbunch, const int64_t* nper, int32_t history_de
   s.sched = c->d_sched;
   s.bunch_of = c->d_bunch_of;
   s.mlp_image = c->mlp_image;
+  e = cudaMallocHost(reinterpret_cast<void**>(&c->page), sizeof(emppp_ctx::HostPage));
+  if (e == cudaSuccess)
+    e = cudaMallocHost(reinterpret_cast<void**>(&c->frames), sizeof(double) * (6 * (size_t)nbunch + D));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    emppp_destroy(c);
+    return fail(EMPPP_ERR_OOM, "page-locked host words: %s", cudaGetErrorString(e));
+  }
   e = cudaMemcpyAsync(c->d_bunch_of, bunch_of.data(), sizeof(int) * N, cudaMemcpyHostToDevice, c->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(c->d_bunches, c->hb.data(), sizeof(BunchDesc) * nbunch, cudaMemcpyHostToDevice, c->stream);
@@ -699,6 +735,8 @@ EMPPP_API void emppp_destroy(emppp_handle h) {
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   for (void* p : h->allocs) cudaFree(p);
+  if (h->page) cudaFreeHost(h->page);
+  if (h->frames) cudaFreeHost(h->frames);
   delete h;
 }
 
@@ -755,12 +793,12 @@ EMPPP_API emppp_status emppp_set_history(emppp_handle h, int64_t n, int32_t nslo
   if (nslots != want)
     return fail(EMPPP_ERR_ARG, "nslots must be min(n + 1, depth) = %lld (got %d)", (long long)want, nslots);
   const size_t N = (size_t)h->N;
-  std::vector<double> hT(nslots);
+  double* hT = h->frames + 6 * (size_t)h->nbunch;
   if (is_device_ptr) {
-    CU(cudaMemcpyAsync(hT.data(), T, sizeof(double) * nslots, cudaMemcpyDeviceToHost, h->stream));
+    CU(cudaMemcpyAsync(hT, T, sizeof(double) * nslots, cudaMemcpyDeviceToHost, h->stream));
     CU(cudaStreamSynchronize(h->stream));
   } else {
-    memcpy(hT.data(), T, sizeof(double) * nslots);
+    memcpy(hT, T, sizeof(double) * nslots);
   }
   for (int s = 0; s < nslots; s++) {
     if (!(hT[s] == hT[s]) || (s > 0 && !(hT[s] > hT[s - 1])))
@@ -959,7 +997,7 @@ EMPPP_API emppp_status emppp_get_state(emppp_handle h, double* x, double* u, dou
   emppp_status st = check_handle(h);
   if (st != EMPPP_OK) return st;
   if (!h->has_state) return fail(EMPPP_ERR_STATE, "no state: call emppp_set_particles first");
-  if ((st = read_err(h)) != EMPPP_OK) return st;
+  if ((st = request_err(h)) != EMPPP_OK || (st = request_time(h)) != EMPPP_OK) return st;
   const size_t N = (size_t)h->N;
   if (x) {
     h->launches += 1;
@@ -972,7 +1010,8 @@ EMPPP_API emppp_status emppp_get_state(emppp_handle h, double* x, double* u, dou
   }
   if (u && (st = from_device(h, u, h->ds.u, 3 * N, is_device_ptr)) != EMPPP_OK) return st;
   CU(cudaStreamSynchronize(h->stream));
-  if ((st = sync_time(h)) != EMPPP_OK) return st;
+  if ((st = check_err(h)) != EMPPP_OK) return st;
+  take_time(h);
   if (t_now) *t_now = h->t;
   if (n_now) *n_now = h->n;
   return EMPPP_OK;
@@ -982,12 +1021,12 @@ EMPPP_API emppp_status emppp_get_fields(emppp_handle h, double* E, double* B, in
   emppp_status st = check_handle(h);
   if (st != EMPPP_OK) return st;
   if (!h->has_state) return fail(EMPPP_ERR_STATE, "no state: call emppp_set_particles first");
-  if ((st = read_err(h)) != EMPPP_OK) return st;
+  if ((st = request_err(h)) != EMPPP_OK) return st;
   const size_t N = (size_t)h->N;
   if (E && (st = from_device(h, E, h->ds.Eself, 3 * N, is_device_ptr)) != EMPPP_OK) return st;
   if (B && (st = from_device(h, B, h->ds.Bout, 3 * N, is_device_ptr)) != EMPPP_OK) return st;
   CU(cudaStreamSynchronize(h->stream));
-  return EMPPP_OK;
+  return check_err(h);
 }
 
 EMPPP_API emppp_status emppp_get_stats(emppp_handle h, emppp_stats* out) {
@@ -1449,10 +1488,11 @@ EMPPP_API emppp_status emppp_get_energy(emppp_handle h, emppp_energy_state* out)
   if (st != EMPPP_OK) return st;
   if (!out) return fail(EMPPP_ERR_ARG, "out is NULL");
   if (!h->energy.on || !h->has_state) return fail(EMPPP_ERR_STATE, "energy monitor off or no state");
-  if ((st = read_err(h)) != EMPPP_OK) return st;
+  if ((st = request_err(h)) != EMPPP_OK) return st;
   std::vector<EnergyMon> m((size_t)h->nbunch);
   CU(cudaMemcpyAsync(m.data(), h->d_mon, sizeof(EnergyMon) * m.size(), cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
+  if ((st = check_err(h)) != EMPPP_OK) return st;
   for (int b = 0; b < h->nbunch; b++) {
     out[b].ebar = m[b].ebar;
     out[b].rate = m[b].rate;
