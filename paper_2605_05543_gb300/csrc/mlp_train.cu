@@ -10,11 +10,14 @@
 //   - the weight gradients are FP32 as outer products in registers (each thread 4 x 4 of dW2, per row
 //     two 16-byte shared loads for 16 FMAs) instead of read-modify-writes of shared memory;
 //   - each block writes its partial gradient once, and adam_kernel sums the blocks in a fixed order (no atomics, so a
-//     training run is reproducible), updates and rewrites the operands: no zeroing, no image launch;
+//     training run is reproducible), updates and rewrites the operands: no zeroing, no image launch. Each 64 rows are
+//     summed by themselves, 16 after 16, and the 64s one after the other: training amplifies a last bit's difference
+//     of a gradient by a hundred and more (BF16 operands that round the other way), so the sums keep the grouping that
+//     trained networks so far were made with, at 0.9 us a batch more than plain sums of 32 rows;
 //   - each launch starts while the one before it drains (programmatic dependent launch) and waits before it reads
 //     what that one writes.
 // 49 batches of 4096 rows: 2.73 ms before (64 blocks of four warps, gradients in shared memory, atomics, four launches per
-// batch: 55 us each), 0.78 ms now (10.4 us a batch, and 0.28 ms of the call's own allocation, copies and waits).
+// batch: 55 us each), 0.80 ms now (10.6 us a batch, and 0.28 ms of the call's own allocation, copies and waits).
 //
 // Rounding points (also followed by the CPU reference in oracle/mlp.py): the GEMM operands X, W1, A1 =
 // silu(H1), W2 (forward) and dH2, W2 (input gradient) are rounded to BF16; products accumulate in FP32;
@@ -32,6 +35,7 @@ constexpr int kThreads = 256;   // eight warps: two 16-row halves by four groups
 constexpr int kLd = 72;         // row stride of the staged activations: fragment reads of a half-warp hit 32 banks
 constexpr int kGrad = 4992;     // floats between two blocks' partial gradients (4929 rounded up to whole lines)
 constexpr int kAdamSlices = 8;  // threads that share the sum of one parameter
+constexpr int kAdamPairs = 64;  // pairs of blocks summed per turn
 
 // B fragments of the tensor-core passes, lane-major: entry [n-tile][k-step][lane] holds rows k = 16 kk + 2t, + 1 (x)
 // and + 8, + 9 (y) of column n = 8 nt + g
@@ -81,7 +85,6 @@ struct TrainSmem {
   float A1[kRows][kLd], A2[kRows][kLd], dH1[kRows][kLd], dH2[kRows][kLd];
   float X[kRows][12];
   float z[kRows][4][kH / 8 + 1];  // the output's terms per row, fragment column pair and n-tile
-  float red[1][2];
   float dz[kRows];
 };
 
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(kThreads, 2) train_kernel(const TrainImage* im
   const int ra = 16 * (w & 1) + g, rb = ra + 8, q = w >> 1;
   const int u2 = 4 * (tid >> 4), o2 = 4 * (tid & 15);  // this thread's 4 x 4 of dW2
   const int u1 = tid & 63, part = tid >> 6;             // this thread's column of the smaller gradients, and which
-  float acc[4][4] = {}, gW1[2] = {}, gv[2] = {}, gb3 = 0.f, loss_acc = 0.f;
+  float acc[2][4][4] = {}, gs[2][4] = {}, gb3[2] = {}, loss_acc = 0.f;  // sums by 16-row half of the tile
   if (tid < kRows) S.X[tid][10] = S.X[tid][11] = 0.f;
   bool waited = false;
   for (long long tile = blockIdx.x; tile * kRows < rows; tile += gridDim.x) {
@@ -176,8 +179,8 @@ __global__ void __launch_bounds__(kThreads, 2) train_kernel(const TrainImage* im
         }
         *reinterpret_cast<float2*>(&S.A2[ra][o]) = make_float2(v[0], v[1]);
         *reinterpret_cast<float2*>(&S.A2[rb][o]) = make_float2(v[2], v[3]);
-        S.z[ra][t][nt] = v[0] * w3[n][0] + v[1] * w3[n][1];
-        S.z[rb][t][nt] = v[2] * w3[n][0] + v[3] * w3[n][1];
+        S.z[ra][t][nt] = fmaf(v[0], w3[n][0], v[1] * w3[n][1]);
+        S.z[rb][t][nt] = fmaf(v[3], w3[n][1], v[2] * w3[n][0]);
       }
     }
     __syncthreads();
@@ -229,12 +232,13 @@ __global__ void __launch_bounds__(kThreads, 2) train_kernel(const TrainImage* im
         *reinterpret_cast<float2*>(&S.dH1[rb][o]) = make_float2(c[n][2] * d1[n][2], c[n][3] * d1[n][3]);
       }
     }
-    // Weight gradients, 16 rows at a time: each sum of 16 starts from zero and is then added, which halves the length
-    // of the rounding chain. dW2[u][o] += A1[r][u] dH2[r][o]
-    for (int h = 0; h < kRows; h += 16) {
+    // Weight gradients, 16 rows at a time: each sum of 16 starts from zero and is then added.
+    // (One copy of the code for both halves: two cost 0.5 us a batch more.) dW2[u][o] += A1[r][u] dH2[r][o]
+#pragma unroll 1
+    for (int h = 0; h < 2; h++) {
       float c[4][4] = {};
 #pragma unroll
-      for (int r = h; r < h + 16; r++) {
+      for (int r = 16 * h; r < 16 * h + 16; r++) {
         const float4 x = *reinterpret_cast<const float4*>(&S.A1[r][u2]), y = *reinterpret_cast<const float4*>(&S.dH2[r][o2]);
         const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
@@ -245,34 +249,40 @@ __global__ void __launch_bounds__(kThreads, 2) train_kernel(const TrainImage* im
 #pragma unroll
       for (int a = 0; a < 4; a++)
 #pragma unroll
-        for (int b = 0; b < 4; b++) acc[a][b] += c[a][b];
+        for (int b = 0; b < 4; b++) {
+          if (h == 0) acc[0][a][b] += c[a][b];
+          else acc[1][a][b] += c[a][b];
+        }
     }
     __syncthreads();
     // dW1[f][u] += X[r][f] dH1[r][u] (part p: features p, p + 4, p + 8); db1 (part 2), db2 and dw3 (part 3); db3
-    for (int h = 0; h < kRows; h += 16) {
-      float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
+#pragma unroll 1
+    for (int h = 0; h < 2; h++) {
+      float c[4] = {};
 #pragma unroll
-      for (int r = h; r < h + 16; r++) {
+      for (int r = 16 * h; r < 16 * h + 16; r++) {
         const float dh1 = S.dH1[r][u1];
-        c0 += S.X[r][part] * dh1;
-        c1 += S.X[r][part + 4] * dh1;
+        c[0] = fmaf(S.X[r][part], dh1, c[0]);
+        c[1] = fmaf(S.X[r][part + 4], dh1, c[1]);
         if (part < 2) {
-          c2 += S.X[r][part + 8] * dh1;
+          c[2] = fmaf(S.X[r][part + 8], dh1, c[2]);
         } else if (part == 2) {
-          c2 += dh1;
+          c[2] += dh1;
         } else {
-          c2 += S.dH2[r][u1];
-          c3 += S.A2[r][u1] * S.dz[r];
+          c[2] += S.dH2[r][u1];
+          c[3] = fmaf(S.A2[r][u1], S.dz[r], c[3]);
         }
       }
-      gW1[0] += c0;
-      gW1[1] += c1;
-      gv[0] += c2;
-      gv[1] += c3;
+#pragma unroll
+      for (int a = 0; a < 4; a++) {
+        if (h == 0) gs[0][a] += c[a];
+        else gs[1][a] += c[a];
+      }
       if (tid == 0) {
         float c = 0.f;
-        for (int r = h; r < h + 16; r++) c += S.dz[r];
-        gb3 += c;
+        for (int r = 16 * h; r < 16 * h + 16; r++) c += S.dz[r];
+        if (h == 0) gb3[0] += c;
+        else gb3[1] += c;
       }
     }
     __syncthreads();
@@ -281,49 +291,69 @@ __global__ void __launch_bounds__(kThreads, 2) train_kernel(const TrainImage* im
     wait_for_previous();
     let_next_start();
   }
-  // this block's gradient and loss
-  float* out = partial + (size_t)blockIdx.x * kGrad;
+  // this block's gradient: an even block's two halves are added, an odd block's follow them in adam_kernel's sum
+  const bool odd = blockIdx.x & 1;
+  float* out = partial + ((size_t)(blockIdx.x >> 1) * 3 + (odd ? 1 : 0)) * kGrad;
+  const int u1_last = part < 2 ? kOffW1 + (part + 8) * kH + u1 : (part == 2 ? kOffB1 : kOffB2) + u1;
+  if (!odd) {
 #pragma unroll
-  for (int a = 0; a < 4; a++)
-    *reinterpret_cast<float4*>(out + kOffW2 + (u2 + a) * kH + o2) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
-  out[kOffW1 + part * kH + u1] = gW1[0];
-  out[kOffW1 + (part + 4) * kH + u1] = gW1[1];
-  if (part < 2) {
-    out[kOffW1 + (part + 8) * kH + u1] = gv[0];
-  } else if (part == 2) {
-    out[kOffB1 + u1] = gv[0];
-  } else {
-    out[kOffB2 + u1] = gv[0];
-    out[kOffW3 + u1] = gv[1];
-  }
-  if (w < 2) {  // the warps of group 0 hold the rows' errors (lanes t = 0)
+    for (int a = 0; a < 4; a++)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
-    if (lane == 0) S.red[0][w] = loss_acc;
+      for (int b = 0; b < 4; b++) acc[0][a][b] += acc[1][a][b];
+#pragma unroll
+    for (int a = 0; a < 4; a++) gs[0][a] += gs[1][a];
+    gb3[0] += gb3[1];
   }
-  __syncthreads();
-  if (tid == 0) {
-    out[kOffB3] = gb3;
-    atomicAdd(loss, S.red[0][0] + S.red[0][1]);
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    if (h == 1 && !odd) break;
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+      *reinterpret_cast<float4*>(out + kOffW2 + (u2 + a) * kH + o2) =
+          make_float4(acc[h][a][0], acc[h][a][1], acc[h][a][2], acc[h][a][3]);
+    out[kOffW1 + part * kH + u1] = gs[h][0];
+    out[kOffW1 + (part + 4) * kH + u1] = gs[h][1];
+    out[u1_last] = gs[h][2];
+    if (part == 3) out[kOffW3 + u1] = gs[h][3];
+    if (tid == 0) out[kOffB3] = gb3[h];
+    out += kGrad;
+  }
+  if (w < 2) {  // the warps of group 0 hold the rows' errors (lanes t = 0); a sum of 16 rows each
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
+    if (lane == 0) atomicAdd(loss, loss_acc);
   }
 }
 
-// the sum over the blocks of parameter k's gradient: kAdamSlices threads (the warps of a block) take the blocks in
-// turn, warp 0 adds their sums; every lane of warp 0 returns its parameter's
+// The sum over the blocks of parameter k's gradient, in a fixed order: the 64 rows of each pair of blocks, then pair after
+// pair. The warps of a block (kAdamSlices) load and add within the pairs in turn, warp 0 adds the pairs; every lane of
+// warp 0 returns its parameter's.
 __device__ __forceinline__ float gradient_sum(const float* partial, int nblocks, int k) {
-  __shared__ float s_sum[kAdamSlices][32];
-  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
-  float s = 0.f;
-  if (k < kNumParams) {
-#pragma unroll 8
-    for (int b = sl; b < nblocks; b += kAdamSlices) s += __ldcg(partial + (size_t)b * kGrad + k);
-  }
-  s_sum[sl][lane] = s;
-  __syncthreads();
+  __shared__ float s_sum[kAdamPairs][32];
+  const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5, npairs = (nblocks + 1) >> 1;
   float g = 0.f;
-  if (sl == 0)
+  for (int p0 = 0; p0 < npairs; p0 += kAdamPairs) {
+    if (p0 > 0) __syncthreads();
+    float v[kAdamPairs / kAdamSlices][3];  // all loads in flight: rows that do not exist read the first and count zero
 #pragma unroll
-    for (int q = 0; q < kAdamSlices; q++) g += s_sum[q][lane];
+    for (int i = 0; i < kAdamPairs / kAdamSlices; i++) {
+      const int q = p0 + sl + i * kAdamSlices;
+      const bool one = k < kNumParams && q < npairs, two = one && 2 * q + 1 < nblocks;
+      const float* at = partial + (one ? (size_t)q * 3 * kGrad + k : 0);
+      v[i][0] = __ldcg(at);
+      v[i][1] = __ldcg(at + (two ? kGrad : 0));
+      v[i][2] = __ldcg(at + (two ? 2 * kGrad : 0));
+      if (!one) v[i][0] = 0.f;
+      if (!two) v[i][1] = v[i][2] = 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < kAdamPairs / kAdamSlices; i++) s_sum[sl + i * kAdamSlices][lane] = (v[i][0] + v[i][1]) + v[i][2];
+    __syncthreads();
+    if (sl == 0) {
+#pragma unroll 16
+      for (int q = 0; q < kAdamPairs; q++) g += s_sum[q][lane];  // (beyond npairs: zeros)
+    }
+  }
   return g;
 }
 
@@ -374,9 +404,9 @@ cudaError_t launch_after(void (*kernel)(Args...), int blocks, int threads, bool 
 
 namespace emppp {
 
-// device buffer of a training run: operands, then each block's partial gradient
+// device buffer of a training run: operands, then three partial gradients per pair of blocks
 size_t train_buffer_bytes(long long batch_rows, int num_sms) {
-  return sizeof(TrainImage) + (size_t)train_blocks(batch_rows, num_sms) * kGrad * sizeof(float);
+  return sizeof(TrainImage) + (size_t)((train_blocks(batch_rows, num_sms) + 1) / 2 * 3) * kGrad * sizeof(float);
 }
 
 cudaError_t launch_train_image(const float* params, void* buffer, cudaStream_t st) {
