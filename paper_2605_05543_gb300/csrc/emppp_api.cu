@@ -1,6 +1,7 @@
 // C ABI of the EM-PP library: handle lifetime, state transfer, the step driver, the stage-2 handoff
 // and transport. Every entry point validates its arguments, enqueues work on the handle's stream and
 // returns a status; nothing here aborts or prints.
+#include <algorithm>
 #include <cmath>
 #include <cstddef>
 #include <cstdarg>
@@ -192,11 +193,11 @@ void invalidate_graph(emppp_handle h) {
 }
 
 // Work split of the persistent pair kernel, per bunch: one block per resident slot of the kernel that
-// is launched (occupancy query) and about 16 work items per block over all bunches, so that the uneven
+// is launched (occupancy query) and a few dozen work items per block over all bunches, so that the uneven
 // cost of the items (the branch mix differs across a bunch) evens out; systems too small for that get
 // one round of items with short chunks instead. At most max_split chunks per bunch. Uploaded when the
 // configuration changes.
-// fewest sources per chunk: 4 on the mixed path, 2 on the FP64 path, whose pairs are a longer chain (N = 256: 127 us with 4,
+// fewest sources per chunk of a single round: 4 on the mixed path, 2 on the FP64 path, whose pairs are a longer chain (N = 256: 127 us with 4,
 // 115 with 2, a call that takes one step and reads the state back)
 constexpr long long kMinChunkMixed = 4, kMinChunkFp64 = 2;
 
@@ -239,38 +240,43 @@ emppp_status update_schedule(emppp_handle c) {
     for (int b = 0; b < c->nbunch; b++) t += (c->hb[b].n + 127) / 128;
     return t;
   }();
-  // chunking of one bunch: about items_per_block items per resident block over all bunches (counted in
-  // 128-target tiles), in whole tiles of TB sources and at least 256 sources (small == false); or, for a
-  // system too small to fill the resident blocks that way, one round of items with short chunks
-  // (small == true), since then each block's time is its own chunk length
-  const long long kMin = mixed ? kMinChunkMixed : kMinChunkFp64;
+  // Chunking of one bunch. Mixed path: about 2 items_per_block items per resident block over all bunches (counted in
+  // 128-target tiles), in whole tiles of TB sources and at least 256 sources (small == false); or, for a system too
+  // small to fill the resident blocks that way, one round of items with short chunks (small == true), since then each
+  // block's time is its own chunk length.
+  // FP64 path: an SM with few blocks left runs below its FP64 rate, and a pair in the history costs twice one beyond
+  // it, so the items are many and short: as many as 2 items_per_block per resident block allow, of at least 8 sources
+  // (below which an item's own set-up shows), or one round if that is more. The step in us by sources per chunk, with
+  // bisection, 512 slots: N = 1024: 12 (one round) 267, 8 277, 4 260; N = 2048: 44 (one round) 770, 32 832, 16 724,
+  // 8 711; N = 4096: 256 2922, 128 2765, 64 2481, 32 2382, 16 2354; N = 8192: 256 9351, 64 8732, 32 8623; N = 16381
+  // with the guess: 256 29434, 64 28638. (The partial sums, 200 MB there, cost less than they save.)
   auto chunks = [&](long long n, bool small) -> long long {
+    const long long one_round = Rreal / total_tiles > 1 ? Rreal / total_tiles : 1;
+    const long long many = (2LL * c->items_per_block * Rsched + tiles128 - 1) / tiles128;
+    auto of = [&](long long nchunk, long long fewest) { return std::min(nchunk, (n + fewest - 1) / fewest); };
+    const long long kMin = mixed ? kMinChunkMixed : kMinChunkFp64;
     long long nchunk;
-    if (c->opt.source_split > 0) {
+    if (c->opt.source_split > 0)
       nchunk = c->opt.source_split;
-    } else if (!small) {
-      // the FP64 path gathers both rings, so its chunks are cut 4x shorter to keep a chunk's window in L2
-      const long long ipb = mixed ? 2LL * c->items_per_block : 4LL * c->items_per_block;
-      nchunk = (ipb * Rsched + tiles128 - 1) / tiles128;
-      const long long by_size = (n + 255) / 256;
-      if (nchunk > by_size) nchunk = by_size;
-    } else {
-      nchunk = Rreal / total_tiles > 1 ? Rreal / total_tiles : 1;
-      const long long by_size = (n + kMin - 1) / kMin;
-      if (nchunk > by_size) nchunk = by_size;
-    }
-    if (nchunk > c->ds.max_split) nchunk = c->ds.max_split;
-    if (nchunk < 1) nchunk = 1;
-    long long chunk = (n + nchunk - 1) / nchunk;
-    return chunk >= TB ? (chunk + TB - 1) / TB * TB : (chunk + kMin - 1) / kMin * kMin;
+    else if (!mixed)
+      nchunk = std::max(of(one_round, kMin), of(many, 8));
+    else
+      nchunk = small ? of(one_round, kMin) : of(many, 256);
+    nchunk = std::max(1LL, std::min(nchunk, (long long)c->ds.max_split));
+    const long long chunk = (n + nchunk - 1) / nchunk;
+    const bool tiles = chunk >= TB && (mixed || c->opt.source_split > 0);
+    return tiles ? (chunk + TB - 1) / TB * TB : (chunk + kMin - 1) / kMin * kMin;
   };
-  long long items_large = 0;
-  for (int b = 0; b < c->nbunch; b++) {
-    const long long n = c->hb[b].n;
-    const long long chunk = chunks(n, false);
-    items_large += ((n + TB - 1) / TB) * ((n + chunk - 1) / chunk);
+  bool small = false;
+  if (mixed) {
+    long long items_large = 0;
+    for (int b = 0; b < c->nbunch; b++) {
+      const long long n = c->hb[b].n;
+      const long long chunk = chunks(n, false);
+      items_large += ((n + TB - 1) / TB) * ((n + chunk - 1) / chunk);
+    }
+    small = items_large < Rreal;
   }
-  const bool small = items_large < Rreal;
   int item = 0;
   for (int b = 0; b < c->nbunch; b++) {
     BunchSched& s = c->hs[b];

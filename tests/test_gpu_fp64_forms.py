@@ -63,7 +63,7 @@ def extended_fields(h, D):
     (63, 20, 64, 10e-6, 3.0, 1e-15, 1),   # one source short of a tile
     (64, 70, 32, 10e-6, 3.0, 1e-15, 1),   # a whole tile, wrapped ring
     (65, 70, 128, 10e-6, 3.0, 1e-15, 1),  # a tile of one source
-    (193, 40, 64, 10e-6, 20.0, 1e-15, 2),  # chunks of 97 and 96: a tile and a remainder each
+    (193, 40, 64, 10e-6, 20.0, 1e-15, 2),  # chunks of 98 and 95: a tile and a remainder each
     (130, 0, 8, 10e-6, 3.0, 1e-15, 1),    # the present slot alone
     (150, 30, 64, 1e-6, 3.0, 1e-13, 1),   # c dt = 30 um, pairs down to a few nm: the last segment
 ])
