@@ -240,16 +240,20 @@ emppp_status update_schedule(emppp_handle c) {
     for (int b = 0; b < c->nbunch; b++) t += (c->hb[b].n + 127) / 128;
     return t;
   }();
-  // Chunking of one bunch. Mixed path: about 2 items_per_block items per resident block over all bunches (counted in
-  // 128-target tiles), in whole tiles of TB sources and at least 256 sources (small == false); or, for a system too
-  // small to fill the resident blocks that way, one round of items with short chunks (small == true), since then each
-  // block's time is its own chunk length.
-  // FP64 path: an SM with few blocks left runs below its FP64 rate, and a pair in the history costs twice one beyond
-  // it, so the items are many and short: as many as 2 items_per_block per resident block allow, of at least 8 sources
-  // (below which an item's own set-up shows), or one round if that is more. The step in us by sources per chunk, with
-  // bisection, 512 slots: N = 1024: 12 (one round) 267, 8 277, 4 260; N = 2048: 44 (one round) 770, 32 832, 16 724,
-  // 8 711; N = 4096: 256 2922, 128 2765, 64 2481, 32 2382, 16 2354; N = 8192: 256 9351, 64 8732, 32 8623; N = 16381
-  // with the guess: 256 29434, 64 28638. (The partial sums, 200 MB there, cost less than they save.)
+  // Chunking of one bunch, by sources per chunk. An SM with few blocks left runs below its rate, and a pair in the
+  // history costs more than one beyond it, so the items are many and short: as many as 2 items_per_block items per
+  // resident block over all bunches allow (counted in 128-target tiles), but of at least 8 (FP64) or 32 (mixed)
+  // sources, below which an item's own set-up shows, and on the mixed path at most 128 chunks; or one round of items,
+  // if that is more (a system too small to fill the resident blocks: each block's time is then its own chunk length).
+  // Steps in us by sources per chunk:
+  //   FP64, bisection, 512 slots: N = 1024: 12 (one round) 267, 8 277, 4 260; N = 2048: 44 (one round) 770, 32 832,
+  //   16 724, 8 711; N = 4096: 256 2922, 128 2765, 64 2481, 32 2382, 16 2354; N = 8192: 256 9351, 64 8732, 32 8623;
+  //   N = 16381 with the guess: 256 29434, 64 28638. (The partial sums, 200 MB there, cost less than they save.)
+  //   Mixed, closed form, 251 slots: N = 4096: 256 429, 64 297, 32 288; N = 8192: 256 810, 128 724, 64 700, 32 726;
+  //   N = 16384: 256 2252, 128 2197, 64 2239. 16 bunches of 188 on average: 256 824, 64 652, 32 657.
+  // With the adaptive step the mixed path's chunks are whole tiles of at least 256 sources, or one round: its step
+  // size follows the last bit of FP32 sums, so their grouping stays what it was for runs made so far.
+  const bool whole = mixed && ad;
   auto chunks = [&](long long n, bool small) -> long long {
     const long long one_round = Rreal / total_tiles > 1 ? Rreal / total_tiles : 1;
     const long long many = (2LL * c->items_per_block * Rsched + tiles128 - 1) / tiles128;
@@ -258,17 +262,21 @@ emppp_status update_schedule(emppp_handle c) {
     long long nchunk;
     if (c->opt.source_split > 0)
       nchunk = c->opt.source_split;
-    else if (!mixed)
-      nchunk = std::max(of(one_round, kMin), of(many, 8));
-    else
+    else if (whole)
       nchunk = small ? of(one_round, kMin) : of(many, 256);
+    else
+      nchunk = std::max(of(one_round, kMin), mixed ? of(std::min(many, 128LL), 32) : of(many, 8));
     nchunk = std::max(1LL, std::min(nchunk, (long long)c->ds.max_split));
     const long long chunk = (n + nchunk - 1) / nchunk;
-    const bool tiles = chunk >= TB && (mixed || c->opt.source_split > 0);
-    return tiles ? (chunk + TB - 1) / TB * TB : (chunk + kMin - 1) / kMin * kMin;
+    long long unit = kMin;
+    if ((whole || c->opt.source_split > 0) && chunk >= TB)
+      unit = TB;
+    else if (mixed && !whole && chunk >= 32)
+      unit = 32;  // whole FP32 sums
+    return (chunk + unit - 1) / unit * unit;
   };
   bool small = false;
-  if (mixed) {
+  if (whole) {
     long long items_large = 0;
     for (int b = 0; b < c->nbunch; b++) {
       const long long n = c->hb[b].n;
