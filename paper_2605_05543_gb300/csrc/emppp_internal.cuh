@@ -19,7 +19,7 @@
 //                             w_{k0} + v_{k0} (t_n - t_{k0}) - w_n, the chord w_n - w_{k0} with the
 //                             threshold of the oldest-slot bound, and the FP32 record's beta - beta_ref,
 //                             1/gamma^2 and gamma^2 of slot k0 (kExt* below).
-//   ext64  [N][12] double     per step (FP64 path): the out-of-history line of each source (kExt64).
+//   ext64  [N][12] double     per step: the out-of-history line of each source (kExt64).
 //   u      [N][3]             present proper velocities (FP64).
 //   Eself/Bself [N][3]        self fields of the current step; Bout [N][3] = Bself + B_ext.
 //   ke     [N]                kinetic-energy terms of the energy monitor (small systems, formed by the push).
@@ -137,9 +137,11 @@ enum {
   kExtCount = 5
 };
 
-// doubles per source of ext64 (FP64 path): w_n (3), the line offset w_{k0} + v_{k0} (t_n - t_{k0}) - w_n (3),
-// v_{k0} (3), c^2 - v_{k0}^2, c w_j and c w_j (c^2 - v_{k0}^2)
+// doubles per source of ext64: w_n (3), the line offset w_{k0} + v_{k0} (t_n - t_{k0}) - w_n (3), and on the FP64 path
+// v_{k0} (3), c^2 - v_{k0}^2, c w_j and c w_j (c^2 - v_{k0}^2); on the mixed path v_{k0} / c (3), for sources whose
+// 1/gamma^2 at slot k0 is below kXbGamma alone
 constexpr int kExt64 = 12;
+constexpr float kXbGamma = 0.01f;
 
 struct SlotTables {
   double* lhs64;    // [D] (c (t_n - t_k))^2, formed as c*(t_n - t_k) then squared (no FMA)
@@ -209,7 +211,7 @@ struct DeviceState {
   // w_{k0} + v_{k0} (t_n - t_{k0}) - w_n (where the out-of-history line of eq:linear2 is at t_n), and the
   // oldest slot's chord, bound and velocity (the out-of-history pairs' node test and line)
   float4* ext32;
-  double2* ext64;  // [N][kExt64 / 2] per source and step (FP64 path): the out-of-history line
+  double2* ext64;  // [N][kExt64 / 2] per source and step: the out-of-history line
   // adaptive time step (Sec. 2.4)
   unsigned long long* scale;  // [nbunch][2] bit patterns of eta_min (m, by min) and v_max^2 ((m/s)^2, by max)
   double* adapt_info;         // [3] dt, eta_min, v_max of the last adaptive step
@@ -221,6 +223,13 @@ struct AdaptParams {
   double c_dt, eta_allow, dt_min, dt_max;
 };
 
+// one warp's interaction scale into its bunch's slots
+__device__ __forceinline__ void update_scale(unsigned long long* scale, double emin, double vmax2) {
+  if (emin < __longlong_as_double(0x7ff0000000000000LL))
+    atomicMin(scale, (unsigned long long)__double_as_longlong(emin));
+  if (vmax2 > 0.0) atomicMax(scale + 1, (unsigned long long)__double_as_longlong(vmax2));
+}
+
 // Warp-wide min of eta and max of dv^2, then one atomic per warp into scale. Non-negative doubles order
 // like their bit patterns read as unsigned integers, so the min and max are exact and independent of
 // the order of the pairs. Every lane of the warp must call it.
@@ -230,11 +239,7 @@ __device__ __forceinline__ void reduce_scale(unsigned long long* scale, double e
     emin = fmin(emin, __shfl_xor_sync(0xffffffffu, emin, o));
     vmax2 = fmax(vmax2, __shfl_xor_sync(0xffffffffu, vmax2, o));
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (emin < __longlong_as_double(0x7ff0000000000000LL))
-      atomicMin(scale, (unsigned long long)__double_as_longlong(emin));
-    if (vmax2 > 0.0) atomicMax(scale + 1, (unsigned long long)__double_as_longlong(vmax2));
-  }
+  if ((threadIdx.x & 31) == 0) update_scale(scale, emin, vmax2);
 }
 
 // stage-switch monitor (Sec. 2.7): the criterion, and the per-bunch record the device keeps

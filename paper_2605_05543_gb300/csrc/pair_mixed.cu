@@ -73,7 +73,6 @@ struct MixedArgs {
   const float4* __restrict__ rec32;
   const double* __restrict__ rec64;
   const double* __restrict__ lhs64;
-  const double* __restrict__ slot_t;  // time stamps of the physical slots
   const float4* __restrict__ tab32;  // per slot: upper guard-band threshold of L^2, lo and hi of c (t - t_k), 1 / (c dt_k)
   const double2* __restrict__ tab64;  // per slot: t - t_k, 1 / dt_k
   const float* __restrict__ kq32;  // -e w_j / (4 pi eps0), FP32
@@ -94,6 +93,7 @@ struct MixedArgs {
   const float* __restrict__ fac;  // learned proposal: delay factors [groups][n] per bunch (factor kernel)
   unsigned long long* scale;  // adaptive time step: eta_min / v_max^2 reduction
   float eta_allow;
+  const double2* __restrict__ ext64;  // [N][kExt64 / 2]: lines in FP64 of fast sources
   const float4* __restrict__ ext32;  // [N][kExtCount] per source: segment end hi/lo, out-of-history line, oldest slot
   int* __restrict__ dump;  // [N][N] bracket of every evaluated pair, 4 (k1 - k0) + branch (DUMP instances only)
   int wait_limit;          // probes of a bounded wait on a staged history window (window shapes)
@@ -151,12 +151,35 @@ __device__ __forceinline__ bool exact_test(const double* __restrict__ rr, const 
   return lhs <= rhs;
 }
 
+// (float)x, round to nearest even, on the integer pipe: the 11 exponent bits become 8 (bias 1023 - 127 = 0x380), the
+// significand loses 29 bits. Outside FP32's normal range, the conversion itself.
+__device__ __forceinline__ float rounded_to_float(double x) {
+  const unsigned lo = (unsigned)__double2loint(x), hi = (unsigned)__double2hiint(x), e = hi & 0x7ff00000u;
+  if (e - 0x38100000u >= 0x0fd00000u) return (float)x;
+  unsigned t = __funnelshift_l(lo, hi, 3) - 0xc0000000u;  // exponent and the 23 significand bits that stay
+  if ((lo & 0x1fffffffu) + (t & 1u) > 0x10000000u) t += 1u;
+  return __uint_as_float(t | (hi & 0x80000000u));
+}
+
 // a0 b0 + a1 b1 + a2 b2 and a0 b1 - a1 b0 in a fixed rounding sequence (no compiler contraction)
 __device__ __forceinline__ float dot3(float a0, float a1, float a2, float b0, float b1, float b2) {
   return __fmaf_rn(a2, b2, __fmaf_rn(a1, b1, __fmul_rn(a0, b0)));
 }
 __device__ __forceinline__ float cross1(float a0, float a1, float b0, float b1) {
   return __fmaf_rn(a0, b1, -__fmul_rn(a1, b0));
+}
+
+// whether Heaviside's field of a pair needs X and X.beta from FP64 (why, at its use)
+__device__ __forceinline__ bool needs_fp64_line(float XX, float Xb, float ig2) {
+  return ig2 < kXbGamma && __fmul_rn(kXbGuard, __fmul_rn(sqrtf(XX), fabsf(Xb))) > __fmaf_rn(XX, ig2, __fmul_rn(Xb, Xb));
+}
+
+// X and X.beta of a target at (r0, r1, r2) from the source's line in FP64 (ext64)
+__device__ __forceinline__ float4 fp64_line(const double2* __restrict__ e, double r0, double r1, double r2) {
+  const double2 e0 = __ldg(e), e1 = __ldg(e + 1), e2 = __ldg(e + 2), e3 = __ldg(e + 3), e4 = __ldg(e + 4);
+  const double y0 = (r0 - e0.x) - e1.y, y1 = (r1 - e0.y) - e2.x, y2 = (r2 - e1.x) - e2.y;
+  return make_float4(rounded_to_float(y0), rounded_to_float(y1), rounded_to_float(y2),
+                     rounded_to_float(y0 * e3.x + y1 * e3.y + y2 * e4.x));
 }
 
 // a - (b.x, b.y) by one packed FP32x2 addition of the negation (the same rounding as two subtractions)
@@ -255,6 +278,14 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
   __shared__ float4 s_ck[kTileG];
   __shared__ float s_acc[12][kBlock];  // per-thread compensated sums
 
+  // adaptive step: the targets' present positions in FP64, and per warp the pairs of a group of kSub sources that need
+  // their line in FP64 (lane + 32 source) and what fp64_line gives for them
+  constexpr int kLines = ADAPT ? 64 : 1;
+  __shared__ double s_r[ADAPT ? 3 : 1][ADAPT ? kBlock : 1];
+  __shared__ unsigned char s_pair[kWarps][kLines];
+  __shared__ float4 s_y[kWarps][kLines];
+  static_assert(!ADAPT || kSub <= 8, "a lane's list is eight bits");
+
   __shared__ int s_item;
   // block constants read only when a tile is staged: shared memory instead of registers live across the pairs
   __shared__ float s_inv_cdt;  // 1 / (c dt)
@@ -336,6 +367,11 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
     r.l2 = q1.z;
     r.idx = i;
     r.exact_only = fmaxf(fabsf(r.h01.x), fmaxf(fabsf(r.h01.y), fabsf(r.h2))) > 0.5f;
+    if (ADAPT) {
+      const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
+#pragma unroll
+      for (int c = 0; c < 3; c++) s_r[c][threadIdx.x] = __ldg(rr + c);
+    }
   }
   // learned proposal: the delay factors of this target tile's group (kFacGroup targets, a multiple of the
   // tile), one per source of the bunch
@@ -393,7 +429,12 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
         s_ck[threadIdx.x] = make_float4(2.f * ck.x, 2.f * ck.y, 2.f * ck.z, ck.w);
       }
     }
-    __syncthreads();
+    // (adaptive step) whether any source of the tile is fast enough to need its line in FP64
+    bool fast_sources = false;
+    if (ADAPT)
+      fast_sources = __syncthreads_or(threadIdx.x < tn && s_k0[threadIdx.x].w < kXbGamma);
+    else
+      __syncthreads();
     // window of staged source jn into buffer sb: the offsets lo .. hi + 1 of the guessed brackets [lg, lg + 1]
     // of the warp's lanes that predict one in history, at most kWin slots from lo (one or two contiguous
     // runs of the ring)
@@ -428,6 +469,38 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
     for (int jj0 = 0; jj0 < tn; jj0 += kSub) {
       float P[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       const int jend = min(jj0 + kSub, tn);
+      // Adaptive step (the paper's runs, up to 100 MeV). One pair in eleven needs FP64 at gamma 197, which as a branch
+      // of the pair loop nearly every warp takes with three lanes of 32, and the FP64 pipe then bounds the kernel. So
+      // the pairs of a group that need it are listed first and evaluated with all lanes.
+      unsigned listed = 0;  // bit k: source jj0 + k is in the list; from bit 8: the lane's first entry
+      if (ADAPT && fast_sources) {
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        for (int k = 0; active && k < jend - jj0; k++) {
+          const float4 o = s_k0[jj0 + k], gx = s_x[jj0 + k];
+          const float3 dn = separation(r, s_q0[jj0 + k], s_q1[jj0 + k]);
+          const float X0 = dn.x - gx.x, X1 = dn.y - gx.y, X2 = dn.z - gx.z;
+          const float Xb = dot3(X0, X1, X2, bref01.x + o.x, bref01.y + o.y, bref2 + o.z);
+          if (needs_fp64_line(dot3(X0, X1, X2, X0, X1, X2), Xb, o.w)) listed |= 1u << k;
+        }
+        const int cnt = __popc(listed);
+        int end = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, end, o);
+          if (lane >= o) end += v;
+        }
+        const int total = min(__shfl_sync(0xffffffffu, end, 31), kLines);
+        int at = end - cnt;
+        for (unsigned q = listed; q && at < kLines; q &= q - 1u, at++)
+          s_pair[w][at] = (unsigned char)(lane + 32 * (__ffs(q) - 1));
+        __syncwarp();
+        for (int e = lane; e < total; e += 32) {
+          const int pr = s_pair[w][e], tl = 32 * w + (pr & 31);
+          s_y[w][e] = fp64_line(a.ext64 + (size_t)(tile + jj0 + (pr >> 5)) * (kExt64 / 2), s_r[0][tl], s_r[1][tl], s_r[2][tl]);
+        }
+        __syncwarp();
+        listed |= (unsigned)(end - cnt) << 8;
+      }
       for (int jj = jj0; (WIN || active) && jj < jend; ++jj) {
         const int j = debug_index(tile + jj, boff, boff + bd.n, a.err);
         // history window of this source (WIN): guessed offset, first offset and slots of the staged run
@@ -479,18 +552,19 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
           // denominator relative, at most u gamma. Above 1.3e-6 (only for gamma above ~20, at directions
           // near perpendicular to beta) X and X.beta are formed in FP64 from the FP64 records instead.
           // (as the shift is at most u gamma, sources with gamma^2 < 100 never need it)
-          if (ig2 < 0.01f && __fmul_rn(kXbGuard, __fmul_rn(sqrtf(XX), fabsf(Xb))) > __fmaf_rn(XX, ig2, __fmul_rn(Xb, Xb))) {
-            const double* w0 = src64 + 6 * win.p0;  // FP64 record of slot k0: X = r - w_k0 - v_k0 (t_n - t_k0)
-            const double ct = kC * (a.state->t - __ldg(a.slot_t + win.p0));  // c (t_n - t_k0)
-            const double ic = 1.0 / kC;
-            const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
-            const double y0 = (__ldg(rr + 0) - __ldg(w0 + 0)) - __ldg(w0 + 3) * ic * ct;
-            const double y1 = (__ldg(rr + 1) - __ldg(w0 + 1)) - __ldg(w0 + 4) * ic * ct;
-            const double y2 = (__ldg(rr + 2) - __ldg(w0 + 2)) - __ldg(w0 + 5) * ic * ct;
-            X0 = (float)y0;
-            X1 = (float)y1;
-            X2 = (float)y2;
-            Xb = (float)((y0 * __ldg(w0 + 3) + y1 * __ldg(w0 + 4) + y2 * __ldg(w0 + 5)) * ic);
+          if (needs_fp64_line(XX, Xb, ig2)) {
+            const int k = jj - jj0, at = (int)(listed >> 8) + __popc(listed & ((1u << k) - 1u));
+            float4 y;
+            if (ADAPT && ((listed >> k) & 1u) && at < kLines) {
+              y = s_y[threadIdx.x >> 5][at];
+            } else {
+              const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
+              y = fp64_line(a.ext64 + (size_t)j * (kExt64 / 2), __ldg(rr), __ldg(rr + 1), __ldg(rr + 2));
+            }
+            X0 = y.x;
+            X1 = y.y;
+            X2 = y.z;
+            Xb = y.w;
             XX = dot3(X0, X1, X2, X0, X1, X2);
             count_fallback<kShared>(n_fb);
           }
@@ -992,7 +1066,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
   }
   if (ADAPT) {
     // this item's interaction scale into its bunch's slots (every lane of the warp takes part)
-    reduce_scale(a.scale + 2 * b, (double)emin, (double)vmax2 * (kC * kC));
+    // (reduced as FP32 bits, whose order is that of the values: they are not negative)
+    const float e = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(emin)));
+    const float v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(vmax2)));
+    if ((threadIdx.x & 31) == 0) update_scale(a.scale + 2 * b, (double)e, (double)v * (kC * kC));
     emin = __int_as_float(0x7f800000);
     vmax2 = 0.f;
   }
@@ -1074,7 +1151,6 @@ cudaError_t launch_pair_mixed(const DeviceState& s, const int* order, int propos
   a.rec32 = reinterpret_cast<const float4*>(s.rec32);
   a.rec64 = s.rec64;
   a.lhs64 = s.tab.lhs64;
-  a.slot_t = s.slot_t;
   a.tab32 = s.tab.tab32;
   a.tab64 = s.tab.tab64;
   a.kq32 = s.kq32;
@@ -1095,6 +1171,7 @@ cudaError_t launch_pair_mixed(const DeviceState& s, const int* order, int propos
   a.fac = s.mlp_fac;
   a.scale = s.scale;
   a.eta_allow = (float)ap.eta_allow;
+  a.ext64 = s.ext64;
   a.ext32 = s.ext32;
   a.dump = dump;
   a.wait_limit = pl.wait_limit;

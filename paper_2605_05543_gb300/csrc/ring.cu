@@ -186,6 +186,18 @@ __global__ void prep_kernel(DeviceState s) {
   for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nwin; l += gridDim.x * blockDim.x) slot_table(s, l, p0, nwin, t_n);
 }
 
+// the first ten doubles of a source's ext64: present position, line offset after T0 from slot k0's record r0, and the four
+// values given (the velocity, in units of the path's own, and what follows it)
+__device__ __forceinline__ void write_line(const DeviceState& s, long long j, const double* rn, const double* r0,
+                                           double T0, double e6, double e7, double e8, double e9) {
+  double2* e = s.ext64 + (size_t)j * (kExt64 / 2);
+  e[0] = make_double2(rn[0], rn[1]);
+  e[1] = make_double2(rn[2], fma(r0[3], T0, r0[0] - rn[0]));
+  e[2] = make_double2(fma(r0[4], T0, r0[1] - rn[1]), fma(r0[5], T0, r0[2] - rn[2]));
+  e[3] = make_double2(e6, e7);
+  e[4] = make_double2(e8, e9);
+}
+
 // Per-step set-up, one launch before the pair kernel: the window k0..n and its slot tables (as
 // prep_kernel), the pair kernel's work counter, and, for the mixed path, per-source vectors (eq:linear at
 // t_n):
@@ -228,16 +240,14 @@ __global__ void setup_kernel(DeviceState s, SetupExt extrap) {
     const double v0 = r0[3], v1 = r0[4], v2 = r0[5];
     const double C2 = fma(-v0, v0, fma(-v1, v1, fma(-v2, v2, kC * kC)));
     const double cw = kC * s.wts[j];
-    double2* e = s.ext64 + (size_t)j * (kExt64 / 2);
-    e[0] = make_double2(rn[0], rn[1]);
-    e[1] = make_double2(rn[2], fma(v0, T0, r0[0] - rn[0]));
-    e[2] = make_double2(fma(v1, T0, r0[1] - rn[1]), fma(v2, T0, r0[2] - rn[2]));
-    e[3] = make_double2(v0, v1);
-    e[4] = make_double2(v2, C2);
-    e[5] = make_double2(cw, cw * C2);
+    write_line(s, j, rn, r0, T0, v0, v1, v2, C2);
+    s.ext64[(size_t)j * (kExt64 / 2) + 5] = make_double2(cw, cw * C2);
     return;
   }
   const float* q0 = s.rec32 + ((size_t)j * s.D + p0) * 12;  // FP32 record of slot k0
+  // fast sources: the mixed kernel may need their line in FP64 (kXbGuard)
+  if (q0[3] < kXbGamma)
+    write_line(s, j, rn, r0, t_n - s.slot_t[p0], r0[3] * (1.0 / kC), r0[4] * (1.0 / kC), r0[5] * (1.0 / kC), 0.0);
   float4* ext = s.ext32 + (size_t)j * kExtCount;
   const double dt0 = s.slot_t[pn] - s.slot_t[p0];
   ext[kExtLine] = make_float4((float)((r0[0] + r0[3] * dt0) - rn[0]), (float)((r0[1] + r0[4] * dt0) - rn[1]),
