@@ -54,6 +54,8 @@ struct NvtxRange {
 };
 }  // namespace
 
+constexpr int kGraphs = 4;  // a step's graphs: with and without the target order, with and without the set-up launch
+
 struct emppp_ctx {
   DeviceState ds{};
   int64_t N = 0;
@@ -118,17 +120,20 @@ struct emppp_ctx {
   int ev_used = 0;
   // one step captured in two variants, replayed by emppp_step: [1] recomputes the spatial target order,
   // [0] reuses the last one
-  cudaGraph_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
-  int graph_launches[2] = {0, 0};  // kernels per replayed step
+  cudaGraph_t graph[kGraphs] = {};
+  cudaGraphExec_t graph_exec[kGraphs] = {};
+  int graph_launches[kGraphs] = {};  // kernels per replayed step
   unsigned char graph_key[sizeof(emppp_options) + sizeof(BextParams) + sizeof(AdaptParams) +
-                          sizeof(EnergyParams)];  // configuration of both variants
-  bool graph_valid[2] = {false, false};
+                          sizeof(EnergyParams)];  // configuration of the variants
+  bool graph_valid[kGraphs] = {};
   // Steps since the target order was computed (-1: not for the present state). The order is a
   // permutation of each bunch whatever its age, and a target's sum runs over the sources in a fixed
   // order whichever thread evaluates it, so an older order changes no result; it is recomputed every
   // kOrderEvery steps, since a bunch's particles move far less than their spacing in that time.
   int order_age = -1;
+  // the path whose slot tables and source vectors the last step's post-pair launch formed for the present state (none:
+  // the next step starts with its own set-up launch); every other call that touches the state or these resets it
+  SetupExt prepared = SetupExt::none;
 };
 
 // steps between two computations of the spatial target order
@@ -182,7 +187,7 @@ emppp_status validate_options(const emppp_options* o) {
 }
 
 void invalidate_graph(emppp_handle h) {
-  for (int v = 0; v < 2; v++) {
+  for (int v = 0; v < kGraphs; v++) {
     if (h->graph_exec[v]) cudaGraphExecDestroy(h->graph_exec[v]);
     if (h->graph[v]) cudaGraphDestroy(h->graph[v]);
     h->graph_exec[v] = nullptr;
@@ -190,6 +195,7 @@ void invalidate_graph(emppp_handle h) {
     h->graph_valid[v] = false;
   }
   h->order_age = -1;  // every change of state or configuration recomputes the order at the next step
+  h->prepared = SetupExt::none;
 }
 
 // Work split of the persistent pair kernel, per bunch: one block per resident slot of the kernel that
@@ -381,6 +387,7 @@ emppp_status from_device(emppp_handle h, double* dst, const double* src, size_t 
 // the bunch's first particle when the state is set. x and v_or_u index the present positions and
 // velocities (or proper velocities). Device arrays are read with one wait, which also serves what the caller enqueued.
 emppp_status set_bunch_frames(emppp_handle h, const double* x, const double* v_or_u, bool is_u, int is_dev) {
+  h->prepared = SetupExt::none;
   double* f = h->frames;
   for (int b = 0; b < h->nbunch; b++) {
     const long long i = h->hb[b].off;
@@ -435,9 +442,19 @@ emppp_status convert_bext(const emppp_bext* bext, BextParams* bp) {
   return EMPPP_OK;
 }
 
+// the path whose vectors a step needs, and whether its post-pair launch forms them for the step after it
+SetupExt setup_of(emppp_handle h) {
+  if (!h->opt.pair_fields) return SetupExt::none;
+  return h->opt.precision == EMPPP_MIXED ? SetupExt::mixed : SetupExt::fp64;
+}
+SetupExt next_setup_of(emppp_handle h) {
+  return h->opt.field_point == EMPPP_FIELD_HALF_STEP ? SetupExt::none : setup_of(h);
+}
+
 // enqueues the kernels of one step and reports how many kernels it launched; refresh_order recomputes the
-// spatial target order first (else the last one is used)
-emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev, int* nkernels, bool refresh_order) {
+// spatial target order first (else the last one is used), set_up launches the set-up (else the step before formed it)
+emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev, int* nkernels, bool refresh_order,
+                          bool set_up) {
   int k = 0;
   if (ev) CU(cudaEventRecord(ev[0], h->stream));
   const bool half = h->opt.pair_fields && h->opt.field_point == EMPPP_FIELD_HALF_STEP;
@@ -461,9 +478,10 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
       CU(cudaEventRecord(h->ev_join, h->aux));
       k += 1;
     }
-    CU(launch_setup(h->ds,
-                    !h->opt.pair_fields ? SetupExt::none : (mixed_pairs ? SetupExt::mixed : SetupExt::fp64), h->stream));
-    k += 1;
+    if (set_up) {
+      CU(launch_setup(h->ds, setup_of(h), h->stream));
+      k += 1;
+    }
   }
   if (ordered && refresh_order) CU(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
   if (ev) CU(cudaEventRecord(ev[1], h->stream));
@@ -491,7 +509,7 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
   // launch evaluates the bunches in parallel, one block each)
   const bool fused_energy = h->energy.on && h->N <= 16384 && h->nbunch <= 8;
   NvtxRange r_post("emppp:push_append");
-  CU(launch_step_post(h->ds, bp, h->adapt, chunked, half, fused_energy ? &h->energy : nullptr, h->d_mon, h->stream));
+  CU(launch_step_post(h->ds, bp, h->adapt, chunked, half, next_setup_of(h), fused_energy ? &h->energy : nullptr, h->d_mon, h->stream));
   k += 1;
   if (h->energy.on && !fused_energy) {
     // mean energy of the new state and the switch criterion (Sec. 2.7)
@@ -504,9 +522,11 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
 }
 
 // captures one step into a CUDA graph for the current configuration (options and background field), in the
-// variant that recomputes the target order (refresh_order) or the one that reuses it
-emppp_status capture_step(emppp_handle h, const BextParams& bp, bool refresh_order) {
-  const int v = refresh_order ? 1 : 0;
+// variant that recomputes the target order (refresh_order) or reuses it, with the set-up launch (set_up) or without
+int graph_variant(bool refresh_order, bool set_up) { return (refresh_order ? 1 : 0) + (set_up ? 2 : 0); }
+
+emppp_status capture_step(emppp_handle h, const BextParams& bp, bool refresh_order, bool set_up) {
+  const int v = graph_variant(refresh_order, set_up);
   unsigned char key[sizeof(emppp_options) + sizeof(BextParams) + sizeof(AdaptParams) + sizeof(EnergyParams)];
   memset(key, 0, sizeof(key));
   memcpy(key, &h->opt, sizeof(emppp_options));
@@ -522,7 +542,7 @@ emppp_status capture_step(emppp_handle h, const BextParams& bp, bool refresh_ord
   if (h->graph_valid[v]) return EMPPP_OK;
   CU(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   int k = 0;
-  emppp_status st = enqueue_step(h, bp, nullptr, &k, refresh_order);
+  emppp_status st = enqueue_step(h, bp, nullptr, &k, refresh_order, set_up);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(h->stream, &g);
   if (st != EMPPP_OK) {
@@ -793,6 +813,7 @@ EMPPP_API emppp_status emppp_set_particles(emppp_handle h, const double* x, cons
   h->hist_start = 0;
   h->has_state = true;
   h->order_age = -1;  // a new state: the next step recomputes the target order
+  h->prepared = SetupExt::none;
   return EMPPP_OK;
 }
 
@@ -865,6 +886,7 @@ EMPPP_API emppp_status emppp_set_history(emppp_handle h, int64_t n, int32_t nslo
   h->hist_start = hs;
   h->has_state = true;
   h->order_age = -1;  // a new state: the next step recomputes the target order
+  h->prepared = SetupExt::none;
   return EMPPP_OK;
 }
 
@@ -923,23 +945,29 @@ EMPPP_API emppp_status emppp_step(emppp_handle h, int64_t nsteps, const emppp_be
   if ((st = update_schedule(h)) != EMPPP_OK) return st;
   const bool use_graph = h->opt.graphs && !h->opt.timing && h->stream != nullptr && nsteps > 1;
   NvtxRange r_step(use_graph ? "emppp_step (graph replay)" : "emppp_step");
+  // in a capture of the caller's own the step may be replayed from any state: it carries its set-up launch
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool captured = cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
   long long pairs_per_step = 0;
   if (h->opt.pair_fields)
     for (int b = 0; b < h->nbunch; b++) pairs_per_step += (long long)h->hb[b].n * (h->hb[b].n - 1);
   for (int64_t k = 0; k < nsteps; k++) {
     int nk = 0;
     const bool refresh = h->order_age < 0 || h->order_age >= kOrderEvery - 1;
+    const bool set_up = captured || h->prepared == SetupExt::none || h->prepared != setup_of(h);
+    h->prepared = SetupExt::none;  // also if this step fails
     if (use_graph) {
-      if ((st = capture_step(h, bp, refresh)) != EMPPP_OK) return st;
-      const int v = refresh ? 1 : 0;
+      if ((st = capture_step(h, bp, refresh, set_up)) != EMPPP_OK) return st;
+      const int v = graph_variant(refresh, set_up);
       CU(cudaGraphLaunch(h->graph_exec[v], h->stream));
       nk = h->graph_launches[v];
     } else {
       cudaEvent_t* ev = nullptr;
       if (h->opt.timing && h->ev_used < emppp_ctx::kTimedSteps) ev = &h->events[4 * h->ev_used++];
-      if ((st = enqueue_step(h, bp, ev, &nk, refresh)) != EMPPP_OK) return st;
+      if ((st = enqueue_step(h, bp, ev, &nk, refresh, set_up)) != EMPPP_OK) return st;
     }
     h->order_age = refresh ? 0 : h->order_age + 1;
+    if (!captured) h->prepared = next_setup_of(h);
     h->launches += nk;
     h->pairs_acc += pairs_per_step;
     h->steps_acc += 1;
@@ -959,6 +987,7 @@ EMPPP_API emppp_status emppp_handoff(emppp_handle h, const double* center) {
   if (!center) return fail(EMPPP_ERR_ARG, "center is NULL");
   if ((st = read_err(h)) != EMPPP_OK) return st;
   CU(launch_bunch_sums(h->ds, h->stream));
+  h->prepared = SetupExt::none;
   std::vector<double> sums((size_t)h->nbunch * 4);
   CU(cudaMemcpyAsync(sums.data(), h->ds.bsum, sizeof(double) * sums.size(), cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
@@ -990,6 +1019,7 @@ EMPPP_API emppp_status emppp_transport(emppp_handle h, int64_t nsteps, double dt
   BextParams bp;
   if ((st = convert_bext(bext, &bp)) != EMPPP_OK) return st;
   if ((st = sync_time(h)) != EMPPP_OK) return st;
+  h->prepared = SetupExt::none;
   const int64_t kChunk = 4096;
   for (int64_t done = 0; done < nsteps;) {
     const int k = (int)(nsteps - done < kChunk ? nsteps - done : kChunk);
@@ -1090,6 +1120,7 @@ EMPPP_API emppp_status emppp_reset_stats(emppp_handle h) {
 // one evaluation of the self fields of the present state: slot tables, target order, pair kernel,
 // reduction (no push: the state does not change)
 emppp_status enqueue_fields(emppp_handle h, int* dump = nullptr) {
+  h->prepared = SetupExt::none;  // the pair kernel's work counter is spent
   CU(launch_setup(h->ds, h->opt.precision == EMPPP_MIXED ? SetupExt::mixed : SetupExt::fp64, h->stream));
   const bool ordered = h->target_order != 0;
   if (ordered) CU(launch_target_order(h->ds, h->ord_key, h->order, h->max_bunch, h->stream));
@@ -1294,6 +1325,7 @@ EMPPP_API emppp_status emppp_sample_delays(emppp_handle h, const int32_t* pairs,
     dd = delays;
     dz = targets;
   }
+  h->prepared = SetupExt::none;
   cudaError_t e = launch_prep(h->ds, h->stream);
   if (e == cudaSuccess)
     e = launch_sample(h->ds, pp, m, static_cast<float*>(df), static_cast<double*>(dd), static_cast<float*>(dz),
@@ -1590,6 +1622,7 @@ EMPPP_API emppp_status emppp_set_options(emppp_handle h, const emppp_options* op
   if (h->adapt.on && is_variant(*opt))
     return fail(EMPPP_ERR_STATE, "the midpoint reconstruction and the half-step field point run with a fixed dt");
   h->opt = *opt;
+  h->prepared = SetupExt::none;
   if ((st = ensure_events(h)) != EMPPP_OK) return st;
   return update_schedule(h);
 }

@@ -338,7 +338,7 @@ cudaError_t launch_pair_fp64(const DeviceState& s, const int* order, int proposa
 cudaError_t launch_zero_self(const DeviceState& s, cudaStream_t st);
 // push.cu
 cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked,
-                             bool half, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st);
+                             bool half, SetupExt next, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st);
 cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_half_slot(const DeviceState& s, cudaStream_t st);
 // stage2.cu

@@ -15,6 +15,7 @@
 #include "energy.cuh"
 #include "fp64_roots.cuh"
 #include "push_math.cuh"
+#include "setup.cuh"
 #include "shadow.cuh"
 
 namespace emppp {
@@ -192,12 +193,15 @@ cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st) {
 // fields, the adaptive step size, the push of every particle and the append of slot
 // n+1, then (by the last block to finish) the clock advance n -> n+1, t -> t + dt and the reset of the
 // interaction-scale reduction. The last block is found with a counter that every block increments once
-// after its work; nothing waits on it. With half = 1 (half-step field point) the clock already stands at
+// after its work; nothing waits on it. With next it also forms what the pair kernel of the next step needs (setup.cuh),
+// so that step goes without its set-up launch (6 us and a gap between launches, of 43 us a step with the paper's 400
+// macroparticles): the slot tables need the step size alone and are formed by the warps that sum no chunks while others
+// push, the source vectors by a warp whose loads are there by then. With half = 1 (half-step field point) the clock already stands at
 // the provisional slot n+1: the push starts from slot n, the provisional slot is overwritten and the
 // clock moves from t_n + dt/2 to t_n + dt (formed from t_n, as without the variant).
 template <int P>
 __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s, BextParams bp, AdaptParams ap,
-                                                                   int chunked, int half, EnergyParams ep,
+                                                                   int chunked, int half, SetupExt next, EnergyParams ep,
                                                                    EnergyMon* __restrict__ mon) {
   __shared__ ChunkSums<P> sums;
   __shared__ double s_step[3];
@@ -222,11 +226,30 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
       u[c] = s.u[3 * i + c];
     }
   }
+  const int task = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long it = i0 + lane;
+  // the next step's window (fixed here: half and next exclude one another)
+  const bool slides = st.n + 1 - s.D + 1 > st.k0;
+  const long long k0_next = slides ? st.k0 + 1 : st.k0;
+  const int p0_next = !slides ? st.p0 : (st.p0 + 1 == s.D ? 0 : st.p0 + 1);
+  const bool sets_up = next != SetupExt::none && task == 3 && lane < P && it < s.N;
+  Oldest old;
+  double t_old = 0.0;
+  if (sets_up) {
+    old.load(s, next, it, p0_next);
+    t_old = s.slot_t[p0_next];
+  }
   if (chunked)
     sums.run(s, i0);
   else if (ap.on)
     __syncthreads();  // s_step
   const double dt = ap.on ? s_step[0] : st.dt;
+  if (next != SetupExt::none && threadIdx.x >= kSumThreads) {
+    constexpr int kTableThreads = kEnergyThreads - kSumThreads;
+    const int nwin = (int)(st.n + 1 - k0_next) + 1;
+    for (int l = blockIdx.x * kTableThreads + (int)threadIdx.x - kSumThreads; l < nwin; l += gridDim.x * kTableThreads)
+      slot_table(s, l, p0_next, pnext, nwin, t_n + dt);
+  }
   if (i == 0) {
     s.slot_t[pnext] = t_n + dt;
     if (ap.on) {
@@ -275,10 +298,16 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
     vn[2] = v[2];
   }
   __syncthreads();
-  // What follows from the pushed state, by a warp each: the FP32 record, the monitor's term, and how far slot n + 1
-  // lies from slot n's line (newer-node bound of the mixed path)
-  const int task = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long it = i0 + lane;
+  // What follows from the pushed state, by a warp each: the FP32 record, the monitor's term, how far slot n + 1 lies from
+  // slot n's line (newer-node bound of the mixed path), and the next step's source vectors
+  if (sets_up) {
+    const double* o = s_new[lane];
+    const double T0 = (t_n + dt) - t_old;
+    if (next == SetupExt::fp64)
+      source_vectors_fp64(s, it, o, old, T0);
+    else
+      source_vectors_mixed(s, it, o, old, T0, o + 6, (t_n + dt) - t_n);
+  }
   if (task < 3 && lane < P && it < s.N) {
     const double* o = s_new[lane];
     if (task == 0) {
@@ -310,6 +339,12 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
       s.state->n = half ? st.n : st.n + 1;
       s.state->t = t_n + dt;
       s.state->dt = dt;
+      if (next != SetupExt::none) {
+        s.state->k0 = k0_next;
+        s.state->p0 = p0_next;
+        s.state->pn = pnext;
+        *s.work = 0;
+      }
       if (ap.on) {
         for (int b = 0; b < s.nbunch; b++) {
           s.scale[2 * b] = (unsigned long long)0x7ff0000000000000ULL;  // +inf
@@ -328,18 +363,18 @@ __global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s
 }
 
 cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked,
-                             bool half, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st) {
+                             bool half, SetupExt next, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st) {
   EnergyParams e{0, 1, 0.0};
   if (ep) e = *ep;  // the energy monitor in the last block (small systems)
   const int p = post_particles(s.N);
   const unsigned blocks = (unsigned)((s.N + p - 1) / p);
   const int c = chunked ? 1 : 0, h = half ? 1 : 0;
   if (p == 8)
-    step_post_kernel<8><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, e, mon);
+    step_post_kernel<8><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, e, mon);
   else if (p == 16)
-    step_post_kernel<16><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, e, mon);
+    step_post_kernel<16><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, e, mon);
   else
-    step_post_kernel<32><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, e, mon);
+    step_post_kernel<32><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, e, mon);
   return cudaGetLastError();
 }
 

@@ -2,6 +2,7 @@
 // stored) and per-step slot tables.
 #include "emppp_internal.cuh"
 #include "fp64_roots.cuh"
+#include "setup.cuh"
 #include "shadow.cuh"
 
 namespace emppp {
@@ -140,35 +141,6 @@ __global__ void set_state_kernel(DeviceState s, long long n, double t, double dt
   s.kq32[i] = (float)(-kQe * s.wts[i] / (4.0 * kPi * kEps0));
 }
 
-// Slot-table entry of window offset l (slot p0 + l, modulo D) at time t_n (Sec. 2.2): the squared
-// light-travel distance (c (t_n - t_k))^2 in exactly the operation order of the reference evaluation
-// (so that the FP64 node test decides identically), its upper guard-band threshold in FP32, c (t_n - t_k) in
-// FP32 hi and lo, t_n - t_k and 1 / (t_{k+1} - t_k).
-constexpr double kGuardHi = (1.0 + kGuardBand) / (1.0 - kGuardBand);
-
-// FP32 upper threshold of a slot's (c (t_n - t_k))^2 (the node test is true above it)
-__device__ __forceinline__ float upper_threshold(double lhs) { return __double2float_ru(lhs * kGuardHi); }
-
-__device__ __forceinline__ void slot_table(const DeviceState& s, int l, int p0, int nwin, double t_n) {
-  int p = p0 + l;
-  if (p >= s.D) p -= s.D;
-  const double tk = s.slot_t[p];
-  const double ct = __dmul_rn(kC, __dsub_rn(t_n, tk));
-  const double lhs = __dmul_rn(ct, ct);
-  s.tab.lhs64[p] = lhs;
-  float icdt = 0.f;
-  if (l + 1 < nwin) {
-    int q = p + 1 == s.D ? 0 : p + 1;
-    const double dtk = s.slot_t[q] - tk;
-    const double idt = recip_refined(dtk);
-    s.tab.tab64[p] = make_double2(t_n - tk, idt);
-    icdt = (float)(idt * (1.0 / kC));
-  } else {
-    s.tab.tab64[p] = make_double2(t_n - tk, 0.0);
-  }
-  s.tab.tab32[p] = make_float4(upper_threshold(lhs), (float)(ct - (double)(float)ct), (float)ct, icdt);
-}
-
 // Per-step slot tables over the usable window k0..n alone (used before the delay sampler).
 __global__ void prep_kernel(DeviceState s) {
   const long long n = s.state->n;
@@ -183,22 +155,10 @@ __global__ void prep_kernel(DeviceState s) {
     s.state->pn = pn;
   }
   const int nwin = (int)(n - k0 + 1);
-  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nwin; l += gridDim.x * blockDim.x) slot_table(s, l, p0, nwin, t_n);
+  for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nwin; l += gridDim.x * blockDim.x) slot_table(s, l, p0, pn, nwin, t_n);
 }
 
-// the first ten doubles of a source's ext64: present position, line offset after T0 from slot k0's record r0, and the four
-// values given (the velocity, in units of the path's own, and what follows it)
-__device__ __forceinline__ void write_line(const DeviceState& s, long long j, const double* rn, const double* r0,
-                                           double T0, double e6, double e7, double e8, double e9) {
-  double2* e = s.ext64 + (size_t)j * (kExt64 / 2);
-  e[0] = make_double2(rn[0], rn[1]);
-  e[1] = make_double2(rn[2], fma(r0[3], T0, r0[0] - rn[0]));
-  e[2] = make_double2(fma(r0[4], T0, r0[1] - rn[1]), fma(r0[5], T0, r0[2] - rn[2]));
-  e[3] = make_double2(e6, e7);
-  e[4] = make_double2(e8, e9);
-}
-
-// Per-step set-up, one launch before the pair kernel: the window k0..n and its slot tables (as
+// Set-up of the pair kernel, for a step that the post-pair launch of the step before did not prepare: the window k0..n and its slot tables (as
 // prep_kernel), the pair kernel's work counter, and, for the mixed path, per-source vectors (eq:linear at
 // t_n):
 //   P_j = w_{j,n-1} + v_{j,n-1} (t_n - t_{n-1}), the end of the last history segment, split hi/lo about
@@ -230,48 +190,19 @@ __global__ void setup_kernel(DeviceState s, SetupExt extrap) {
     *s.work = 0;
   }
   const int nwin = (int)(n - k0 + 1);
-  if (gid < nwin) slot_table(s, (int)gid, p0, nwin, t_n);
+  if (gid < nwin) slot_table(s, (int)gid, p0, pn, nwin, t_n);
   if (extrap == SetupExt::none || gid >= s.N) return;
-  const long long j = gid;
-  const double* rn = s.rec64 + ((size_t)j * s.D + pn) * 6;
-  const double* r0 = s.rec64 + ((size_t)j * s.D + p0) * 6;
+  const double* x = s.rec64 + ((size_t)gid * s.D + pn) * 6;
+  const double T0 = t_n - s.slot_t[p0];
+  Oldest o;
+  o.load(s, extrap, gid, p0);
   if (extrap == SetupExt::fp64) {
-    const double T0 = t_n - s.slot_t[p0];
-    const double v0 = r0[3], v1 = r0[4], v2 = r0[5];
-    const double C2 = fma(-v0, v0, fma(-v1, v1, fma(-v2, v2, kC * kC)));
-    const double cw = kC * s.wts[j];
-    write_line(s, j, rn, r0, T0, v0, v1, v2, C2);
-    s.ext64[(size_t)j * (kExt64 / 2) + 5] = make_double2(cw, cw * C2);
+    source_vectors_fp64(s, gid, x, o, T0);
     return;
   }
-  const float* q0 = s.rec32 + ((size_t)j * s.D + p0) * 12;  // FP32 record of slot k0
-  // fast sources: the mixed kernel may need their line in FP64 (kXbGuard)
-  if (q0[3] < kXbGamma)
-    write_line(s, j, rn, r0, t_n - s.slot_t[p0], r0[3] * (1.0 / kC), r0[4] * (1.0 / kC), r0[5] * (1.0 / kC), 0.0);
-  float4* ext = s.ext32 + (size_t)j * kExtCount;
-  const double dt0 = s.slot_t[pn] - s.slot_t[p0];
-  ext[kExtLine] = make_float4((float)((r0[0] + r0[3] * dt0) - rn[0]), (float)((r0[1] + r0[4] * dt0) - rn[1]),
-                              (float)((r0[2] + r0[5] * dt0) - rn[2]), q0[11]);
-  ext[kExtOldest] = make_float4(q0[8], q0[9], q0[10], q0[3]);
-  {
-    const double c0 = rn[0] - r0[0], c1 = rn[1] - r0[1], c2 = rn[2] - r0[2];
-    const double ct = __dmul_rn(kC, __dsub_rn(t_n, s.slot_t[p0]));
-    const double cc = c0 * c0 + c1 * c1 + c2 * c2;
-    const double rhs = (double)upper_threshold(__dmul_rn(ct, ct)) * (1.0 + kChordMargin) - cc * (1.0 - kChordMargin);
-    const float inf = __int_as_float(0x7f800000);
-    ext[kExtChord] = make_float4((float)c0, (float)c1, (float)c2, n > k0 ? fmaxf(__double2float_ru(rhs), 0.f) : inf);
-  }
-  if (n <= k0) return;  // no segment [n-1, n] in the window
   const int p1 = pn == 0 ? s.D - 1 : pn - 1;
-  const double dtl = s.slot_t[pn] - s.slot_t[p1];
-  const double* r = s.rec64 + ((size_t)j * s.D + p1) * 6;
-  const BunchDesc& bd = s.bunches[s.bunch_of[j]];
-  const double d0 = (r[0] + r[3] * dtl) - bd.origin[0];
-  const double d1 = (r[1] + r[4] * dtl) - bd.origin[1];
-  const double d2 = (r[2] + r[5] * dtl) - bd.origin[2];
-  const float h0 = (float)d0, h1 = (float)d1, h2 = (float)d2;
-  ext[kExtSegHi] = make_float4(h0, h1, h2, 0.f);
-  ext[kExtSegLo] = make_float4((float)(d0 - (double)h0), (float)(d1 - (double)h1), (float)(d2 - (double)h2), 0.f);
+  source_vectors_mixed(s, gid, x, o, T0, n > k0 ? s.rec64 + ((size_t)gid * s.D + p1) * 6 : nullptr,
+                       t_n - s.slot_t[p1]);
 }
 
 __global__ void reset_scale_kernel(DeviceState s) {
