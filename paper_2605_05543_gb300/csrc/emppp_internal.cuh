@@ -350,7 +350,7 @@ cudaError_t launch_transport_chunk(const DeviceState& s, const BextParams& b, do
 cudaError_t prepare_target_order();
 cudaError_t launch_target_order(const DeviceState& s, unsigned* key, int* order, long long max_bunch, cudaStream_t st);
 // spatial order of n positions x [n][3] (key, order [n])
-cudaError_t launch_array_order(const double* x, int n, unsigned* key, int* order, cudaStream_t st);
+cudaError_t launch_array_order(const double* x, const double* v, int n, unsigned* key, int* order, cudaStream_t st);
 // mlp.cu
 size_t mlp_image_bytes();
 cudaError_t launch_build_image(const float* params, void* image, cudaStream_t st);

@@ -362,7 +362,7 @@ extern "C" EMPPP_API emppp_status emppp_fields_noalloc(int64_t n, int32_t nslots
   // 87 with; n = 1000: 272 without, 266 with)
   const bool ordered = n > kMinOrdered;
   if (ordered) {
-    e = launch_array_order(W + (size_t)(nslots - 1) * n * 3, (int)n, key, order, s);
+    e = launch_array_order(W + (size_t)(nslots - 1) * n * 3, V + (size_t)(nslots - 1) * n * 3, (int)n, key, order, s);
     if (e != cudaSuccess) {
       set_error_text(cudaGetErrorString(e));
       return EMPPP_ERR_CUDA;
