@@ -347,9 +347,9 @@ cudaError_t launch_translate(const DeviceState& s, const double* shifts, cudaStr
 cudaError_t launch_transport_chunk(const DeviceState& s, const BextParams& b, double dt, int nsteps, double t_end,
                                    cudaStream_t st);
 // order.cu
-cudaError_t prepare_target_order();
 cudaError_t launch_target_order(const DeviceState& s, unsigned* key, int* order, long long max_bunch, cudaStream_t st);
-// spatial order of n positions x [n][3] (key, order [n])
+// spatial order of n positions x [n][3] with velocities v (key, order [n])
+cudaError_t load_array_order();
 cudaError_t launch_array_order(const double* x, const double* v, int n, unsigned* key, int* order, cudaStream_t st);
 // mlp.cu
 size_t mlp_image_bytes();

@@ -294,7 +294,7 @@ emppp_status scratch_address(int dev, void** out) {
       set_error_text(cudaGetErrorString(e));
       return EMPPP_ERR_CUDA;
     }
-    e = prepare_target_order();
+    e = load_array_order();
     if (e != cudaSuccess) {
       set_error_text(cudaGetErrorString(e));
       return EMPPP_ERR_CUDA;

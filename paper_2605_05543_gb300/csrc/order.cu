@@ -7,10 +7,13 @@
 // The delay of a source changes 1 + beta times as fast along the bunch's motion as across it, so that axis is
 // stretched. (Branches that a warp takes for a source, N = 4096, 512 slots: 0.79 in history and 0.45 beyond with a
 // Morton curve of the leading bits alone, 0.75 and 0.42 now; the FP64 step there 2.36 -> 2.22 ms, N = 16381 28.9 ->
-// 27.6.) One block of 1024 threads sorts one bunch in shared memory: latency-bound, and rarely run. The order is a
-// permutation of each bunch's index range (each target is evaluated exactly once whatever the order); the order inside
-// a cell comes from shared-memory atomics and may differ run to run, which changes which thread evaluates a target but
-// not its result.
+// 27.6.) A bunch of more than 2048 particles is sorted by a cluster of eight blocks, each of which holds the
+// counts of an eighth of the cells, a smaller one by one block: latency and the shared-memory sort bound it (N = 8192:
+// 85 us with one block, 32 with eight; 65536: 697 and 100). The order is a permutation of each bunch's index range
+// (each target is evaluated exactly once whatever the order); the order inside a cell comes from shared-memory atomics
+// and may differ run to run, which changes which thread evaluates a target but not its result.
+#include <cooperative_groups.h>
+
 #include "emppp_internal.cuh"
 
 namespace emppp {
@@ -23,6 +26,10 @@ constexpr int kUnroll = 4;  // particles whose positions a thread loads before i
 
 constexpr int kKeyBits = 10;     // per axis
 constexpr int kWindow = 2048;    // particles sorted by the whole key at a time
+constexpr int kCluster = 8;      // blocks of a bunch of more than kWindow particles
+constexpr int kCells = 4096;     // cell counts of a block
+static_assert((1 << (3 * kMaxBits)) <= kCluster * kCells && kCells * sizeof(int) == kWindow * sizeof(unsigned long long),
+              "the cells of a bunch fit its blocks, and a window the place of a block's counts");
 
 // index along the Hilbert curve of a cell (Skilling's transform of the axes, AIP Conf. Proc. 707, 381, 2004)
 __device__ __forceinline__ unsigned hilbert_index(unsigned x, unsigned y, unsigned z) {
@@ -65,14 +72,15 @@ __host__ __device__ __forceinline__ int cell_bits(int n) {
 struct RingPositions {  // present positions of a solver's bunches (hi parts about their origins)
   DeviceState s;
   const float4* rec;
-  int pn;
-  __device__ __forceinline__ void begin() {
+  int pn, bunch;
+  __device__ __forceinline__ void begin(int b) {
+    bunch = b;
     rec = reinterpret_cast<const float4*>(s.rec32);
     pn = (int)(s.state->n % s.D);
   }
-  __device__ __forceinline__ int count() const { return s.bunches[blockIdx.x].n; }
-  __device__ __forceinline__ long long offset() const { return s.bunches[blockIdx.x].off; }
-  __device__ __forceinline__ float stretch(int c) const { return 1.f + fabsf((float)s.bunches[blockIdx.x].beta_ref[c]); }
+  __device__ __forceinline__ int count() const { return s.bunches[bunch].n; }
+  __device__ __forceinline__ long long offset() const { return s.bunches[bunch].off; }
+  __device__ __forceinline__ float stretch(int c) const { return 1.f + fabsf((float)s.bunches[bunch].beta_ref[c]); }
   // one record per particle's ring run, so every particle is its own cache line
   __device__ __forceinline__ float4 at(long long k) const { return __ldg(rec + ((size_t)k * s.D + pn) * 3); }
 };
@@ -80,7 +88,7 @@ struct ArrayPositions {  // x [n][3], about the first particle; v: its velocity
   const double* x;
   const double* v;
   int n;
-  __device__ __forceinline__ void begin() {}
+  __device__ __forceinline__ void begin(int) {}
   __device__ __forceinline__ int count() const { return n; }
   __device__ __forceinline__ long long offset() const { return 0; }
   __device__ __forceinline__ float stretch(int c) const { return 1.f + fabsf((float)(__ldg(v + c) * (1.0 / kC))); }
@@ -91,23 +99,28 @@ struct ArrayPositions {  // x [n][3], about the first particle; v: its velocity
 };
 
 template <class Positions>
-__global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsigned* __restrict__ key,
-                                                         int* __restrict__ order) {
-  extern __shared__ __align__(16) int hist[];  // cell counts, then the window being sorted
-  __shared__ float s_lo[3][32], s_hi[3][32];
-  __shared__ int s_warp[32];
-  where.begin();
+__global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsigned* key, int* order) {
+  __shared__ __align__(16) unsigned long long win[kWindow];  // the window being sorted; before that, cell counts
+  int* hist = reinterpret_cast<int*>(win);
+  __shared__ float s_lo[3][32], s_hi[3][32], s_box[6];
+  __shared__ int s_warp[32], s_total;
+  const cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int rank = (int)cl.block_rank(), nblocks = (int)cl.num_blocks();
+  where.begin((int)blockIdx.x / nblocks);
   const int n = where.count();
   const long long off = where.offset();
   const int bits = cell_bits(n);
-  const int cells = 1 << (3 * bits);
+  // this block's share of the particles' loops and of the cells
+  const int step = nblocks * kUnroll * kThreads, begin = rank * kUnroll * kThreads;
+  const int share = 3 * bits - (nblocks > 1 ? 3 : 0), cells = 1 << share;
+  static_assert(kCluster == 8, "eight blocks take the key's first three bits");
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
   // position of particle k of the bunch; kUnroll of them are loaded before any is used
   auto position = [&](int k) { return where.at(off + k); };
   // bounding box of the present FP32 positions
   float lo[3] = {3.0e38f, 3.0e38f, 3.0e38f}, hi[3] = {-3.0e38f, -3.0e38f, -3.0e38f};
-  for (int k0 = tid; k0 < n; k0 += kUnroll * kThreads) {
+  for (int k0 = begin + tid; k0 < n; k0 += step) {
     float4 q[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; u++) {
@@ -139,13 +152,24 @@ __global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsign
   }
   for (int k = tid; k < cells; k += kThreads) hist[k] = 0;
   __syncthreads();
+  if (tid < 3) {
+    float a = 3.0e38f, b2 = -3.0e38f;
+    for (int w = 0; w < kThreads / 32; w++) {
+      a = fminf(a, s_lo[tid][w]);
+      b2 = fmaxf(b2, s_hi[tid][w]);
+    }
+    s_box[tid] = a;
+    s_box[3 + tid] = b2;
+  }
+  cl.sync();
   // the box as a cube of stretched axes
   float blo[3], sc[3], side = 0.f;
   for (int c = 0; c < 3; c++) {
     float a = 3.0e38f, b2 = -3.0e38f;
-    for (int w = 0; w < kThreads / 32; w++) {
-      a = fminf(a, s_lo[c][w]);
-      b2 = fmaxf(b2, s_hi[c][w]);
+    for (int r = 0; r < nblocks; r++) {
+      const float* box = cl.map_shared_rank(s_box, r);
+      a = fminf(a, box[c]);
+      b2 = fmaxf(b2, box[3 + c]);
     }
     blo[c] = a;
     sc[c] = where.stretch(c);
@@ -153,8 +177,9 @@ __global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsign
   }
   const float to_cell = side > 0.f ? (float)(1 << kKeyBits) / side : 0.f;
   const int drop = 3 * (kKeyBits - bits);  // bits of the key that the counting sort leaves out
+  auto count_of = [&](unsigned m) { return cl.map_shared_rank(hist, (int)((m >> drop) >> share)) + ((m >> drop) & (unsigned)(cells - 1)); };
   // cell keys and histogram
-  for (int k0 = tid; k0 < n; k0 += kUnroll * kThreads) {
+  for (int k0 = begin + tid; k0 < n; k0 += step) {
     float4 q[kUnroll];
 #pragma unroll
     for (int u = 0; u < kUnroll; u++) {
@@ -174,10 +199,10 @@ __global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsign
       }
       const unsigned m = hilbert_index(cc[0], cc[1], cc[2]);
       key[off + k] = m;
-      atomicAdd(hist + (m >> drop), 1);
+      atomicAdd(count_of(m), 1);
     }
   }
-  __syncthreads();
+  cl.sync();
   // exclusive scan of the cell counts: each thread owns a contiguous run of cells
   const int per = (cells + kThreads - 1) / kThreads;
   const int c0 = tid * per, c1 = min(cells, c0 + per);
@@ -197,34 +222,57 @@ __global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsign
       if (lane >= o) w += y;
     }
     s_warp[lane] = w;
+    if (lane == 31) s_total = w;
   }
-  __syncthreads();
+  cl.sync();
   int base = x - sum + (wid > 0 ? s_warp[wid - 1] : 0);
+  for (int r = 0; r < rank; r++) base += *cl.map_shared_rank(&s_total, r);
   for (int k = c0; k < c1; k++) {
     const int v = hist[k];
     hist[k] = base;
     base += v;
   }
-  __syncthreads();
+  cl.sync();
   // scatter
-  for (int k = tid; k < n; k += kThreads) {
-    const int pos = atomicAdd(hist + (key[off + k] >> drop), 1);
+  for (int k = rank * kThreads + tid; k < n; k += nblocks * kThreads) {
+    const int pos = atomicAdd(count_of(__ldcg(key + off + k)), 1);
     order[off + pos] = (int)(off + k);
   }
-  __syncthreads();
-  // windows of the list by the whole key: bitonic sort of (key, particle), whose last strides stay inside a warp
-  unsigned long long* win = reinterpret_cast<unsigned long long*>(hist);
-  for (int w0 = 0; w0 < n; w0 += kWindow) {
+  cl.sync();
+  // windows of the list by the whole key: bitonic sort of (key, particle)
+  for (int w0 = rank * kWindow; w0 < n; w0 += nblocks * kWindow) {
     const int m = min(kWindow, n - w0);
     int size = 64;
     while (size < m) size <<= 1;
-    for (int k = tid; k < size; k += kThreads) {
-      const int p = k < m ? order[off + w0 + k] : 0;
-      win[k] = k < m ? ((unsigned long long)key[p] << 32) | (unsigned)p : ~0ull;
-    }
-    __syncthreads();
-    for (int len = 2; len <= size; len <<= 1) {
-      for (int j = len >> 1; j > 0; j >>= 1) {
+    // a warp holds elements 64 wid + lane and + 32: strides below 64 stay in its registers
+    const int e0 = 64 * wid + lane, e1 = e0 + 32;
+    auto element = [&](int e) -> unsigned long long {
+      if (e >= m) return ~0ull;
+      const int p = __ldcg(order + off + w0 + e);
+      return ((unsigned long long)__ldcg(key + p) << 32) | (unsigned)p;
+    };
+    unsigned long long v0 = element(e0), v1 = element(e1);
+    auto inner = [&](int len, int j) {  // strides j, j / 2, .. 1
+      if (j == 32) {
+        const bool up = (e0 & len) == 0;
+        const unsigned long long lo = v0 < v1 ? v0 : v1, hi = v0 < v1 ? v1 : v0;
+        v0 = up ? lo : hi;
+        v1 = up ? hi : lo;
+        j = 16;
+      }
+      for (; j > 0; j >>= 1) {
+        const unsigned long long o0 = __shfl_xor_sync(0xffffffffu, v0, j), o1 = __shfl_xor_sync(0xffffffffu, v1, j);
+        const bool low = (lane & j) == 0;
+        if ((low == ((e0 & len) == 0)) == (o0 < v0)) v0 = o0;
+        if ((low == ((e1 & len) == 0)) == (o1 < v1)) v1 = o1;
+      }
+    };
+    for (int len = 2; len <= 64; len <<= 1) inner(len, len >> 1);
+    for (int len = 128; len <= size; len <<= 1) {
+      win[e0] = v0;
+      win[e1] = v1;
+      __syncthreads();
+      for (int j = len >> 1; j > 32; j >>= 1) {
         if (tid < size / 2) {
           const int lo_k = 2 * tid - (tid & (j - 1));
           const unsigned long long u = win[lo_k], v = win[lo_k + j];
@@ -233,44 +281,48 @@ __global__ void __launch_bounds__(kThreads) order_kernel(Positions where, unsign
             win[lo_k + j] = u;
           }
         }
-        if (j > 32 || (j == 1 && len >= 64))
-          __syncthreads();
-        else
-          __syncwarp();
+        __syncthreads();
       }
+      v0 = win[e0];
+      v1 = win[e1];
+      inner(len, 32);
     }
-    for (int k = tid; k < m; k += kThreads) order[off + w0 + k] = (int)(unsigned)win[k];
+    if (e0 < m) order[off + w0 + e0] = (int)(unsigned)v0;
+    if (e1 < m) order[off + w0 + e1] = (int)(unsigned)v1;
     __syncthreads();
   }
 }
 
 }  // namespace
 
-constexpr size_t kSmem = sizeof(int) << (3 * kMaxBits);
-
-// the largest bunch's cell counts or a window: a small system does not reserve 128 KB of shared memory
-static size_t shared_bytes(int n) {
-  const size_t cells = sizeof(int) << (3 * cell_bits(n)), window = sizeof(unsigned long long) * kWindow;
-  return cells > window ? cells : window;
+template <class Positions>
+static cudaError_t launch(const Positions& where, int nbunch, long long max_bunch, unsigned* key, int* order, cudaStream_t st) {
+  const int blocks = max_bunch > kWindow ? kCluster : 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(nbunch * blocks));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)blocks;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, order_kernel<Positions>, where, key, order);
 }
 
-// allows the kernel its shared-memory histogram on the current device (call before launching)
-cudaError_t prepare_target_order() {
-  cudaError_t e =
-      cudaFuncSetAttribute(order_kernel<RingPositions>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(order_kernel<ArrayPositions>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+// loads the caller-held positions' kernel, which its first launch would otherwise do (and take device memory for)
+cudaError_t load_array_order() {
+  cudaFuncAttributes attr;
+  return cudaFuncGetAttributes(&attr, order_kernel<ArrayPositions>);
 }
 
 cudaError_t launch_array_order(const double* x, const double* v, int n, unsigned* key, int* order, cudaStream_t st) {
-  order_kernel<<<1, kThreads, shared_bytes(n), st>>>(ArrayPositions{x, v, n}, key, order);
-  return cudaGetLastError();
+  return launch(ArrayPositions{x, v, n}, 1, n, key, order, st);
 }
 
 cudaError_t launch_target_order(const DeviceState& s, unsigned* key, int* order, long long max_bunch, cudaStream_t st) {
-  const size_t smem = shared_bytes((int)(max_bunch < (1LL << 30) ? max_bunch : (1LL << 30)));
-  order_kernel<<<s.nbunch, kThreads, smem, st>>>(RingPositions{s, nullptr, 0}, key, order);
-  return cudaGetLastError();
+  return launch(RingPositions{s, nullptr, 0, 0}, s.nbunch, max_bunch, key, order, st);
 }
 
 }  // namespace emppp
