@@ -45,6 +45,7 @@
 // the arithmetic and the work split are those of the same shape without it, so the fields are too.
 #include "bulk.cuh"
 #include "emppp_internal.cuh"
+#include "fp64_roots.cuh"
 #include "shadow.cuh"
 
 namespace emppp {
@@ -149,16 +150,6 @@ __device__ __forceinline__ bool exact_test(const double* __restrict__ rr, const 
   const double d2 = __dsub_rn(__ldg(rr + 2), __ldg(w + 2));
   const double rhs = __dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2));
   return lhs <= rhs;
-}
-
-// (float)x, round to nearest even, on the integer pipe: the 11 exponent bits become 8 (bias 1023 - 127 = 0x380), the
-// significand loses 29 bits. Outside FP32's normal range, the conversion itself.
-__device__ __forceinline__ float rounded_to_float(double x) {
-  const unsigned lo = (unsigned)__double2loint(x), hi = (unsigned)__double2hiint(x), e = hi & 0x7ff00000u;
-  if (e - 0x38100000u >= 0x0fd00000u) return (float)x;
-  unsigned t = __funnelshift_l(lo, hi, 3) - 0xc0000000u;  // exponent and the 23 significand bits that stay
-  if ((lo & 0x1fffffffu) + (t & 1u) > 0x10000000u) t += 1u;
-  return __uint_as_float(t | (hi & 0x80000000u));
 }
 
 // a0 b0 + a1 b1 + a2 b2 and a0 b1 - a1 b0 in a fixed rounding sequence (no compiler contraction)

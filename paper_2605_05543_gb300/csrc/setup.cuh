@@ -85,23 +85,25 @@ __device__ __forceinline__ void source_vectors_mixed(const DeviceState& s, long 
   if (o.ig2 < kXbGamma)
     write_line(s, j, x, o.r, T0, o.r[3] * (1.0 / kC), o.r[4] * (1.0 / kC), o.r[5] * (1.0 / kC), 0.0);
   float4* ext = s.ext32 + (size_t)j * kExtCount;
-  ext[kExtLine] = make_float4((float)((o.r[0] + o.r[3] * T0) - x[0]), (float)((o.r[1] + o.r[4] * T0) - x[1]),
-                              (float)((o.r[2] + o.r[5] * T0) - x[2]), o.gamma2);
+  ext[kExtLine] = make_float4(rounded_to_float((o.r[0] + o.r[3] * T0) - x[0]),
+                              rounded_to_float((o.r[1] + o.r[4] * T0) - x[1]),
+                              rounded_to_float((o.r[2] + o.r[5] * T0) - x[2]), o.gamma2);
   ext[kExtOldest] = make_float4(o.db[0], o.db[1], o.db[2], o.ig2);
   const double c0 = x[0] - o.r[0], c1 = x[1] - o.r[1], c2 = x[2] - o.r[2];
   const double ct = __dmul_rn(kC, T0);
   const double cc = c0 * c0 + c1 * c1 + c2 * c2;
   const double rhs = (double)upper_threshold(__dmul_rn(ct, ct)) * (1.0 + kChordMargin) - cc * (1.0 - kChordMargin);
-  ext[kExtChord] = make_float4((float)c0, (float)c1, (float)c2,
+  ext[kExtChord] = make_float4(rounded_to_float(c0), rounded_to_float(c1), rounded_to_float(c2),
                                seg ? fmaxf(__double2float_ru(rhs), 0.f) : __int_as_float(0x7f800000));
   if (!seg) return;  // no segment [n-1, n] in the window
   const BunchDesc& bd = s.bunches[s.nbunch == 1 ? 0 : s.bunch_of[j]];
-  const double d0 = (seg[0] + seg[3] * dtl) - bd.origin[0];
-  const double d1 = (seg[1] + seg[4] * dtl) - bd.origin[1];
-  const double d2 = (seg[2] + seg[5] * dtl) - bd.origin[2];
-  const float h0 = (float)d0, h1 = (float)d1, h2 = (float)d2;
-  ext[kExtSegHi] = make_float4(h0, h1, h2, 0.f);
-  ext[kExtSegLo] = make_float4((float)(d0 - (double)h0), (float)(d1 - (double)h1), (float)(d2 - (double)h2), 0.f);
+  float4 h, l;
+  split_to_floats((seg[0] + seg[3] * dtl) - bd.origin[0], h.x, l.x);
+  split_to_floats((seg[1] + seg[4] * dtl) - bd.origin[1], h.y, l.y);
+  split_to_floats((seg[2] + seg[5] * dtl) - bd.origin[2], h.z, l.z);
+  h.w = l.w = 0.f;
+  ext[kExtSegHi] = h;
+  ext[kExtSegLo] = l;
 }
 
 }  // namespace emppp

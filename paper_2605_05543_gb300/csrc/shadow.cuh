@@ -13,20 +13,21 @@
 #pragma once
 
 #include "emppp_internal.cuh"
+#include "fp64_roots.cuh"
 
 namespace emppp {
 
 __device__ __forceinline__ void shadow_record(const double origin[3], const double beta_ref[3], double w0, double w1,
                                               double w2, double v0, double v1, double v2, double gamma2, double inv_gamma2,
                                               float4 q[3]) {
-  const double d0 = w0 - origin[0], d1 = w1 - origin[1], d2 = w2 - origin[2];
-  const float h0 = (float)d0, h1 = (float)d1, h2 = (float)d2;
   const double ic = 1.0 / kC;
-  q[0] = make_float4(h0, h1, h2, (float)inv_gamma2);
-  q[1] = make_float4((float)(d0 - (double)h0), (float)(d1 - (double)h1), (float)(d2 - (double)h2),
-                     __int_as_float(0x7f800000));
-  q[2] = make_float4((float)(v0 * ic - beta_ref[0]), (float)(v1 * ic - beta_ref[1]), (float)(v2 * ic - beta_ref[2]),
-                     (float)gamma2);
+  split_to_floats(w0 - origin[0], q[0].x, q[1].x);
+  split_to_floats(w1 - origin[1], q[0].y, q[1].y);
+  split_to_floats(w2 - origin[2], q[0].z, q[1].z);
+  q[0].w = rounded_to_float(inv_gamma2);
+  q[1].w = __int_as_float(0x7f800000);
+  q[2] = make_float4(rounded_to_float(v0 * ic - beta_ref[0]), rounded_to_float(v1 * ic - beta_ref[1]),
+                     rounded_to_float(v2 * ic - beta_ref[2]), rounded_to_float(gamma2));
 }
 
 __device__ __forceinline__ void shadow_record(const double origin[3], const double beta_ref[3], double w0, double w1,
@@ -34,15 +35,20 @@ __device__ __forceinline__ void shadow_record(const double origin[3], const doub
   shadow_record(origin, beta_ref, w0, w1, w2, v0, v1, v2, gamma2, 1.0 / gamma2, q);
 }
 
-// dev of a slot at w0 with velocity v0 whose next slot, dt later, is at w1 (rounded up: the FP32 norm is within 4u, and
-// the added 1e-20 m covers squares that underflow)
+// dev of a slot at w0 with velocity v0 (inv_gamma2: 1 - v0.v0 / c^2) whose next slot, dt later, is at w1 (rounded up: the
+// FP32 norm is within 4u, and the added 1e-20 m covers squares that underflow)
+__device__ __forceinline__ float line_deviation(double w00, double w01, double w02, double v00, double v01, double v02,
+                                                double w10, double w11, double w12, double dt, double inv_gamma2) {
+  static_assert(kDevGamma2 == 16384.0, "the comparison below");
+  const float d0 = rounded_to_float((w10 - w00) - v00 * dt), d1 = rounded_to_float((w11 - w01) - v01 * dt),
+              d2 = rounded_to_float((w12 - w02) - v02 * dt);
+  const float up = fmaf(sqrtf(d0 * d0 + d1 * d1 + d2 * d2), 1.0302f, 1e-20f);
+  return at_least_2_m14(inv_gamma2) ? up : __int_as_float(0x7f800000);
+}
 __device__ __forceinline__ float line_deviation(double w00, double w01, double w02, double v00, double v01, double v02,
                                                 double w10, double w11, double w12, double dt) {
-  const float d0 = (float)((w10 - w00) - v00 * dt), d1 = (float)((w11 - w01) - v01 * dt),
-              d2 = (float)((w12 - w02) - v02 * dt);
-  const float up = fmaf(sqrtf(d0 * d0 + d1 * d1 + d2 * d2), 1.0302f, 1e-20f);
-  const double c2mv2 = kC * kC - (v00 * v00 + v01 * v01 + v02 * v02);
-  return c2mv2 >= kC * kC / kDevGamma2 ? up : __int_as_float(0x7f800000);
+  return line_deviation(w00, w01, w02, v00, v01, v02, w10, w11, w12, dt,
+                        1.0 - (v00 * v00 + v01 * v01 + v02 * v02) * (1.0 / (kC * kC)));
 }
 
 // gamma^2 of a stored velocity: 1 / (1 - v.v / c^2)
