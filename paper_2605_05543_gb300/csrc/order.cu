@@ -4,14 +4,15 @@
 // one source lie within a few cache lines, and they mostly take the same branch of the retarded-time search. Each
 // bunch's present positions get a key along a Hilbert curve of 1024^3 cells; a counting sort lists the particles by the
 // key's leading bits (6 to 15 from the bunch size), and windows of 2048 of the list are then sorted by the whole key.
-// The delay of a source changes 1 + beta times as fast along the bunch's motion as across it, so that axis is
-// stretched. (Branches that a warp takes for a source, N = 4096, 512 slots: 0.79 in history and 0.45 beyond with a
-// Morton curve of the leading bits alone, 0.75 and 0.42 now; the FP64 step there 2.36 -> 2.22 ms, N = 16381 28.9 ->
-// 27.6.) A bunch of more than 2048 particles is sorted by a cluster of eight blocks, each of which holds the
-// counts of an eighth of the cells, a smaller one by one block: latency and the shared-memory sort bound it (N = 8192:
-// 85 us with one block, 32 with eight; 65536: 697 and 100). The order is a permutation of each bunch's index range
-// (each target is evaluated exactly once whatever the order); the order inside a cell comes from shared-memory atomics
-// and may differ run to run, which changes which thread evaluates a target but not its result.
+// The delay of a source changes faster along the bunch's motion than across it, so that axis is stretched, by 1 + 2 beta
+// (N = 6000 mixed: 451 us with 1 + beta, 441 with 1 + 2 beta; 4096 FP64 2268 and 2241). Branches that a warp takes for
+// a source, N = 4096, 512 slots: 0.79 in history and 0.45 beyond with a Morton curve of the leading bits alone, 0.75 and
+// 0.42 with 1 + beta; the FP64 step there 2.36 -> 2.24 ms, N = 16381 28.7 -> 27.6, the mixed step of 65536 29.0 -> 28.2.
+// A bunch of more than 2048 particles is sorted by a cluster of eight blocks, each of which holds the counts of an
+// eighth of the cells, a smaller one by one block: latency and the shared-memory sort bound it (N = 8192: 85 us with one
+// block, 32 with eight; 65536: 697 and 100). The order is a permutation of each bunch's index range (each target is
+// evaluated exactly once whatever the order); the order inside a cell comes from shared-memory atomics and may differ
+// run to run, which changes which thread evaluates a target but not its result.
 #include <cooperative_groups.h>
 
 #include "emppp_internal.cuh"
@@ -80,7 +81,7 @@ struct RingPositions {  // present positions of a solver's bunches (hi parts abo
   }
   __device__ __forceinline__ int count() const { return s.bunches[bunch].n; }
   __device__ __forceinline__ long long offset() const { return s.bunches[bunch].off; }
-  __device__ __forceinline__ float stretch(int c) const { return 1.f + fabsf((float)s.bunches[bunch].beta_ref[c]); }
+  __device__ __forceinline__ float stretch(int c) const { return 1.f + 2.f * fabsf((float)s.bunches[bunch].beta_ref[c]); }
   // one record per particle's ring run, so every particle is its own cache line
   __device__ __forceinline__ float4 at(long long k) const { return __ldg(rec + ((size_t)k * s.D + pn) * 3); }
 };
@@ -91,7 +92,7 @@ struct ArrayPositions {  // x [n][3], about the first particle; v: its velocity
   __device__ __forceinline__ void begin(int) {}
   __device__ __forceinline__ int count() const { return n; }
   __device__ __forceinline__ long long offset() const { return 0; }
-  __device__ __forceinline__ float stretch(int c) const { return 1.f + fabsf((float)(__ldg(v + c) * (1.0 / kC))); }
+  __device__ __forceinline__ float stretch(int c) const { return 1.f + 2.f * fabsf((float)(__ldg(v + c) * (1.0 / kC))); }
   __device__ __forceinline__ float4 at(long long k) const {
     return make_float4((float)(__ldg(x + 3 * k) - __ldg(x)), (float)(__ldg(x + 3 * k + 1) - __ldg(x + 1)),
                        (float)(__ldg(x + 3 * k + 2) - __ldg(x + 2)), 0.f);

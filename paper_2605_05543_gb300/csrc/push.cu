@@ -199,8 +199,10 @@ cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st) {
 // push, the source vectors by a warp whose loads are there by then. With half = 1 (half-step field point) the clock already stands at
 // the provisional slot n+1: the push starts from slot n, the provisional slot is overwritten and the
 // clock moves from t_n + dt/2 to t_n + dt (formed from t_n, as without the variant).
+// With a full warp of pushers a block's phases (sums, push, records) use different units, so four blocks of 64 registers
+// to an SM beat two of 104: 196 us and 121 at N = 65536.
 template <int P>
-__global__ void __launch_bounds__(kEnergyThreads) step_post_kernel(DeviceState s, BextParams bp, AdaptParams ap,
+__global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_kernel(DeviceState s, BextParams bp, AdaptParams ap,
                                                                    int chunked, int half, SetupExt next, EnergyParams ep,
                                                                    EnergyMon* __restrict__ mon) {
   __shared__ ChunkSums<P> sums;
