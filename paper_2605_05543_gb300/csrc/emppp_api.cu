@@ -54,7 +54,9 @@ struct NvtxRange {
 };
 }  // namespace
 
-constexpr int kGraphs = 4;  // a step's graphs: with and without the target order, with and without the set-up launch
+// what a step does about the spatial target order, and the number of a step's graphs: each with and without the set-up
+enum OrderMode { kOrderNone, kOrderReuse, kOrderRefresh, kOrderModes };
+constexpr int kGraphs = 2 * kOrderModes;
 
 struct emppp_ctx {
   DeviceState ds{};
@@ -138,6 +140,8 @@ struct emppp_ctx {
 
 // steps between two computations of the spatial target order
 constexpr int kOrderEvery = 16;
+// particles up to which the mixed path goes without the order, and without it in the first step from a new state
+constexpr long long kUnorderedMixed = 1024, kLateOrderMixed = 2048;
 
 namespace {
 
@@ -451,9 +455,20 @@ SetupExt next_setup_of(emppp_handle h) {
   return h->opt.field_point == EMPPP_FIELD_HALF_STEP ? SetupExt::none : setup_of(h);
 }
 
-// enqueues the kernels of one step and reports how many kernels it launched; refresh_order recomputes the
-// spatial target order first (else the last one is used), set_up launches the set-up (else the step before formed it)
-emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev, int* nkernels, bool refresh_order,
+// The target order of the next step. Small systems on the mixed path go without: a few target tiles gain less from it
+// than its launch costs. Middle ones there go without in the first step from a new state, which would wait for it (one
+// step of 2000 particles: 166 us without, 172 with; a run of 25 adaptive steps of 1600 2520 without, 2361 from its second step). The FP64 path
+// always has it, since it keeps out-of-history and bracketed pairs in separate warps.
+OrderMode order_mode(emppp_handle h) {
+  const bool mixed = h->opt.precision == EMPPP_MIXED;
+  if (!h->opt.pair_fields || !h->target_order || (mixed && h->N <= kUnorderedMixed)) return kOrderNone;
+  if (h->order_age < 0) return mixed && h->N <= kLateOrderMixed ? kOrderNone : kOrderRefresh;
+  return h->order_age >= kOrderEvery - 1 ? kOrderRefresh : kOrderReuse;
+}
+
+// enqueues the kernels of one step and reports how many kernels it launched; set_up launches the set-up (else the step
+// before formed it)
+emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev, int* nkernels, OrderMode order,
                           bool set_up) {
   int k = 0;
   if (ev) CU(cudaEventRecord(ev[0], h->stream));
@@ -463,15 +478,12 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
     CU(launch_half_slot(h->ds, h->stream));
     k += 1;
   }
-  // window, slot tables, work counter and (mixed path) per-source segment vectors; beside it, on the
-  // second stream, the spatial order of the targets (it reads only the present positions). Small systems
-  // on the mixed path skip the order: a few target tiles gain less from it than its launch costs (the
-  // FP64 path keeps it, since it keeps out-of-history and bracketed pairs in separate warps).
-  const bool mixed_pairs = h->opt.pair_fields && h->opt.precision == EMPPP_MIXED;
-  const bool ordered = h->opt.pair_fields && h->target_order && !(mixed_pairs && h->N <= 2048);
+  // window, slot tables, work counter and per-source vectors; beside it, on the second stream, the spatial order of the
+  // targets (it reads only the present positions)
+  const bool ordered = order != kOrderNone;
   {
     NvtxRange r("emppp:setup");
-    if (ordered && refresh_order) {
+    if (order == kOrderRefresh) {
       CU(cudaEventRecord(h->ev_fork, h->stream));
       CU(cudaStreamWaitEvent(h->aux, h->ev_fork, 0));
       CU(launch_target_order(h->ds, h->ord_key, h->order, h->max_bunch, h->aux));
@@ -483,7 +495,7 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
       k += 1;
     }
   }
-  if (ordered && refresh_order) CU(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+  if (order == kOrderRefresh) CU(cudaStreamWaitEvent(h->stream, h->ev_join, 0));
   if (ev) CU(cudaEventRecord(ev[1], h->stream));
   if (h->opt.pair_fields) {
     NvtxRange r("emppp:pair_fields");
@@ -522,11 +534,11 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
 }
 
 // captures one step into a CUDA graph for the current configuration (options and background field), in the
-// variant that recomputes the target order (refresh_order) or reuses it, with the set-up launch (set_up) or without
-int graph_variant(bool refresh_order, bool set_up) { return (refresh_order ? 1 : 0) + (set_up ? 2 : 0); }
+// variant of its target order, with the set-up launch (set_up) or without
+int graph_variant(OrderMode order, bool set_up) { return order + (set_up ? kOrderModes : 0); }
 
-emppp_status capture_step(emppp_handle h, const BextParams& bp, bool refresh_order, bool set_up) {
-  const int v = graph_variant(refresh_order, set_up);
+emppp_status capture_step(emppp_handle h, const BextParams& bp, OrderMode order, bool set_up) {
+  const int v = graph_variant(order, set_up);
   unsigned char key[sizeof(emppp_options) + sizeof(BextParams) + sizeof(AdaptParams) + sizeof(EnergyParams)];
   memset(key, 0, sizeof(key));
   memcpy(key, &h->opt, sizeof(emppp_options));
@@ -542,7 +554,7 @@ emppp_status capture_step(emppp_handle h, const BextParams& bp, bool refresh_ord
   if (h->graph_valid[v]) return EMPPP_OK;
   CU(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   int k = 0;
-  emppp_status st = enqueue_step(h, bp, nullptr, &k, refresh_order, set_up);
+  emppp_status st = enqueue_step(h, bp, nullptr, &k, order, set_up);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(h->stream, &g);
   if (st != EMPPP_OK) {
@@ -952,20 +964,21 @@ EMPPP_API emppp_status emppp_step(emppp_handle h, int64_t nsteps, const emppp_be
     for (int b = 0; b < h->nbunch; b++) pairs_per_step += (long long)h->hb[b].n * (h->hb[b].n - 1);
   for (int64_t k = 0; k < nsteps; k++) {
     int nk = 0;
-    const bool refresh = h->order_age < 0 || h->order_age >= kOrderEvery - 1;
+    const OrderMode order = order_mode(h);
     const bool set_up = captured || h->prepared == SetupExt::none || h->prepared != setup_of(h);
     h->prepared = SetupExt::none;  // also if this step fails
     if (use_graph) {
-      if ((st = capture_step(h, bp, refresh, set_up)) != EMPPP_OK) return st;
-      const int v = graph_variant(refresh, set_up);
+      if ((st = capture_step(h, bp, order, set_up)) != EMPPP_OK) return st;
+      const int v = graph_variant(order, set_up);
       CU(cudaGraphLaunch(h->graph_exec[v], h->stream));
       nk = h->graph_launches[v];
     } else {
       cudaEvent_t* ev = nullptr;
       if (h->opt.timing && h->ev_used < emppp_ctx::kTimedSteps) ev = &h->events[4 * h->ev_used++];
-      if ((st = enqueue_step(h, bp, ev, &nk, refresh, set_up)) != EMPPP_OK) return st;
+      if ((st = enqueue_step(h, bp, ev, &nk, order, set_up)) != EMPPP_OK) return st;
     }
-    h->order_age = refresh ? 0 : h->order_age + 1;
+    // (without an order: the next step forms one)
+    h->order_age = order == kOrderRefresh ? 0 : (order == kOrderReuse ? h->order_age + 1 : kOrderEvery - 1);
     if (!captured) h->prepared = next_setup_of(h);
     h->launches += nk;
     h->pairs_acc += pairs_per_step;

@@ -34,3 +34,24 @@ def test_order_is_a_permutation(sizes, shape):
             out.append(s.get_state()[:2] + s.get_fields())
     for a, b in zip(*out):
         assert np.array_equal(a, b) and np.all(np.isfinite(a))
+
+
+@pytest.mark.parametrize("N", [1024, 1025, 2048, 2049])
+@pytest.mark.parametrize("adaptive,graphs", [(False, False), (False, True), (True, True)])
+def test_order_from_the_second_step(N, adaptive, graphs):
+    """Middle systems on the mixed path form the order in their second step, and again after a new state."""
+    b = inputs.gaussian_bunch(N, 8e-6, 3.0, seed=N)
+    out = []
+    for order in (0, 1):
+        with emppp.Solver(N, 8, 1e-15, precision="mixed", proposal="closed_form", graphs=graphs,
+                          stream=torch.cuda.Stream()) as s:
+            if adaptive:
+                s.set_adaptive_dt()
+            s.set_tuning(items_per_block=16, target_order=order)
+            for _ in range(2):
+                s.set_particles(b.x.copy(), b.u.copy())
+                s.step(1)
+                s.step(18)
+            out.append(s.get_state()[:2] + s.get_fields())
+    for a, c in zip(*out):
+        assert np.array_equal(a, c)
