@@ -207,8 +207,8 @@ void invalidate_graph(emppp_handle h) {
 // cost of the items (the branch mix differs across a bunch) evens out; systems too small for that get
 // one round of items with short chunks instead. At most max_split chunks per bunch. Uploaded when the
 // configuration changes.
-// fewest sources per chunk of a single round: 4 on the mixed path, 2 on the FP64 path, whose pairs are a longer chain (N = 256: 127 us with 4,
-// 115 with 2, a call that takes one step and reads the state back)
+// fewest sources per chunk of a single round: 4 on the mixed path, 2 on the FP64 path, whose pairs are a longer chain
+// (N = 256: 127 us with 4, 115 with 2, a call that takes one step and reads the state back)
 constexpr long long kMinChunkMixed = 4, kMinChunkFp64 = 2;
 
 emppp_status update_schedule(emppp_handle c) {
@@ -457,8 +457,8 @@ SetupExt next_setup_of(emppp_handle h) {
 
 // The target order of the next step. Small systems on the mixed path go without: a few target tiles gain less from it
 // than its launch costs. Middle ones there go without in the first step from a new state, which would wait for it (one
-// step of 2000 particles: 166 us without, 172 with; a run of 25 adaptive steps of 1600 2520 without, 2361 from its second step). The FP64 path
-// always has it, since it keeps out-of-history and bracketed pairs in separate warps.
+// step of 2000 particles: 166 us without, 172 with; a run of 25 adaptive steps of 1600 2520 without, 2361 from its second
+// step). The FP64 path always has it, since it keeps out-of-history and bracketed pairs in separate warps.
 OrderMode order_mode(emppp_handle h) {
   const bool mixed = h->opt.precision == EMPPP_MIXED;
   if (!h->opt.pair_fields || !h->target_order || (mixed && h->N <= kUnorderedMixed)) return kOrderNone;

@@ -195,7 +195,7 @@ struct DeviceState {
   double* ke;       // [N] kinetic-energy terms of the energy monitor, formed by the push (small systems)
   double* partial;  // [C][N][6] per-source-chunk partial sums
   int max_split;    // chunks the partial buffer holds
-  int* work;        // work-item counter of the persistent pair kernels (zeroed by the set-up launch)
+  int* work;        // work-item counter of the persistent pair kernels (zero when a pair launch starts)
   unsigned* done;   // blocks of the post-pair launch that have finished (reset by its last block)
   StepState* state;
   unsigned long long* stats;  // [kStatCount]
@@ -322,7 +322,7 @@ cudaError_t launch_gather_slot(const DeviceState& s, int p, double* W, double* V
 cudaError_t launch_set_state(const DeviceState& s, long long n, double t, double dt, long long hist_start,
                              const double* u, const double* w, cudaStream_t st);
 cudaError_t launch_prep(const DeviceState& s, cudaStream_t st);
-// per-source vectors the set-up launch forms: none, the mixed path's (ext32) or the FP64 path's (ext64)
+// per-source vectors a set-up forms: none, the mixed path's (ext32) or the FP64 path's (ext64)
 enum class SetupExt { none, mixed, fp64 };
 cudaError_t launch_setup(const DeviceState& s, SetupExt ext, cudaStream_t st);
 cudaError_t launch_reset_scale(const DeviceState& s, cudaStream_t st);

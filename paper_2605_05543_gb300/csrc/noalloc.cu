@@ -79,7 +79,7 @@ __device__ __forceinline__ bool na_node_test(double d0, double d1, double d2, do
 // order, so that a warp's pairs mostly take the same branch. What bounds it: the FP64 pipe (fp64_fields.cuh). The
 // tile's sources are staged with the factors that no target changes and, in FP32, what the guess reads. With the
 // paper's bisection, its node tests in FP64, the quadratic about the older node, divisions and square roots in place
-// of the refined approximations and targets in index order, n = 4096 with 200 slots took 6.71 ms; now 2.62 ms.
+// of the refined approximations and targets in index order, n = 4096 with 200 slots took 6.71 ms; now 2.54 ms.
 __global__ void __launch_bounds__(kBlock)
     na_pair_kernel(const double* __restrict__ W, const double* __restrict__ V, const double* __restrict__ wts,
                    const int* __restrict__ order, long long n, int nslots, long long chunk,

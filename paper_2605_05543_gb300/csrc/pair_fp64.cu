@@ -100,7 +100,8 @@ constexpr int kTile = 64;
 // Against the same inputs in 113 bits, pairs and sums are off by 0.3 to 0.9 of what the previous form was (quadratic
 // about t1, cross products; 50 and 118 operations) over gamma 2 to 197, and by under 1 % of it where R is far
 // below c (t_n - t_{n-1}). One step, before and after: 45.8 and 29.6 ms at N = 16381 (251 slots, closed-form guess),
-// 4.64 and 2.96 ms at N = 4096 (512 slots, bisection); the FP64 pipe is 90 % busy while an SM has work.
+// 4.64 and 2.96 ms at N = 4096 (512 slots, bisection); 27.6 and 2.23 with the short work items and the target order it
+// has now. The FP64 pipe is 90 % busy while an SM has work.
 // SHAPE: targets per block (kBlock = shape_block(SHAPE); shapes 3 and 4 run as shape 0)
 template <int PROP, bool ADAPT, bool MID, bool DUMP, int SHAPE>
 __global__ void __launch_bounds__(shape_block(SHAPE)) pair_fp64_kernel(PairArgs a) {
@@ -522,7 +523,7 @@ cudaError_t launch_pair_fp64(const DeviceState& s, const int* order, int proposa
   a.eta_allow = ap.eta_allow;
   a.order = order;
   a.dump = dump;
-  // the work counter is zeroed by the set-up launch that precedes every pair launch
+  // the work counter is zeroed by the set-up launch or the post-pair launch before
   // the midpoint reconstruction runs with a fixed time step only (the host refuses the combination);
   // the bracket dump runs the method's instance (the brackets depend on neither variant)
   if (dump)

@@ -19,7 +19,8 @@
 //             first: 32.6 against 30.8 ms at N = 65536, 251 slots).
 //   retarded  and fields, fixed step: from the source's line at t_n (at the code below).
 //   retarded  adaptive step: the textbook forms, whose every rounding is kept: the last bit of |eta| and v_j(t_r)
-//             decides the step and with it every later time stamp: in light units (lengths in m, velocities as beta = v/c): with L1 = c (t - t1) and d = r - w1,
+//             decides the step and with it every later time stamp: in light units (lengths in m, velocities as
+//             beta = v/c): with L1 = c (t - t1) and d = r - w1,
 //             (1 - beta1^2) s^2 + 2 (d.beta1 - L1) s + (L1^2 - |d|^2) = 0 for s = c (t_r - t1) (eq:dt),
 //             smaller root without cancellation; eta = d - beta1 s (eq:linear, retarded position w1 + v1 dt);
 //             in the near-field shortcut bracket the same point is formed from the segment's end
@@ -38,8 +39,8 @@
 // Vector arithmetic takes x and y in one packed FP32x2 instruction where both operands come as pairs
 // (separations, velocity differences, the retarded point, u', F, the sums) and z as a scalar.
 // Sources are walked in tiles of kTile (half a block's targets) whose present records, out-of-history
-// lines, oldest-slot chords and FP32 charges are staged in shared memory; targets are taken in the spatial order of order.cu so that a warp's retarded slots of a
-// source are close together in the source-major FP32 shadow ring. The window instance (shape_win)
+// lines, oldest-slot chords and FP32 charges are staged in shared memory; targets are taken in the spatial order of
+// order.cu so that a warp's retarded slots of a source are close together in the source-major FP32 shadow ring. The window instance (shape_win)
 // also copies, per warp and one source ahead, the ring slots its lanes' guessed brackets fall in to
 // shared memory by bulk copy (bulk.cuh) and reads the predicted brackets' records there; the search,
 // the arithmetic and the work split are those of the same shape without it, so the fields are too.
@@ -1166,7 +1167,7 @@ cudaError_t launch_pair_mixed(const DeviceState& s, const int* order, int propos
   a.ext32 = s.ext32;
   a.dump = dump;
   a.wait_limit = pl.wait_limit;
-  // the work counter is zeroed by the set-up launch that precedes every pair launch; the bracket dump
+  // the work counter is zeroed by the set-up launch or the post-pair launch before; the bracket dump
   // runs the instance without the adaptive step's reduction (the brackets do not depend on it)
   if (dump)
     launch_mixed<false, true, 0>(proposal, pl, a, st);

@@ -196,7 +196,8 @@ cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st) {
 // after its work; nothing waits on it. With next it also forms what the pair kernel of the next step needs (setup.cuh),
 // so that step goes without its set-up launch (6 us and a gap between launches, of 43 us a step with the paper's 400
 // macroparticles): the slot tables need the step size alone and are formed by the warps that sum no chunks while others
-// push, the source vectors by a warp whose loads are there by then. With half = 1 (half-step field point) the clock already stands at
+// push, the source vectors by a warp whose loads are there by then. With half = 1 (half-step field point) the clock
+// already stands at
 // the provisional slot n+1: the push starts from slot n, the provisional slot is overwritten and the
 // clock moves from t_n + dt/2 to t_n + dt (formed from t_n, as without the variant).
 // With a full warp of pushers a block's phases (sums, push, records) use different units, so four blocks of 64 registers

@@ -170,9 +170,9 @@ __global__ void prep_kernel(DeviceState s) {
   for (int l = blockIdx.x * blockDim.x + threadIdx.x; l < nwin; l += gridDim.x * blockDim.x) slot_table(s, l, p0, pn, nwin, t_n);
 }
 
-// Set-up of the pair kernel, for a step that the post-pair launch of the step before did not prepare: the window k0..n and its slot tables (as
-// prep_kernel), the pair kernel's work counter, and, for the mixed path, per-source vectors (eq:linear at
-// t_n):
+// Set-up of the pair kernel, for a step that the post-pair launch of the step before did not prepare: the window k0..n
+// and its slot tables (as prep_kernel), the pair kernel's work counter, and, for the mixed path, per-source vectors
+// (eq:linear at t_n):
 //   P_j = w_{j,n-1} + v_{j,n-1} (t_n - t_{n-1}), the end of the last history segment, split hi/lo about
 //     the bunch origin. For a pair in the near-field shortcut bracket [n-1, n] the retarded point is
 //     written as P_j - v_{j,n-1} tau with tau = t_n - t_r: the same point as w_{j,n-1} + v_{j,n-1}
