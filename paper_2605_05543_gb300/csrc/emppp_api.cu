@@ -251,8 +251,8 @@ emppp_status update_schedule(emppp_handle c) {
     return t;
   }();
   // Chunking of one bunch, by sources per chunk. An SM with few blocks left runs below its rate, and a pair in the
-  // history costs more than one beyond it, so the items are many and short: as many as 2 items_per_block items per
-  // resident block over all bunches allow (counted in 128-target tiles), but of at least 8 (FP64) or 32 (mixed)
+  // history costs more than one beyond it, so the items are many and short: as many as 2 (FP64: 4)
+  // items_per_block items per resident block over all bunches allow (counted in 128-target tiles), but of at least 8 (FP64) or 32 (mixed)
   // sources, below which an item's own set-up shows, and on the mixed path at most 128 chunks; or one round of items,
   // if that is more (a system too small to fill the resident blocks: each block's time is then its own chunk length).
   // Steps in us by sources per chunk:
@@ -266,7 +266,7 @@ emppp_status update_schedule(emppp_handle c) {
   const bool whole = mixed && ad;
   auto chunks = [&](long long n, bool small) -> long long {
     const long long one_round = Rreal / total_tiles > 1 ? Rreal / total_tiles : 1;
-    const long long many = (2LL * c->items_per_block * Rsched + tiles128 - 1) / tiles128;
+    const long long many = ((mixed ? 2LL : 4LL) * c->items_per_block * Rsched + tiles128 - 1) / tiles128;
     auto of = [&](long long nchunk, long long fewest) { return std::min(nchunk, (n + fewest - 1) / fewest); };
     const long long kMin = mixed ? kMinChunkMixed : kMinChunkFp64;
     long long nchunk;
