@@ -122,8 +122,9 @@ constexpr float kChordLo = 1.0f - 32.0f * 5.9604644775390625e-08f;
 // in units of c dt: 27u L_A in all; the slope is off by less than 3 % for gamma^2 up to kDevGamma2. So if
 //   (1 - f) sq  >  tau / (c dt) [33u L_A + 1.03 dev]
 // as computed, the exact |r - w_B| exceeds L_B by more than 5u L_A, far above the FP64 test's rounding: P(B) is
-// true. The FP32 record of A holds 1.03 dev in q1.w (rounded up), +inf while it has no newer node or above
-// kDevGamma2, which leaves the test to the node itself.
+// true. (Not for a target more than 0.5 m from the split's origin: the low part of a coordinate x there rounds by up to
+// 2^-49 |x|, which the margin does not cover.) The FP32 record of A holds 1.03 dev in q1.w (rounded up), +inf while it
+// has no newer node or above kDevGamma2, which leaves the test to the node itself.
 constexpr float kNewerMargin = 33.0f * 5.9604644775390625e-08f;
 constexpr double kDevGamma2 = 16384.0;
 

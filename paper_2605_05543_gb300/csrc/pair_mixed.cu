@@ -794,7 +794,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
             if (!tA) {
               const bool last = lg == win.nw - 2;  // the newer node is the present slot: P(n) is always true
               if (!last) n_tests += 1;
-              if (!ADAPT && line_fields(A, dA, tabA, q2b, pA, last ? 1 : 2, !last)) {
+              // (a target that the FP32 split cannot hold has a separation too coarse for the bound)
+              if (!ADAPT && (last || !r.exact_only) && line_fields(A, dA, tabA, q2b, pA, last ? 1 : 2, !last)) {
                 brc += last ? 1u << 10 : 1u << 20;
                 if (DUMP) a.dump[(size_t)i * N + j] = 4 * lg + (last ? 1 : 2);
                 continue;
