@@ -234,13 +234,14 @@ emppp_status update_schedule(emppp_handle c) {
   // The history-window shape splits the work like the same shape without the window, so that their fields
   // are identical.
   const int shp_ref = shape_win(shp) > 0 ? 4 : shp;
-  int& nref = mixed ? c->blocks_mixed[ad][EMPPP_PROPOSAL_CLOSED_FORM][shp_ref]
-                    : c->blocks_fp64[ad][EMPPP_PROPOSAL_CLOSED_FORM][shp_ref];
-  if (nref <= 0)
-    nref = mixed ? max_blocks_pair_mixed(EMPPP_PROPOSAL_CLOSED_FORM, ad, shp_ref)
-                 : max_blocks_pair_fp64(EMPPP_PROPOSAL_CLOSED_FORM, ad, shp_ref);
+  int& nref_cached = mixed ? c->blocks_mixed[ad][EMPPP_PROPOSAL_CLOSED_FORM][shp_ref]
+                           : c->blocks_fp64[ad][EMPPP_PROPOSAL_CLOSED_FORM][shp_ref];
+  if (nref_cached <= 0)
+    nref_cached = mixed ? max_blocks_pair_mixed(EMPPP_PROPOSAL_CLOSED_FORM, ad, shp_ref)
+                        : max_blocks_pair_fp64(EMPPP_PROPOSAL_CLOSED_FORM, ad, shp_ref);
+  const int nref = mixed && ad ? kAdaptRound : nref_cached;
   // resident blocks in units of 128 threads, so that the item count per SM does not depend on the shape
-  const long long R = (long long)nb * c->num_sms;
+  long long R = (long long)nb * c->num_sms;
   const long long Rsched = (long long)nref * c->num_sms * TB / 128;
   const long long Rreal = (long long)nref * c->num_sms;  // resident blocks of the shape
   long long total_tiles = 0;
@@ -307,6 +308,9 @@ emppp_status update_schedule(emppp_handle c) {
     item += s.ntb * s.nchunk;
   }
   c->launch.nitems = item;
+  // one round of blocks that only the instance with more of them per SM holds at once (why, at mixed_min_blocks)
+  c->launch.adapt_round = mixed && ad && c->opt.proposal != EMPPP_PROPOSAL_BISECT && item > R && item <= Rreal;
+  if (c->launch.adapt_round) R = Rreal;
   c->launch.grid = (int)(R < item ? R : item);
   c->launch.shape = shp;
   CU(cudaMemcpyAsync(c->d_sched, c->hs.data(), sizeof(BunchSched) * c->nbunch, cudaMemcpyHostToDevice, c->stream));

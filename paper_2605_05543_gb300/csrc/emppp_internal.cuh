@@ -286,7 +286,12 @@ struct PairLaunch {
   int grid;    // blocks launched
   int shape;   // tile shape (shape_block(shape) threads per block, targets per work item)
   int wait_limit = 1 << 16;  // probes of a bounded wait on a staged history window (window shapes)
+  bool adapt_round = false;  // mixed path, adaptive step, guessed search: the instance of kAdaptRound blocks per SM
 };
+
+// Resident blocks per SM with which the mixed path's adaptive steps split their work: their step size follows the last
+// bit of FP32 sums, so the grouping stays that of runs made so far whichever instance runs
+constexpr int kAdaptRound = 8;
 
 // the work item a block takes after `item` (-1: its first): from the counter, or, with a block for every item (small
 // systems), its own and no other, without the counter's round trips

@@ -60,7 +60,12 @@ namespace {
 // Resident blocks per SM, of 128 threads: 8 at 64 registers (N = 32768: 7.69 ms; 7 at 72 registers 8.08, 9 at 56 with
 // spills 10.0). The history-window shape holds more state across a pair and spills 132 bytes at 64 registers: 7 blocks
 // (N = 16384: 3.21 ms against 3.88 at 8 and 3.41 at 6).
-constexpr int mixed_min_blocks(int shape) {
+// The guessed-search instances of the adaptive step hold the textbook forms and the list of FP64 lines: 112 / 152 bytes of
+// spill stores / loads at 64 registers, 36 / 64 at 72. So 7 blocks (gamma 3, N = 5000: 1.30 ms against 1.37 at 8; 12000:
+// 4.23 and 4.31), but 8 where all items fit one round of those alone (3000: 422 us against 450; 3900: 661 and 736).
+constexpr int kAdaptBlocks = 7;
+constexpr int mixed_min_blocks(int shape, bool adapt, int prop) {
+  if (adapt && prop != kPropBisect) return kAdaptBlocks;
   return (shape_win(shape) > 0 ? EMPPP_MIXED_MIN_BLOCKS - 1 : EMPPP_MIXED_MIN_BLOCKS) * 128 / shape_block(shape);
 }
 
@@ -236,8 +241,8 @@ __device__ __forceinline__ int bisect(const Target& r, const float4* __restrict_
 
 // SHAPE: targets per block (kBlock), sources per FP32 partial sum (kSub); the
 // register budget stays at 64 per thread for every block size
-template <int PROP, bool ADAPT, bool DUMP, int SHAPE>
-__global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
+template <int PROP, bool ADAPT, bool DUMP, int SHAPE, int BLOCKS = mixed_min_blocks(SHAPE, ADAPT, PROP)>
+__global__ void __launch_bounds__(shape_block(SHAPE), BLOCKS)
     pair_mixed_kernel(MixedArgs a) {
   constexpr int kBlock = shape_block(SHAPE);
   // sources per staged tile: half a block's targets, which keeps 8 blocks of the (128, *) shapes within the
@@ -270,12 +275,14 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
   __shared__ float4 s_ck[kTileG];
   __shared__ float s_acc[12][kBlock];  // per-thread compensated sums
 
-  // adaptive step: the targets' present positions in FP64, and per warp the pairs of a group of kSub sources that need
-  // their line in FP64 (lane + 32 source) and what fp64_line gives for them
-  constexpr int kLines = ADAPT ? 64 : 1;
-  __shared__ double s_r[ADAPT ? 3 : 1][ADAPT ? kBlock : 1];
+  // adaptive step: per warp the pairs of a group of kSub sources that need their line in FP64 (lane + 32 source) and what
+  // fp64_line gives for them (their targets' FP64 positions are read from the ring: a staged copy, 3 KB a block, took the
+  // blocks past the 132 KB carveout, and with 8 blocks of the guessed search so does a list of more than 36). s_listed, per
+  // lane: bit k: source k of the group is in the list; from bit 8: the lane's first entry
+  constexpr int kLines = !ADAPT ? 1 : (BLOCKS == 8 && PROP != kPropBisect ? 36 : 64);
   __shared__ unsigned char s_pair[kWarps][kLines];
   __shared__ float4 s_y[kWarps][kLines];
+  __shared__ unsigned short s_listed[ADAPT ? kBlock : 1];
   static_assert(!ADAPT || kSub <= 8, "a lane's list is eight bits");
 
   __shared__ int s_item;
@@ -359,11 +366,6 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
     r.l2 = q1.z;
     r.idx = i;
     r.exact_only = fmaxf(fabsf(r.h01.x), fmaxf(fabsf(r.h01.y), fabsf(r.h2))) > 0.5f;
-    if (ADAPT) {
-      const double* rr = a.rec64 + ((size_t)i * D + pn) * 6;
-#pragma unroll
-      for (int c = 0; c < 3; c++) s_r[c][threadIdx.x] = __ldg(rr + c);
-    }
   }
   // learned proposal: the delay factors of this target tile's group (kFacGroup targets, a multiple of the
   // tile), one per source of the bunch
@@ -464,8 +466,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
       // Adaptive step (the paper's runs, up to 100 MeV). One pair in eleven needs FP64 at gamma 197, which as a branch
       // of the pair loop nearly every warp takes with three lanes of 32, and the FP64 pipe then bounds the kernel. So
       // the pairs of a group that need it are listed first and evaluated with all lanes.
-      unsigned listed = 0;  // bit k: source jj0 + k is in the list; from bit 8: the lane's first entry
       if (ADAPT && fast_sources) {
+        unsigned listed = 0;
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
         for (int k = 0; active && k < jend - jj0; k++) {
           const float4 o = s_k0[jj0 + k], gx = s_x[jj0 + k];
@@ -486,12 +488,14 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
         for (unsigned q = listed; q && at < kLines; q &= q - 1u, at++)
           s_pair[w][at] = (unsigned char)(lane + 32 * (__ffs(q) - 1));
         __syncwarp();
-        for (int e = lane; e < total; e += 32) {
-          const int pr = s_pair[w][e], tl = 32 * w + (pr & 31);
-          s_y[w][e] = fp64_line(a.ext64 + (size_t)(tile + jj0 + (pr >> 5)) * (kExt64 / 2), s_r[0][tl], s_r[1][tl], s_r[2][tl]);
+        for (int e0 = 0; e0 < total; e0 += 32) {
+          const int e = e0 + lane, pr = s_pair[w][min(e, total - 1)];
+          const double* rr = a.rec64 + ((size_t)__shfl_sync(0xffffffffu, i, pr & 31) * D + pn) * 6;
+          if (e < total)
+            s_y[w][e] = fp64_line(a.ext64 + (size_t)(tile + jj0 + (pr >> 5)) * (kExt64 / 2), __ldg(rr), __ldg(rr + 1), __ldg(rr + 2));
         }
         __syncwarp();
-        listed |= (unsigned)(end - cnt) << 8;
+        s_listed[threadIdx.x] = (unsigned short)(listed | (unsigned)(end - cnt) << 8);
       }
       for (int jj = jj0; (WIN || active) && jj < jend; ++jj) {
         const int j = debug_index(tile + jj, boff, boff + bd.n, a.err);
@@ -545,7 +549,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), mixed_min_blocks(SHAPE))
           // near perpendicular to beta) X and X.beta are formed in FP64 from the FP64 records instead.
           // (as the shift is at most u gamma, sources with gamma^2 < 100 never need it)
           if (needs_fp64_line(XX, Xb, ig2)) {
-            const int k = jj - jj0, at = (int)(listed >> 8) + __popc(listed & ((1u << k) - 1u));
+            const unsigned listed = ADAPT ? s_listed[threadIdx.x] : 0;
+            const int k = jj & (kSub - 1), at = (int)(listed >> 8) + __popc(listed & ((1u << k) - 1u));
             float4 y;
             if (ADAPT && ((listed >> k) & 1u) && at < kLines) {
               y = s_y[threadIdx.x >> 5][at];
@@ -1130,6 +1135,16 @@ int max_blocks_pair_mixed(int proposal, bool adapt, int shape) {
 template <bool ADAPT, bool DUMP, int SHAPE>
 void launch_mixed(int proposal, const PairLaunch& pl, const MixedArgs& a, cudaStream_t st) {
   constexpr int B = shape_block(SHAPE);
+  if constexpr (ADAPT) {
+    if (pl.adapt_round && proposal == kPropClosedForm) {
+      pair_mixed_kernel<kPropClosedForm, ADAPT, DUMP, SHAPE, kAdaptRound><<<pl.grid, B, 0, st>>>(a);
+      return;
+    }
+    if (pl.adapt_round && proposal == kPropMlp) {
+      pair_mixed_kernel<kPropMlp, ADAPT, DUMP, SHAPE, kAdaptRound><<<pl.grid, B, 0, st>>>(a);
+      return;
+    }
+  }
   if (proposal == kPropClosedForm)
     pair_mixed_kernel<kPropClosedForm, ADAPT, DUMP, SHAPE><<<pl.grid, B, 0, st>>>(a);
   else if (proposal == kPropMlp)
