@@ -525,7 +525,8 @@ emppp_status enqueue_step(emppp_handle h, const BextParams& bp, cudaEvent_t* ev,
   // launch evaluates the bunches in parallel, one block each)
   const bool fused_energy = h->energy.on && h->N <= 16384 && h->nbunch <= 8;
   NvtxRange r_post("emppp:push_append");
-  CU(launch_step_post(h->ds, bp, h->adapt, chunked, half, next_setup_of(h), fused_energy ? &h->energy : nullptr, h->d_mon, h->stream));
+  CU(launch_step_post(h->ds, bp, h->adapt, chunked, half, next_setup_of(h), h->opt.pair_fields != 0,
+                      fused_energy ? &h->energy : nullptr, h->d_mon, h->num_sms, h->stream));
   k += 1;
   if (h->energy.on && !fused_energy) {
     // mean energy of the new state and the switch criterion (Sec. 2.7)

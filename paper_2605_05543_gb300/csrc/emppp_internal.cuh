@@ -343,8 +343,9 @@ cudaError_t launch_pair_fp64(const DeviceState& s, const int* order, int proposa
                              const AdaptParams& ap, const PairLaunch& pl, cudaStream_t st, int* dump = nullptr);
 cudaError_t launch_zero_self(const DeviceState& s, cudaStream_t st);
 // push.cu
-cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked,
-                             bool half, SetupExt next, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st);
+cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked, bool half,
+                             SetupExt next, bool dev, const EnergyParams* ep, EnergyMon* mon, int num_sms,
+                             cudaStream_t st);
 cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_half_slot(const DeviceState& s, cudaStream_t st);
 // stage2.cu

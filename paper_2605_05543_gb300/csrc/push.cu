@@ -202,13 +202,18 @@ cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st) {
 // clock moves from t_n + dt/2 to t_n + dt (formed from t_n, as without the variant).
 // With a full warp of pushers a block's phases (sums, push, records) use different units, so four blocks of 64 registers
 // to an SM beat two of 104: 196 us and 121 at N = 65536.
+// P = kEnergyThreads: a thread per particle that does all of its particle's work, for systems without partial sums that
+// would take more than one round of the blocks of 32, most of whose threads have nothing to do then. Eight steps without
+// pair fields, 32 particles a block and a thread each: N = 10000 154 us and 200; 20000 220 and 195; 65536 385 and 286;
+// 1e6 4250 and 2470.
 template <int P>
 __global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_kernel(DeviceState s, BextParams bp, AdaptParams ap,
-                                                                   int chunked, int half, SetupExt next, EnergyParams ep,
-                                                                   EnergyMon* __restrict__ mon) {
-  __shared__ ChunkSums<P> sums;
+                                                                   int chunked, int half, SetupExt next, int dev,
+                                                                   EnergyParams ep, EnergyMon* __restrict__ mon) {
+  constexpr bool kOwn = P == kEnergyThreads;
+  __shared__ ChunkSums<kOwn ? 8 : P> sums;  // (not used, and left out, with a thread per particle)
   __shared__ double s_step[3];
-  __shared__ double s_new[P][12];  // pushed particles: x, u, and the slot before, x and v
+  __shared__ double s_new[kOwn ? 1 : P][12];  // pushed particles: x, u, and the slot before, x and v
   const long long i0 = (long long)blockIdx.x * P;
   const StepState st = *s.state;
   // slot of x^n, the slot the push writes and t_n
@@ -230,27 +235,31 @@ __global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_ker
     }
   }
   const int task = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long it = i0 + lane;
+  const long long it = kOwn ? i : i0 + lane;
+  // whether this thread does task k of particle it
+  auto does = [&](int k) { return kOwn ? pusher : task == k && lane < P && it < s.N; };
   // the next step's window (fixed here: half and next exclude one another)
   const bool slides = st.n + 1 - s.D + 1 > st.k0;
   const long long k0_next = slides ? st.k0 + 1 : st.k0;
   const int p0_next = !slides ? st.p0 : (st.p0 + 1 == s.D ? 0 : st.p0 + 1);
-  const bool sets_up = next != SetupExt::none && task == 3 && lane < P && it < s.N;
+  const bool sets_up = next != SetupExt::none && does(3);
   Oldest old;
   double t_old = 0.0;
-  if (sets_up) {
+  auto load_oldest = [&] {
     old.load(s, next, it, p0_next);
     t_old = s.slot_t[p0_next];
-  }
-  if (chunked)
+  };
+  if (!kOwn && sets_up) load_oldest();
+  if (!kOwn && chunked)
     sums.run(s, i0);
   else if (ap.on)
     __syncthreads();  // s_step
   const double dt = ap.on ? s_step[0] : st.dt;
-  if (next != SetupExt::none && threadIdx.x >= kSumThreads) {
-    constexpr int kTableThreads = kEnergyThreads - kSumThreads;
+  constexpr int kTableFirst = kOwn ? 0 : kSumThreads;
+  if (next != SetupExt::none && (int)threadIdx.x >= kTableFirst) {
+    constexpr int kTableThreads = kEnergyThreads - kTableFirst;
     const int nwin = (int)(st.n + 1 - k0_next) + 1;
-    for (int l = blockIdx.x * kTableThreads + (int)threadIdx.x - kSumThreads; l < nwin; l += gridDim.x * kTableThreads)
+    for (int l = blockIdx.x * kTableThreads + (int)threadIdx.x - kTableFirst; l < nwin; l += gridDim.x * kTableThreads)
       slot_table(s, l, p0_next, pnext, nwin, t_n + dt);
   }
   if (i == 0) {
@@ -261,9 +270,10 @@ __global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_ker
       s.adapt_info[2] = s_step[2];
     }
   }
+  double own[12];
   if (pusher) {
     double E[3], Bs[3];
-    if (chunked && sums.chunks[threadIdx.x] > 1) {
+    if (!kOwn && chunked && sums.chunks[threadIdx.x] > 1) {
       const double2 a = sums.sum[3 * threadIdx.x], b = sums.sum[3 * threadIdx.x + 1], c = sums.sum[3 * threadIdx.x + 2];
       E[0] = a.x;
       E[1] = a.y;
@@ -277,7 +287,7 @@ __global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_ker
         Bs[c] = s.Bself[3 * i + c];
       }
     }
-    double* out = s_new[threadIdx.x];
+    double* out = kOwn ? own : s_new[threadIdx.x];
     for (int c = 0; c < 3; c++) {
       out[6 + c] = x[c];
       out[9 + c] = vn[c];
@@ -300,36 +310,34 @@ __global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_ker
     vn[1] = v[1];
     vn[2] = v[2];
   }
-  __syncthreads();
+  if (!kOwn) __syncthreads();
   // What follows from the pushed state, by a warp each: the FP32 record, the monitor's term, how far slot n + 1 lies from
-  // slot n's line (newer-node bound of the mixed path), and the next step's source vectors
+  // slot n's line (dev: the newer-node bound of the mixed path; without it the record keeps +inf, which the bound takes
+  // as unknown), and the next step's source vectors
+  const double* o = kOwn ? own : s_new[lane];
+  if (kOwn && sets_up) load_oldest();
   if (sets_up) {
-    const double* o = s_new[lane];
     const double T0 = (t_n + dt) - t_old;
     if (next == SetupExt::fp64)
       source_vectors_fp64(s, it, o, old, T0);
     else
       source_vectors_mixed(s, it, o, old, T0, o + 6, (t_n + dt) - t_n);
   }
-  if (task < 3 && lane < P && it < s.N) {
-    const double* o = s_new[lane];
-    if (task == 0) {
-      const BunchDesc& bd = s.bunches[s.nbunch == 1 ? 0 : s.bunch_of[it]];
-      // gamma^2 = 1 + u.u / c^2 and its inverse without divisions (both are rounded to FP32)
-      const double gamma2 = 1.0 + (o[3] * o[3] + o[4] * o[4] + o[5] * o[5]) * (1.0 / (kC * kC));
-      float4 q[3];
-      shadow_record(bd.origin, bd.beta_ref, o[0], o[1], o[2], vn[0], vn[1], vn[2], gamma2, recip_refined(gamma2), q);
-      float4* w = reinterpret_cast<float4*>(s.rec32 + ((size_t)it * s.D + pnext) * 12);
-      w[0] = q[0];
-      w[1] = q[1];
-      w[2] = q[2];
-    } else if (task == 1) {
-      if (ep.on) s.ke[it] = kinetic_term(o[3], o[4], o[5], s.wts[it]);
-    } else {
-      s.rec32[((size_t)it * s.D + pfrom) * 12 + 7] =
-          line_deviation(o[6], o[7], o[8], o[9], o[10], o[11], o[0], o[1], o[2], (t_n + dt) - t_n);
-    }
+  if (does(0)) {
+    const BunchDesc& bd = s.bunches[s.nbunch == 1 ? 0 : s.bunch_of[it]];
+    // gamma^2 = 1 + u.u / c^2 and its inverse without divisions (both are rounded to FP32)
+    const double gamma2 = 1.0 + (o[3] * o[3] + o[4] * o[4] + o[5] * o[5]) * (1.0 / (kC * kC));
+    float4 q[3];
+    shadow_record(bd.origin, bd.beta_ref, o[0], o[1], o[2], vn[0], vn[1], vn[2], gamma2, recip_refined(gamma2), q);
+    float4* w = reinterpret_cast<float4*>(s.rec32 + ((size_t)it * s.D + pnext) * 12);
+    w[0] = q[0];
+    w[1] = q[1];
+    w[2] = q[2];
   }
+  if (ep.on && does(1)) s.ke[it] = kinetic_term(o[3], o[4], o[5], s.wts[it]);
+  if (dev && does(2))
+    s.rec32[((size_t)it * s.D + pfrom) * 12 + 7] =
+        line_deviation(o[6], o[7], o[8], o[9], o[10], o[11], o[0], o[1], o[2], (t_n + dt) - t_n);
   // the last block to finish advances the clock and resets the reduction for the next step (and, with
   // ep.on, evaluates the energy monitor of every bunch on the pushed state)
   __shared__ bool s_last;
@@ -365,19 +373,24 @@ __global__ void __launch_bounds__(kEnergyThreads, P == 32 ? 4 : 1) step_post_ker
   }
 }
 
-cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked,
-                             bool half, SetupExt next, const EnergyParams* ep, EnergyMon* mon, cudaStream_t st) {
+cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked, bool half,
+                             SetupExt next, bool dev, const EnergyParams* ep, EnergyMon* mon, int num_sms,
+                             cudaStream_t st) {
   EnergyParams e{0, 1, 0.0};
   if (ep) e = *ep;  // the energy monitor in the last block (small systems)
-  const int p = post_particles(s.N);
+  const int p = !chunked && s.N > 32LL * 4 * num_sms ? kEnergyThreads : post_particles(s.N);
   const unsigned blocks = (unsigned)((s.N + p - 1) / p);
-  const int c = chunked ? 1 : 0, h = half ? 1 : 0;
+  const int c = chunked ? 1 : 0, h = half ? 1 : 0, dv = dev ? 1 : 0;
+  if (p == kEnergyThreads) {
+    step_post_kernel<kEnergyThreads><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, dv, e, mon);
+    return cudaGetLastError();
+  }
   if (p == 8)
-    step_post_kernel<8><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, e, mon);
+    step_post_kernel<8><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, dv, e, mon);
   else if (p == 16)
-    step_post_kernel<16><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, e, mon);
+    step_post_kernel<16><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, dv, e, mon);
   else
-    step_post_kernel<32><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, e, mon);
+    step_post_kernel<32><<<blocks, kEnergyThreads, 0, st>>>(s, b, ap, c, h, next, dv, e, mon);
   return cudaGetLastError();
 }
 
