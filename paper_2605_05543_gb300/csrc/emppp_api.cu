@@ -126,7 +126,7 @@ struct emppp_ctx {
   cudaGraphExec_t graph_exec[kGraphs] = {};
   int graph_launches[kGraphs] = {};  // kernels per replayed step
   unsigned char graph_key[sizeof(emppp_options) + sizeof(BextParams) + sizeof(AdaptParams) +
-                          sizeof(EnergyParams)];  // configuration of the variants
+                          sizeof(EnergyParams) + sizeof(SetupExt)];  // configuration of the variants
   bool graph_valid[kGraphs] = {};
   // Steps since the target order was computed (-1: not for the present state). The order is a
   // permutation of each bunch whatever its age, and a target's sum runs over the sources in a fixed
@@ -136,6 +136,9 @@ struct emppp_ctx {
   // the path whose slot tables and source vectors the last step's post-pair launch formed for the present state (none:
   // the next step starts with its own set-up launch); every other call that touches the state or these resets it
   SetupExt prepared = SetupExt::none;
+  // a call on this handle was made while the caller captured its stream: a replay of that graph, which the host cannot
+  // see, may move the state at any time, so no step relies on what the one before it prepared
+  bool caller_graph = false;
 };
 
 // steps between two computations of the spatial target order
@@ -456,7 +459,16 @@ SetupExt setup_of(emppp_handle h) {
   return h->opt.precision == EMPPP_MIXED ? SetupExt::mixed : SetupExt::fp64;
 }
 SetupExt next_setup_of(emppp_handle h) {
-  return h->opt.field_point == EMPPP_FIELD_HALF_STEP ? SetupExt::none : setup_of(h);
+  return h->caller_graph || h->opt.field_point == EMPPP_FIELD_HALF_STEP ? SetupExt::none : setup_of(h);
+}
+
+// notes a capture of the handle's stream by the caller
+void note_caller_capture(emppp_handle h) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess)
+    cudaGetLastError();  // (the legacy stream beside a capture elsewhere: the launches report it)
+  else if (cap != cudaStreamCaptureStatusNone)
+    h->caller_graph = true;
 }
 
 // The target order of the next step. Small systems on the mixed path go without: a few target tiles gain less from it
@@ -544,12 +556,14 @@ int graph_variant(OrderMode order, bool set_up) { return order + (set_up ? kOrde
 
 emppp_status capture_step(emppp_handle h, const BextParams& bp, OrderMode order, bool set_up) {
   const int v = graph_variant(order, set_up);
-  unsigned char key[sizeof(emppp_options) + sizeof(BextParams) + sizeof(AdaptParams) + sizeof(EnergyParams)];
+  unsigned char key[sizeof(h->graph_key)];
+  const SetupExt next = next_setup_of(h);
   memset(key, 0, sizeof(key));
   memcpy(key, &h->opt, sizeof(emppp_options));
   memcpy(key + sizeof(emppp_options), &bp, sizeof(BextParams));
   memcpy(key + sizeof(emppp_options) + sizeof(BextParams), &h->adapt, sizeof(AdaptParams));
   memcpy(key + sizeof(emppp_options) + sizeof(BextParams) + sizeof(AdaptParams), &h->energy, sizeof(EnergyParams));
+  memcpy(key + sizeof(key) - sizeof(SetupExt), &next, sizeof(SetupExt));
   if (memcmp(key, h->graph_key, sizeof(key)) != 0) {
     const int age = h->order_age;
     invalidate_graph(h);
@@ -961,16 +975,14 @@ EMPPP_API emppp_status emppp_step(emppp_handle h, int64_t nsteps, const emppp_be
   if ((st = update_schedule(h)) != EMPPP_OK) return st;
   const bool use_graph = h->opt.graphs && !h->opt.timing && h->stream != nullptr && nsteps > 1;
   NvtxRange r_step(use_graph ? "emppp_step (graph replay)" : "emppp_step");
-  // in a capture of the caller's own the step may be replayed from any state: it carries its set-up launch
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool captured = cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  note_caller_capture(h);
   long long pairs_per_step = 0;
   if (h->opt.pair_fields)
     for (int b = 0; b < h->nbunch; b++) pairs_per_step += (long long)h->hb[b].n * (h->hb[b].n - 1);
   for (int64_t k = 0; k < nsteps; k++) {
     int nk = 0;
     const OrderMode order = order_mode(h);
-    const bool set_up = captured || h->prepared == SetupExt::none || h->prepared != setup_of(h);
+    const bool set_up = h->caller_graph || h->prepared == SetupExt::none || h->prepared != setup_of(h);
     h->prepared = SetupExt::none;  // also if this step fails
     if (use_graph) {
       if ((st = capture_step(h, bp, order, set_up)) != EMPPP_OK) return st;
@@ -984,7 +996,7 @@ EMPPP_API emppp_status emppp_step(emppp_handle h, int64_t nsteps, const emppp_be
     }
     // (without an order: the next step forms one)
     h->order_age = order == kOrderRefresh ? 0 : (order == kOrderReuse ? h->order_age + 1 : kOrderEvery - 1);
-    if (!captured) h->prepared = next_setup_of(h);
+    h->prepared = next_setup_of(h);
     h->launches += nk;
     h->pairs_acc += pairs_per_step;
     h->steps_acc += 1;
@@ -1036,6 +1048,7 @@ EMPPP_API emppp_status emppp_transport(emppp_handle h, int64_t nsteps, double dt
   BextParams bp;
   if ((st = convert_bext(bext, &bp)) != EMPPP_OK) return st;
   if ((st = sync_time(h)) != EMPPP_OK) return st;
+  note_caller_capture(h);
   h->prepared = SetupExt::none;
   const int64_t kChunk = 4096;
   for (int64_t done = 0; done < nsteps;) {
