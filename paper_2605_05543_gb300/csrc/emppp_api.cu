@@ -462,13 +462,14 @@ SetupExt next_setup_of(emppp_handle h) {
   return h->caller_graph || h->opt.field_point == EMPPP_FIELD_HALF_STEP ? SetupExt::none : setup_of(h);
 }
 
-// notes a capture of the handle's stream by the caller
-void note_caller_capture(emppp_handle h) {
+// whether the caller is capturing the handle's stream, which the handle remembers
+bool caller_captures(emppp_handle h) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess)
     cudaGetLastError();  // (the legacy stream beside a capture elsewhere: the launches report it)
   else if (cap != cudaStreamCaptureStatusNone)
     h->caller_graph = true;
+  return cap != cudaStreamCaptureStatusNone;
 }
 
 // The target order of the next step. Small systems on the mixed path go without: a few target tiles gain less from it
@@ -975,7 +976,7 @@ EMPPP_API emppp_status emppp_step(emppp_handle h, int64_t nsteps, const emppp_be
   if ((st = update_schedule(h)) != EMPPP_OK) return st;
   const bool use_graph = h->opt.graphs && !h->opt.timing && h->stream != nullptr && nsteps > 1;
   NvtxRange r_step(use_graph ? "emppp_step (graph replay)" : "emppp_step");
-  note_caller_capture(h);
+  const bool captured = caller_captures(h);
   long long pairs_per_step = 0;
   if (h->opt.pair_fields)
     for (int b = 0; b < h->nbunch; b++) pairs_per_step += (long long)h->hb[b].n * (h->hb[b].n - 1);
@@ -994,8 +995,8 @@ EMPPP_API emppp_status emppp_step(emppp_handle h, int64_t nsteps, const emppp_be
       if (h->opt.timing && h->ev_used < emppp_ctx::kTimedSteps) ev = &h->events[4 * h->ev_used++];
       if ((st = enqueue_step(h, bp, ev, &nk, order, set_up)) != EMPPP_OK) return st;
     }
-    // (without an order: the next step forms one)
-    h->order_age = order == kOrderRefresh ? 0 : (order == kOrderReuse ? h->order_age + 1 : kOrderEvery - 1);
+    // (without an order: the next step forms one; a captured step has formed none yet)
+    if (!captured) h->order_age = order == kOrderRefresh ? 0 : (order == kOrderReuse ? h->order_age + 1 : kOrderEvery - 1);
     h->prepared = next_setup_of(h);
     h->launches += nk;
     h->pairs_acc += pairs_per_step;
@@ -1048,7 +1049,7 @@ EMPPP_API emppp_status emppp_transport(emppp_handle h, int64_t nsteps, double dt
   BextParams bp;
   if ((st = convert_bext(bext, &bp)) != EMPPP_OK) return st;
   if ((st = sync_time(h)) != EMPPP_OK) return st;
-  note_caller_capture(h);
+  caller_captures(h);
   h->prepared = SetupExt::none;
   const int64_t kChunk = 4096;
   for (int64_t done = 0; done < nsteps;) {
