@@ -143,6 +143,11 @@ struct emppp_ctx {
 
 // steps between two computations of the spatial target order
 constexpr int kOrderEvery = 16;
+// Turns of the post-pair launch's table threads beyond which a step's slot tables are left to the set-up launch, which has
+// a thread per slot. A turn is a chain of FP64 operations, 0.4 us. 32 steps on the mixed path, tables in the post-pair
+// launch and in a set-up launch: 8 particles (64 threads), 512 slots 0.81 ms and 0.88, 1024 slots 1.00 and 0.88, 65536 slots
+// 26.5 and 0.94; 32 particles (256 threads), 2048 slots 0.87 and 0.95, 4096 slots 1.08 and 0.95.
+constexpr long long kTableTurns = 8;
 // particles up to which the mixed path goes without the order, and without it in the first step from a new state
 constexpr long long kUnorderedMixed = 1024, kLateOrderMixed = 2048;
 
@@ -459,7 +464,8 @@ SetupExt setup_of(emppp_handle h) {
   return h->opt.precision == EMPPP_MIXED ? SetupExt::mixed : SetupExt::fp64;
 }
 SetupExt next_setup_of(emppp_handle h) {
-  return h->caller_graph || h->opt.field_point == EMPPP_FIELD_HALF_STEP ? SetupExt::none : setup_of(h);
+  if (h->caller_graph || h->opt.field_point == EMPPP_FIELD_HALF_STEP) return SetupExt::none;
+  return h->D <= kTableTurns * post_table_threads(h->N) ? setup_of(h) : SetupExt::none;
 }
 
 // whether the caller is capturing the handle's stream, which the handle remembers

@@ -346,6 +346,7 @@ cudaError_t launch_zero_self(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_step_post(const DeviceState& s, const BextParams& b, const AdaptParams& ap, bool chunked, bool half,
                              SetupExt next, bool dev, const EnergyParams* ep, EnergyMon* mon, int num_sms,
                              cudaStream_t st);
+long long post_table_threads(long long n);  // threads that form the next step's slot tables (fewest, for n particles)
 cudaError_t launch_reduce_partials(const DeviceState& s, cudaStream_t st);
 cudaError_t launch_half_slot(const DeviceState& s, cudaStream_t st);
 // stage2.cu

@@ -171,6 +171,11 @@ struct ChunkSums {
 // SM's FP64 pipe for 16 cycles however few of its lanes are active), a full warp of pushers for large ones
 int post_particles(long long n) { return n <= 2432 ? 8 : (n <= 4864 ? 16 : 32); }
 
+long long post_table_threads(long long n) {
+  const int p = post_particles(n);
+  return (n + p - 1) / p * (kEnergyThreads - kSumThreads);
+}
+
 template <int P>
 __global__ void __launch_bounds__(kEnergyThreads) reduce_partials_kernel(DeviceState s) {
   __shared__ ChunkSums<P> sums;
