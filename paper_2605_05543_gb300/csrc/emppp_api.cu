@@ -79,8 +79,9 @@ struct emppp_ctx {
     int err;
     StepState state;
   };
-  HostPage* page = nullptr;
-  double* frames = nullptr;  // page-locked: first positions and velocities of the bunches [nbunch][6], then [D]
+  HostPage* page = nullptr;    // one page-locked allocation with the two arrays below
+  double* frames = nullptr;    // first positions and velocities of the bunches [nbunch][6], then [D]
+  double* results = nullptr;   // [kPageResults] (or 6N, if fewer) results on their way to host arrays
   std::vector<void*> allocs;
   // bunches
   int nbunch = 1;
@@ -141,6 +142,8 @@ struct emppp_ctx {
   bool caller_graph = false;
 };
 
+// doubles of a call's host results that pass through page-locked memory
+constexpr size_t kPageResults = 8192;
 // steps between two computations of the spatial target order
 constexpr int kOrderEvery = 16;
 // Turns of the post-pair launch's table threads beyond which a step's slot tables are left to the set-up launch, which has
@@ -396,6 +399,63 @@ emppp_status to_device(emppp_handle h, double* dst, const double* src, size_t n,
 emppp_status from_device(emppp_handle h, double* dst, const double* src, size_t n, int is_dev) {
   CU(cudaMemcpyAsync(dst, src, n * sizeof(double), is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                      h->stream));
+  return EMPPP_OK;
+}
+
+// whether a kernel on the handle's device may write doubles at p
+bool writable_by_kernel(emppp_handle h, const double* p) {
+  if (!p) return true;
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == h->device);
+}
+
+// Results into the caller's arrays: the present positions to x and [3N] from sa to da and sb to db (any destination may be
+// NULL), with the device's time if it is stale. An array of the caller's is left as it was when the call reports a
+// device error. One wait serves the results and the error word: on the device the kernel that copies looks at the word,
+// for the host the results land in page-locked memory first. Results too many for that, or for memory that only a
+// copy reaches, wait for the word by themselves.
+emppp_status deliver(emppp_handle h, double* x, double* da, const double* sa, double* db, const double* sb, int is_dev) {
+  emppp_status st;
+  const size_t n3 = 3 * (size_t)h->N, bytes = n3 * sizeof(double);
+  double* const dst[3] = {x, da, db};
+  const bool direct = is_dev && writable_by_kernel(h, x) && writable_by_kernel(h, da) && writable_by_kernel(h, db);
+  const bool paged = !is_dev && 2 * n3 <= kPageResults;
+  if ((st = request_time(h)) != EMPPP_OK) return st;
+  if (!direct && !paged && (st = read_err(h)) != EMPPP_OK) return st;
+  const double* src[3] = {h->staging, sa, sb};
+  if (direct) {
+    if (x || da || db) {
+      CU(launch_deliver(h->ds, x, da, sa, db, sb, h->stream));
+      h->launches += 1;
+    }
+  } else {
+    if (x) {
+      CU(launch_deliver(h->ds, h->staging, nullptr, nullptr, nullptr, nullptr, h->stream));
+      h->launches += 1;
+    }
+    size_t at = 0;
+    for (int k = 0; k < 3; k++) {
+      if (!dst[k]) continue;
+      CU(cudaMemcpyAsync(paged ? h->results + at : dst[k], src[k], bytes,
+                         is_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
+      at += n3;
+    }
+  }
+  if ((st = request_err(h)) != EMPPP_OK) return st;
+  CU(cudaStreamSynchronize(h->stream));
+  if ((st = check_err(h)) != EMPPP_OK) return st;
+  size_t at = 0;
+  for (int k = 0; paged && k < 3; k++) {
+    if (!dst[k]) continue;
+    memcpy(dst[k], h->results + at, bytes);
+    at += n3;
+  }
+  take_time(h);
   return EMPPP_OK;
 }
 
@@ -727,10 +787,14 @@ emppp_status create_impl(int32_t nbunch, const int64_t* nper, int32_t history_de
   s.sched = c->d_sched;
   s.bunch_of = c->d_bunch_of;
   s.mlp_image = c->mlp_image;
-  e = cudaMallocHost(reinterpret_cast<void**>(&c->page), sizeof(emppp_ctx::HostPage));
-  if (e == cudaSuccess)
-    e = cudaMallocHost(reinterpret_cast<void**>(&c->frames), sizeof(double) * (6 * (size_t)nbunch + D));
-  if (e != cudaSuccess) {
+  static_assert(sizeof(emppp_ctx::HostPage) % sizeof(double) == 0, "the arrays follow the words");
+  const size_t nframes = 6 * (size_t)nbunch + D;
+  e = cudaMallocHost(reinterpret_cast<void**>(&c->page),
+                     sizeof(emppp_ctx::HostPage) + sizeof(double) * (nframes + std::min(6 * N, kPageResults)));
+  if (e == cudaSuccess) {
+    c->frames = reinterpret_cast<double*>(c->page + 1);
+    c->results = c->frames + nframes;
+  } else {
     cudaGetLastError();
     emppp_destroy(c);
     return fail(EMPPP_ERR_OOM, "page-locked host words: %s", cudaGetErrorString(e));
@@ -807,7 +871,6 @@ EMPPP_API void emppp_destroy(emppp_handle h) {
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   for (void* p : h->allocs) cudaFree(p);
   if (h->page) cudaFreeHost(h->page);
-  if (h->frames) cudaFreeHost(h->frames);
   delete h;
 }
 
@@ -1078,21 +1141,7 @@ EMPPP_API emppp_status emppp_get_state(emppp_handle h, double* x, double* u, dou
   emppp_status st = check_handle(h);
   if (st != EMPPP_OK) return st;
   if (!h->has_state) return fail(EMPPP_ERR_STATE, "no state: call emppp_set_particles first");
-  if ((st = request_err(h)) != EMPPP_OK || (st = request_time(h)) != EMPPP_OK) return st;
-  const size_t N = (size_t)h->N;
-  if (x) {
-    h->launches += 1;
-    if (is_device_ptr) {
-      CU(launch_gather_positions(h->ds, x, h->stream));
-    } else {
-      CU(launch_gather_positions(h->ds, h->staging, h->stream));
-      if ((st = from_device(h, x, h->staging, 3 * N, 0)) != EMPPP_OK) return st;
-    }
-  }
-  if (u && (st = from_device(h, u, h->ds.u, 3 * N, is_device_ptr)) != EMPPP_OK) return st;
-  CU(cudaStreamSynchronize(h->stream));
-  if ((st = check_err(h)) != EMPPP_OK) return st;
-  take_time(h);
+  if ((st = deliver(h, x, u, h->ds.u, nullptr, nullptr, is_device_ptr)) != EMPPP_OK) return st;
   if (t_now) *t_now = h->t;
   if (n_now) *n_now = h->n;
   return EMPPP_OK;
@@ -1102,12 +1151,7 @@ EMPPP_API emppp_status emppp_get_fields(emppp_handle h, double* E, double* B, in
   emppp_status st = check_handle(h);
   if (st != EMPPP_OK) return st;
   if (!h->has_state) return fail(EMPPP_ERR_STATE, "no state: call emppp_set_particles first");
-  if ((st = request_err(h)) != EMPPP_OK) return st;
-  const size_t N = (size_t)h->N;
-  if (E && (st = from_device(h, E, h->ds.Eself, 3 * N, is_device_ptr)) != EMPPP_OK) return st;
-  if (B && (st = from_device(h, B, h->ds.Bout, 3 * N, is_device_ptr)) != EMPPP_OK) return st;
-  CU(cudaStreamSynchronize(h->stream));
-  return check_err(h);
+  return deliver(h, nullptr, E, h->ds.Eself, B, h->ds.Bout, is_device_ptr);
 }
 
 EMPPP_API emppp_status emppp_get_stats(emppp_handle h, emppp_stats* out) {

@@ -332,7 +332,8 @@ cudaError_t launch_prep(const DeviceState& s, cudaStream_t st);
 enum class SetupExt { none, mixed, fp64 };
 cudaError_t launch_setup(const DeviceState& s, SetupExt ext, cudaStream_t st);
 cudaError_t launch_reset_scale(const DeviceState& s, cudaStream_t st);
-cudaError_t launch_gather_positions(const DeviceState& s, double* x, cudaStream_t st);
+cudaError_t launch_deliver(const DeviceState& s, double* x, double* da, const double* sa, double* db, const double* sb,
+                           cudaStream_t st);
 // pair_fp64.cu
 // kernel variant of the FP64 pair path: 0 the method, 1 with the adaptive time step's reduction, 2 the
 // midpoint reconstruction eq:mid

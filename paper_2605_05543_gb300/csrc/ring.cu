@@ -227,14 +227,15 @@ __global__ void reset_scale_kernel(DeviceState s) {
   s.adapt_info[2] = 0.0;
 }
 
-__global__ void gather_positions_kernel(DeviceState s, double* __restrict__ x) {
-  const long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= s.N) return;
-  const int pn = (int)(s.state->n % s.D);
-  const double* r = s.rec64 + ((size_t)j * s.D + pn) * 6;
-  x[3 * j] = r[0];
-  x[3 * j + 1] = r[1];
-  x[3 * j + 2] = r[2];
+// results into arrays of the caller's, unless a device error is pending: the present positions to x, and [3N] from sa to
+// da and sb to db (each destination may be null)
+__global__ void deliver_kernel(DeviceState s, double* __restrict__ x, double* __restrict__ da, const double* __restrict__ sa,
+                               double* __restrict__ db, const double* __restrict__ sb) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= 3 * s.N || *s.err != 0) return;
+  if (x) x[q] = s.rec64[((size_t)(q / 3) * s.D + (size_t)(s.state->n % s.D)) * 6 + q % 3];
+  if (da) da[q] = sa[q];
+  if (db) db[q] = sb[q];
 }
 
 static inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
@@ -292,8 +293,9 @@ cudaError_t launch_reset_scale(const DeviceState& s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_positions(const DeviceState& s, double* x, cudaStream_t st) {
-  gather_positions_kernel<<<blocks_for(s.N, 256), 256, 0, st>>>(s, x);
+cudaError_t launch_deliver(const DeviceState& s, double* x, double* da, const double* sa, double* db, const double* sb,
+                           cudaStream_t st) {
+  deliver_kernel<<<blocks_for(3 * s.N, 256), 256, 0, st>>>(s, x, da, sa, db, sb);
   return cudaGetLastError();
 }
 
