@@ -92,11 +92,11 @@ __global__ void __launch_bounds__(32 * kScatterSlots) scatter_history_kernel(Dev
     const size_t at = ((size_t)k * s.N + j) * 3, next = at + (size_t)s.N * 3;
     const double w0 = __ldg(W + at), w1 = __ldg(W + at + 1), w2 = __ldg(W + at + 2);
     const double v0 = __ldg(V + at), v1 = __ldg(V + at + 1), v2 = __ldg(V + at + 2);
-    // 1 / gamma^2 = 1 - v.v / c^2 and its reciprocal without divisions (both are rounded to FP32)
-    const double ig2 = 1.0 - (v0 * v0 + v1 * v1 + v2 * v2) * (1.0 / (kC * kC));
+    double gamma2, ig2;
+    record_gamma2(v0, v1, v2, gamma2, ig2);
     float4 q[3];
     const BunchDesc& bd = s.bunches[s.nbunch == 1 ? 0 : s.bunch_of[j]];
-    shadow_record(bd.origin, bd.beta_ref, w0, w1, w2, v0, v1, v2, recip_refined(ig2), ig2, q);
+    shadow_record(bd.origin, bd.beta_ref, w0, w1, w2, v0, v1, v2, gamma2, ig2, q);
     if (!last || k + 1 < nslots) {  // the next slot, which may be another block's
       int p = (int)(((long long)p_first + k) % s.D);
       const double t = s.slot_t[p];

@@ -56,6 +56,25 @@ __device__ __forceinline__ double gamma2_of_v(double v0, double v1, double v2) {
   return 1.0 / (1.0 - (v0 * v0 + v1 * v1 + v2 * v2) / (kC * kC));
 }
 
+// Its inverse and gamma^2 as an FP32 record holds them, without the three divisions: the same FP32 values as 1 / g and g
+// = gamma2_of_v. The quotient v.v / c^2 is the correctly rounded one (a product with the rounded reciprocal and one
+// correction by the exact remainder); 1 / gamma2_of_v is within an ulp and a half of m = 1 - that, and recip_refined(m) within
+// two of 1 / m, so FP32 rounds both to the same value unless they lie within eight ulps of the middle of two FP32
+// values, where the divisions decide (also for |v| >= c).
+__device__ __forceinline__ void record_gamma2(double v0, double v1, double v2, double& gamma2, double& inv_gamma2) {
+  constexpr double cc = kC * kC, rc = 1.0 / cc;
+  const double vv = v0 * v0 + v1 * v1 + v2 * v2;
+  double q = vv * rc;
+  q = fma(fma(-q, cc, vv), rc, q);
+  inv_gamma2 = 1.0 - q;
+  gamma2 = recip_refined(inv_gamma2);
+  auto near_middle = [](double x) { return ((unsigned)__double2loint(x) & 0x1fffffffu) - (0x10000000u - 8u) <= 16u; };
+  if (!positive_normal(inv_gamma2) || near_middle(gamma2) || near_middle(inv_gamma2)) {
+    gamma2 = 1.0 / inv_gamma2;
+    inv_gamma2 = 1.0 / gamma2;
+  }
+}
+
 // gamma^2 of a proper velocity: 1 + u.u / c^2 (no cancellation)
 __device__ __forceinline__ double gamma2_of_u(double u0, double u1, double u2) {
   return 1.0 + (u0 * u0 + u1 * u1 + u2 * u2) / (kC * kC);
