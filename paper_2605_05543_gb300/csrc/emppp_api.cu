@@ -956,8 +956,7 @@ EMPPP_API emppp_status emppp_set_history(emppp_handle h, int64_t n, int32_t nslo
       if ((st = to_device(h, h->staging + 3 * N, V + (size_t)s * N * 3, 3 * N, 0)) != EMPPP_OK) return st;
       CU(launch_scatter_slot(h->ds, (p_first + s) % h->D, s > 0 ? hT[s] - hT[s - 1] : 0.0, h->staging, h->staging + 3 * N,
                              h->stream));
-      h->launches += 1;
-      CU(cudaStreamSynchronize(h->stream));  // staging is reused by the next slot
+      h->launches += 1;  // (the next slot's copies into the staging arrays follow in the stream)
     }
   }
   const double* du = u;
