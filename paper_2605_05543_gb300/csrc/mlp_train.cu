@@ -81,12 +81,13 @@ __global__ void train_image_kernel(const float* __restrict__ p, TrainImage* __re
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-struct TrainSmem {
+struct __align__(16) TrainSmem {  // (rows of A1 and dH2 are read as float4)
   float A1[kRows][kLd], A2[kRows][kLd], dH1[kRows][kLd], dH2[kRows][kLd];
   float X[kRows][12];
   float z[kRows][4][kH / 8 + 1];  // the output's terms per row, fragment column pair and n-tile
   float dz[kRows];
 };
+static_assert(alignof(TrainSmem) >= sizeof(float4) && kLd * sizeof(float) % sizeof(float4) == 0, "float4 rows");
 
 // rows [row0, row0 + rows) of X [m][10] and T [m]; per-block gradients of sum_r (z_r - T_r)^2 / norm
 // (img and p are written by the launch that may still be running: no __restrict__, so that their loads stay behind the
