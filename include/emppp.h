@@ -112,8 +112,11 @@ typedef struct {
   int64_t out_of_history;  /* pairs with t_r older than the history (eq:linear2) */
   int64_t shortcut;        /* pairs bracketed by the near-field shortcut */
   int64_t bisection;       /* pairs bracketed by the search */
-  int64_t node_tests;      /* evaluations of c (t - t_k) <= |r - w_k| over all pairs */
-  int64_t guard_fallbacks; /* node tests decided in FP64 after an inconclusive FP32 test */
+  int64_t node_tests;      /* node tests c (t - t_k) <= |r - w_k| settled over all pairs: evaluated, or on the mixed
+                              path shown by a bound that needs no record of the slot */
+  int64_t guard_fallbacks; /* evaluations in FP64 after an FP32 one too coarse to use: node tests between the
+                              guard-band thresholds and, on the mixed path, separations from a fast source's line
+                              (formed twice, and counted twice, for a pair that a bound leaves to its node test) */
   int64_t kernel_launches; /* kernels launched by the library (cumulative since emppp_create) */
   double pair_ms;          /* device time of the pair evaluations (timing option on, else 0) */
   double step_ms;          /* device time of whole steps (timing option on, else 0) */
@@ -126,10 +129,11 @@ typedef struct {
 
 /* Work split and tile shape of the pair kernel: items_per_block work items (bunch, source chunk, target
  * tile) per resident block of 128 threads, which sets the sources per chunk; target_order 1 sorts the
- * targets spatially each step (both paths; the fields do not depend on it; a step of a system of at most
- * 2048 particles on the mixed path skips it). The tile shape: targets_per_block targets per work item and
- * thread block (64, 128 or 256; a mixed-path block stages half that many sources per tile) and, on the
- * mixed path, sources_per_sum sources per FP32 partial sum before the compensated addition (8, 16 or 32;
+ * targets spatially each step (both paths; the fields do not depend on it; on the mixed path systems of at
+ * most 1024 particles go without it, and those of at most 2048 in the first step from a new state). The tile
+ * shape: targets_per_block targets per work item and thread block (64, 128 or 256; a mixed-path block stages
+ * half that many sources per tile) and, on the mixed path, sources_per_sum sources per FP32 partial sum before
+ * the compensated addition (8, 16 or 32;
  * 16 and 32 only at 128 targets per block). The FP64 path ignores sources_per_sum. The shape changes the order
  * of each target's sum, so fields of different shapes agree within rounding, not bit for bit; the
  * adaptive time step and the comparison variants run the default shape (128, 8). history_window nonzero
@@ -218,12 +222,12 @@ EMPPP_API emppp_status emppp_handoff(emppp_handle h, const double* center);
 EMPPP_API emppp_status emppp_transport(emppp_handle h, int64_t nsteps, double dt, const emppp_bext* bext);
 
 /* Present positions x [3n], proper velocities u [3n] (host or device, either may be NULL), time
- * and step index (either may be NULL). Synchronises the stream. */
+ * and step index (either may be NULL). Synchronises the stream. Nothing is written on failure. */
 EMPPP_API emppp_status emppp_get_state(emppp_handle h, double* x, double* u, double* t_now, int64_t* n_now,
                                        int32_t is_device_ptr);
 
 /* Fields used by the last completed step: self E [3n] and B [3n] = self + B_ext(x^{n+1/2})
- * (host or device, either may be NULL). Synchronises the stream. */
+ * (host or device, either may be NULL). Synchronises the stream. Nothing is written on failure. */
 EMPPP_API emppp_status emppp_get_fields(emppp_handle h, double* E, double* B, int32_t is_device_ptr);
 
 /* Counters accumulated since the last emppp_reset_stats (or create / set_particles / set_history).
