@@ -446,9 +446,9 @@ emppp_status deliver(emppp_handle h, double* x, double* da, const double* sa, do
       at += n3;
     }
   }
-  if ((st = request_err(h)) != EMPPP_OK) return st;
+  if ((direct || paged) && (st = request_err(h)) != EMPPP_OK) return st;
   CU(cudaStreamSynchronize(h->stream));
-  if ((st = check_err(h)) != EMPPP_OK) return st;
+  if ((direct || paged) && (st = check_err(h)) != EMPPP_OK) return st;
   size_t at = 0;
   for (int k = 0; paged && k < 3; k++) {
     if (!dst[k]) continue;
