@@ -273,9 +273,13 @@ emppp_status update_schedule(emppp_handle c) {
   //   N = 16381 with the guess: 256 29434, 64 28638. (The partial sums, 200 MB there, cost less than they save.)
   //   Mixed, closed form, 251 slots: N = 4096: 256 429, 64 297, 32 288; N = 8192: 256 810, 128 724, 64 700, 32 726;
   //   N = 16384: 256 2252, 128 2197, 64 2239. 16 bunches of 188 on average: 256 824, 64 652, 32 657.
+  // Where the target tiles alone are one and a half rounds of blocks, a bunch of at most 128 stays in one chunk (mixed):
+  // 16 steps of 4000 bunches of 64 8.60 ms in chunks of 32, 7.41 in one; 2000 of 128 8.72 and 7.41; 3000 of 100 10.32 and
+  // 8.56; but 1500 of 64 (1.2 rounds) 3.43 and 3.52, and 1000 of 200 9.08 in chunks of 32, 9.28 of 128.
   // With the adaptive step the mixed path's chunks are whole tiles of at least 256 sources, or one round: its step
   // size follows the last bit of FP32 sums, so their grouping stays what it was for runs made so far.
   const bool whole = mixed && ad;
+  const bool many_tiles = 2 * total_tiles >= 3 * Rreal;
   auto chunks = [&](long long n, bool small) -> long long {
     const long long one_round = Rreal / total_tiles > 1 ? Rreal / total_tiles : 1;
     const long long many = ((mixed ? 2LL : 4LL) * c->items_per_block * Rsched + tiles128 - 1) / tiles128;
@@ -287,7 +291,7 @@ emppp_status update_schedule(emppp_handle c) {
     else if (whole)
       nchunk = small ? of(one_round, kMin) : of(many, 256);
     else
-      nchunk = std::max(of(one_round, kMin), mixed ? of(std::min(many, 128LL), 32) : of(many, 8));
+      nchunk = std::max(of(one_round, kMin), mixed ? of(std::min(many, 128LL), many_tiles && n <= 128 ? 128 : 32) : of(many, 8));
     nchunk = std::max(1LL, std::min(nchunk, (long long)c->ds.max_split));
     const long long chunk = (n + nchunk - 1) / nchunk;
     long long unit = kMin;
