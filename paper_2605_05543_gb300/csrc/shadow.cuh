@@ -57,20 +57,18 @@ __device__ __forceinline__ double gamma2_of_v(double v0, double v1, double v2) {
 }
 
 // Its inverse and gamma^2 as an FP32 record holds them, without the three divisions: the same FP32 values as 1 / g and g
-// = gamma2_of_v. The quotient v.v / c^2 is the correctly rounded one (a product with the rounded reciprocal and one
-// correction by the exact remainder); 1 / gamma2_of_v is within an ulp and a half of m = 1 - that, and recip_refined(m) within
-// two of 1 / m, so FP32 rounds both to the same value unless they lie within eight ulps of the middle of two FP32
-// values, where the divisions decide (also for |v| >= c).
+// = gamma2_of_v. The rounded constant 1 / c^2, the quotient and the difference move 1 - v.v / c^2 by at most 2.5 * 2^-53, 2.5
+// gamma^2 ulps of it and of its reciprocal, to which recip_refined and the divisions add four; FP32 rounds both ways to
+// the same value unless they lie that near the middle of two FP32 values, where the divisions decide (and for |v| >= c).
 __device__ __forceinline__ void record_gamma2(double v0, double v1, double v2, double& gamma2, double& inv_gamma2) {
-  constexpr double cc = kC * kC, rc = 1.0 / cc;
   const double vv = v0 * v0 + v1 * v1 + v2 * v2;
-  double q = vv * rc;
-  q = fma(fma(-q, cc, vv), rc, q);
-  inv_gamma2 = 1.0 - q;
+  inv_gamma2 = fma(-vv, 1.0 / (kC * kC), 1.0);
   gamma2 = recip_refined(inv_gamma2);
-  auto near_middle = [](double x) { return ((unsigned)__double2loint(x) & 0x1fffffffu) - (0x10000000u - 8u) <= 16u; };
-  if (!positive_normal(inv_gamma2) || near_middle(gamma2) || near_middle(inv_gamma2)) {
-    gamma2 = 1.0 / inv_gamma2;
+  const float g = rounded_to_float(gamma2);
+  const unsigned near = 8u + 4u * (unsigned)fminf(g, 6e7f);
+  auto near_middle = [&](double x) { return ((unsigned)__double2loint(x) & 0x1fffffffu) - (0x10000000u - near) <= 2u * near; };
+  if (!positive_normal(inv_gamma2) || g > 6e7f || near_middle(gamma2) || near_middle(inv_gamma2)) {
+    gamma2 = gamma2_of_v(v0, v1, v2);
     inv_gamma2 = 1.0 / gamma2;
   }
 }
