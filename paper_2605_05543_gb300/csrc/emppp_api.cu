@@ -121,8 +121,8 @@ struct emppp_ctx {
   static constexpr int kTimedSteps = 1024;
   std::vector<cudaEvent_t> events;
   int ev_used = 0;
-  // one step captured in two variants, replayed by emppp_step: [1] recomputes the spatial target order,
-  // [0] reuses the last one
+  // one step captured by the library, replayed by emppp_step: a variant for each OrderMode, with the set-up launch and
+  // without (graph_variant)
   cudaGraph_t graph[kGraphs] = {};
   cudaGraphExec_t graph_exec[kGraphs] = {};
   int graph_launches[kGraphs] = {};  // kernels per replayed step

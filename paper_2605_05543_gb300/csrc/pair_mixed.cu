@@ -59,7 +59,7 @@ namespace {
 
 // Resident blocks per SM, of 128 threads: 8 at 64 registers (N = 32768: 7.69 ms; 7 at 72 registers 8.08, 9 at 56 with
 // spills 10.0). The history-window shape holds more state across a pair and spills 132 bytes at 64 registers: 7 blocks
-// (N = 16384: 3.21 ms against 3.88 at 8 and 3.41 at 6).
+// (N = 16384: a step in 2.89 ms against 3.54 at 8 and 3.04 at 6).
 // The guessed-search instances of the adaptive step hold the textbook forms and the list of FP64 lines: 112 / 152 bytes of
 // spill stores / loads at 64 registers, 36 / 64 at 72. So 7 blocks (gamma 3, N = 5000: 1.30 ms against 1.37 at 8; 12000:
 // 4.23 and 4.31), but 8 where all items fit one round of those alone (3000: 422 us against 450; 3900: 661 and 736).
