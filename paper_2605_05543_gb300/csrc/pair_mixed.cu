@@ -73,8 +73,8 @@ constexpr int mixed_min_blocks(int shape, bool adapt, int prop) {
 constexpr float kC0Guard = 2.0e-6f / 5.9604644775390625e-08f;
 // FP64 separation from the source's line when u L1 / (2 sqrt(Dh)) exceeds 1e-6: kLineGuard = 2e-6 / u. kappa then moves by
 // 2e-6 of itself, and a field, which goes with its cube, by 6e-6 (at twice the bound by up to 1.2e-5: in 720 histories
-// of gamma 6 to 40 the largest error of c B against the oracle was 9.8e-6 of the target's sum, now 4.1e-6, at 0.8 % of
-// a step of 16 bunches of gamma 2 to 20).
+// of gamma 6 to 40 the largest error of c B against the oracle was 9.8e-6 of the target's sum, now 4.1e-6, at 0.3 % of
+// a step of 16 bunches of gamma 2 to 20 with 201 slots, 1.4 % of 20 with 901).
 constexpr float kLineGuard = 2.0e-6f / 5.9604644775390625e-08f;
 // FP64 recomputation of X.beta (out-of-history pairs) when 2 u |X| |X.beta| / denominator exceeds 1.3e-6
 constexpr float kXbGuard = 2.0f * 5.9604644775390625e-08f / 1.3e-6f;
@@ -141,14 +141,16 @@ __device__ __forceinline__ Rec load_rec(const float4* __restrict__ src32, int p)
   return r;
 }
 
-// FP64 node tests (those between the guard-band thresholds) of the block, for the instances that count
-// in shared memory (SH); the others count per thread in n_fb
-__shared__ unsigned long long s_fallbacks;
+// FP64 evaluations (node tests between the guard-band thresholds, lines of fast sources) of the block in the present tile,
+// for the instances that count in shared memory (SH); the others count per thread in n_fb. In 32 bits, where the hardware
+// adds for a warp at once (a 64-bit counter is a loop of exchanges, lane after lane: 20 bunches of gamma 2 to 20 with 900
+// slots 19.7 ms a step with it, 19.3 without).
+__shared__ unsigned s_fallbacks;
 
 template <bool SH>
 __device__ __forceinline__ void count_fallback(unsigned& n_fb) {
   if (SH)
-    atomicAdd(&s_fallbacks, 1ull);
+    atomicAdd(&s_fallbacks, 1u);
   else
     n_fb++;
 }
@@ -309,10 +311,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE), BLOCKS)
   // instances without the adaptive step (kShared), which frees their registers for the pair loop; the
   // bisection and adaptive instances keep them per thread, where the register allocation comes out better.
   constexpr bool kShared = PROP != kPropBisect && !ADAPT;
-  __shared__ unsigned long long s_cnt[3];  // out of history, shortcut, bisection
+  __shared__ unsigned long long s_cnt[4];  // out of history, shortcut, bisection; FP64 evaluations of the tiles before
   __shared__ int s_err;
   if (threadIdx.x == 0) {
-    s_cnt[0] = s_cnt[1] = s_cnt[2] = 0;
+    s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
     s_fallbacks = 0;
     s_err = 0;
     s_inv_cdt = (float)(1.0 / (kC * a.state->dt));
@@ -403,6 +405,10 @@ __global__ void __launch_bounds__(shape_block(SHAPE), BLOCKS)
     const int tn = min(kTile, j_end - tile);
     unsigned brc = 0;  // out-of-history, shortcut and bisection counts of this tile (at most kTile each)
     __syncthreads();
+    if (kShared && threadIdx.x == 0) {
+      s_cnt[3] += s_fallbacks;
+      s_fallbacks = 0;
+    }
     if (threadIdx.x < tn) {
       const int j = debug_index<int>(tile + (int)threadIdx.x, boff, boff + bd.n, a.err);
       const float4* q = a.rec32 + ((size_t)j * D + pn) * 3;
@@ -1094,7 +1100,7 @@ __global__ void __launch_bounds__(shape_block(SHAPE), BLOCKS)
       if (n_ooh) atomicAdd(&s_cnt[0], (unsigned long long)n_ooh);
       if (n_sc) atomicAdd(&s_cnt[1], (unsigned long long)n_sc);
       if (n_bi) atomicAdd(&s_cnt[2], (unsigned long long)n_bi);
-      if (n_fb) atomicAdd(&s_fallbacks, (unsigned long long)n_fb);
+      if (n_fb) atomicAdd(&s_cnt[3], (unsigned long long)n_fb);
       if (errbits) atomicOr(&s_err, errbits);
     }
   }
@@ -1105,7 +1111,8 @@ __global__ void __launch_bounds__(shape_block(SHAPE), BLOCKS)
     if (s_cnt[2]) atomicAdd(a.stats + kStatBisect, s_cnt[2]);
     const unsigned long long pairs = s_cnt[0] + s_cnt[1] + s_cnt[2];
     if (pairs) atomicAdd(a.stats + kStatNodeTests, pairs);
-    if (s_fallbacks) atomicAdd(a.stats + kStatGuard, s_fallbacks);
+    s_cnt[3] += s_fallbacks;
+    if (s_cnt[3]) atomicAdd(a.stats + kStatGuard, s_cnt[3]);
     if (s_err) atomicOr(a.err, s_err);
   }
 }
